@@ -78,22 +78,55 @@ static dim3 grid3(const Geo& g) {
 }
 static inline unsigned nb1(long long n) { return (unsigned)((n + 255) / 256); }
 
-// Grid of the per-cell kernels for cell type N (N::W consecutive x-cells per thread).
-template <class N> static dim3 grid_cells(const Geo& g) {
-  return dim3((unsigned)((g.nx + BX * N::W - 1) / (BX * N::W)), (unsigned)((g.ny + BY - 1) / BY),
-              (unsigned)((g.nz + BZ - 1) / BZ));
+// Thread-block shapes of BX * BY * BZ threads.  On a box whose rows fill whole
+// blocks each kernel takes the first shape of its list, chosen by A/B runs on
+// GB300 at 512^3: long in z for k_tau, k_edge, k_flux and the divergences, long
+// in y for the energy fluxes, k_vel, k_nu_raw and k_nu_faces.  Elsewhere a
+// fixed shape leaves lanes without a cell: 32 lanes of four cells cover 128
+// cells of a row (at nx = 160 three in eight lanes idle, k_flux 210 us against
+// 160 with 8 lanes; at 64 half of them), and blocks long in z have one thread in
+// eight at work on a plane (nz = 1).  block_for takes the first shape of the
+// list that covers the box with at most 1/16 more threads than the best one
+// (384 x 384 x 220: the 2% that 32 x 2 x 4 saves cost k_flux 5%); a row segment
+// of a block is at least 128 bytes (131 x 97 x 75 with one cell a thread: 477 us
+// a right-hand side with 8 lanes along x, 422 with 32).
+static_assert(BX * BY * BZ == 256 && BX == 32, "the shapes keep the launch bounds' thread count");
+enum BlockKind { B_LONGZ = 0, B_LONGY, B_MIXED };
+static dim3 block_for(const Geo& g, int w, BlockKind kind) {
+  static const int shapes[3][9][3] = {
+      {{32, 1, 8}, {16, 2, 8}, {8, 8, 4}, {32, 2, 4}, {8, 16, 2}, {32, 8, 1}, {16, 16, 1}, {8, 32, 1}, {256, 1, 1}},
+      {{32, 8, 1}, {16, 8, 2}, {8, 8, 4}, {32, 2, 4}, {32, 1, 8}, {16, 16, 1}, {8, 32, 1}, {16, 1, 16}, {256, 1, 1}},
+      {{32, 2, 4}, {16, 4, 4}, {8, 8, 4}, {32, 8, 1}, {32, 1, 8}, {16, 16, 1}, {8, 32, 1}, {16, 1, 16}, {256, 1, 1}}};
+  const long long lanes = (g.nx + w - 1) / w;
+  long long least = -1;
+  for (int pass = 0; pass < 2; ++pass)
+    for (const auto& sh : shapes[kind]) {
+      if (sh[0] * w < 32) continue;
+      const long long t = ((lanes + sh[0] - 1) / sh[0]) * sh[0] *
+                          (((long long)g.ny + sh[1] - 1) / sh[1]) * sh[1] *
+                          (((long long)g.nz + sh[2] - 1) / sh[2]) * sh[2];
+      if (pass == 0) least = least < 0 ? t : std::min(least, t);
+      else if (t <= least + least / 16) return dim3((unsigned)sh[0], (unsigned)sh[1], (unsigned)sh[2]);
+    }
+  return dim3(BX, BY, BZ);   // not reached: the least shape passes its own test
 }
-
-// Thread-block shapes of BX * BY * BZ threads, chosen per kernel by A/B runs
-// on GB300 at 512^3: long in z (32 x 1 x 8) for k_tau, k_edge, k_flux and the
-// divergences, long in y (32 x 8 x 1) for the energy fluxes, k_vel, k_nu_raw
-// and k_nu_faces; the default 32 x 2 x 4 for the rest.
-static_assert(BY * BZ == 8, "the per-kernel shapes keep the launch bounds' thread count");
-static const dim3 BB_Z8(BX, 1, 8);
-static const dim3 BB_Y8(BX, 8, 1);
 template <class N> static dim3 grid_for(const Geo& g, dim3 b) {
   return dim3((unsigned)((g.nx + b.x * N::W - 1) / (b.x * N::W)), (unsigned)((g.ny + b.y - 1) / b.y),
               (unsigned)((g.nz + b.z - 1) / b.z));
+}
+// Launch of the marching k_nu_maxsmooth: 128 threads, as many lanes along x as
+// the row fills, and chunks of NUZ_ZC planes, halved (to 4) while the blocks
+// leave SMs without work (64^3 has 32 blocks of 32 planes).
+static void ms_launch(const Geo& g, dim3& gd, dim3& bd) {
+  const int l4 = (g.nx + 3) / 4;
+  int w = 32;
+  for (int c : {16, 8})
+    if ((l4 + c - 1) / c * c < (l4 + w - 1) / w * w) w = c;
+  bd = dim3((unsigned)w, (unsigned)(32 * NUZ_TY / w));
+  gd = dim3((unsigned)((l4 + w - 1) / w), (unsigned)((g.ny + bd.y - 1) / bd.y), 1);
+  int zc = NUZ_ZC;
+  while (zc > 4 && (long long)gd.x * gd.y * ((g.nz + zc - 1) / zc) < 608) zc /= 2;
+  gd.z = (unsigned)((g.nz + zc - 1) / zc);
 }
 
 // Four-cell threads need 16-byte aligned arrays (the workspace always is).
@@ -442,8 +475,9 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
   const Geo& g = F.geo;
   const KPar& k = F.kp;
   float** d = F.fld;
-  const dim3 gg = grid_cells<N>(g), bb(BX, BY, BZ);
-  const dim3 gz8 = grid_for<N>(g, BB_Z8), gy8 = grid_for<N>(g, BB_Y8);
+  const dim3 bb = block_for(g, N::W, B_MIXED), bz8 = block_for(g, N::W, B_LONGZ),
+             by8 = block_for(g, N::W, B_LONGY);
+  const dim3 gg = grid_for<N>(g, bb), gz8 = grid_for<N>(g, bz8), gy8 = grid_for<N>(g, by8);
   using NB = typename N::Base;   // kernels without derivatives or lengths
   const float* ls = k.log_interp ? d[F_LR] : f[0];
   // Plane means of e - e0 (chromospheric cooling, eq. (ediffav)), before the
@@ -467,7 +501,7 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
   TIMED(K_LR, (k_lr_ed<NB><<<nb1(g.n / N::W), 256, 0, s>>>(f[0], f[4], k.log_interp ? d[F_LR] : nullptr,
                                                        d[F_ED], k.ediffav ? d[F_LER] : nullptr,
                                                        k.lnpa ? d[F_LQ] : nullptr, k, g.n, g.sz)));
-  TIMED(K_VEL, (k_vel<NB><<<gy8, BB_Y8, 0, s>>>(ls, f[1], f[2], f[3], d[F_UX], d[F_UY], d[F_UZ],
+  TIMED(K_VEL, (k_vel<NB><<<gy8, by8, 0, s>>>(ls, f[1], f[2], f[3], d[F_UX], d[F_UY], d[F_UZ],
                                         d[F_LFX], d[F_LFY], d[F_LFZ], k, g)));
   if (k.rm) {
     if (k.csmag_dl > 0.f)
@@ -477,28 +511,28 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
     // and <nu> maxima are taken here (cmax[0], cmax[2]).
     auto knu = k.csmag_dl > 0.f ? (cfl ? k_nu_raw<true, true, N> : k_nu_raw<true, false, N>)
                                 : (cfl ? k_nu_raw<false, true, N> : k_nu_raw<false, false, N>);
-    TIMED(K_NU_RAW, (knu<<<gy8, BB_Y8, 0, s>>>(d[F_UX], d[F_UY], d[F_UZ], f[0], f[4], f[5], f[6], f[7],
+    TIMED(K_NU_RAW, (knu<<<gy8, by8, 0, s>>>(d[F_UX], d[F_UY], d[F_UZ], f[0], f[4], f[5], f[6], f[7],
                                            d[F_SQXY], d[F_SQYZ], d[F_SQZX], d[F_NV],
                                            cfl ? F.cmax : nullptr, k, g)));
     if (N::W == 4) {
       // One z-marching pass for the 3x3x3 max and mean (four-cell layout).
-      const dim3 gm((unsigned)((g.nx + 127) / 128), (unsigned)((g.ny + NUZ_TY - 1) / NUZ_TY),
-                    (unsigned)((g.nz + NUZ_ZC - 1) / NUZ_ZC));
+      dim3 gm, bm;
+      ms_launch(g, gm, bm);
       auto kms = cfl ? k_nu_maxsmooth<true> : k_nu_maxsmooth<false>;
-      TIMED(K_NU_MS, (kms<<<gm, dim3(32, NUZ_TY), 0, s>>>(d[F_NV], d[F_NU], d[F_LNU], F.cmax + 2, g)));
+      TIMED(K_NU_MS, (kms<<<gm, bm, 0, s>>>(d[F_NV], d[F_NU], d[F_LNU], F.cmax + 2, g)));
     } else {
       TIMED(K_NU_MAX, (k_nu_max<NB><<<gg, bb, 0, s>>>(d[F_NV], d[F_NM], g)));
       auto ksm = cfl ? k_nu_smooth<NB, true> : k_nu_smooth<NB, false>;
       TIMED(K_NU_SMOOTH, (ksm<<<gg, bb, 0, s>>>(d[F_NM], d[F_NU], d[F_LNU], F.cmax + 2, g)));
     }
-    TIMED(K_NU_FACES, (k_nu_faces<NB><<<gy8, BB_Y8, 0, s>>>(d[F_LNU], d[F_LNX], d[F_LNY], d[F_LNZ], g)));
+    TIMED(K_NU_FACES, (k_nu_faces<NB><<<gy8, by8, 0, s>>>(d[F_LNU], d[F_LNX], d[F_LNY], d[F_LNZ], g)));
   }
   if (k.d2div)
     TIMED(K_D2FLAG, (k_d2flag<NB><<<gg, bb, 0, s>>>(f[0], f[4], F.d2flag, k, g)));
   // The fused flux-divergence kernel forms J itself: k_tau only for viscous runs.
   auto ktau = k.d2div ? k_tau<N, true> : k_tau<N, false>;
   if (!F.fdiv || k.visc)
-  TIMED(K_TAU, (ktau<<<gz8, BB_Z8, 0, s>>>(d[F_UX], d[F_UY], d[F_UZ], f[0], d[F_LFX], d[F_LFY],
+  TIMED(K_TAU, (ktau<<<gz8, bz8, 0, s>>>(d[F_UX], d[F_UY], d[F_UZ], f[0], d[F_LFX], d[F_LFY],
                                        d[F_LFZ], d[F_NU], d[F_LNX], d[F_LNY], d[F_LNZ], f[5],
                                        f[6], f[7], d[F_TXX], d[F_TYY], d[F_TZZ], d[F_TXY],
                                        d[F_TYZ], d[F_TZX], d[F_RX], d[F_RY], d[F_RZ], d[F_JX],
@@ -506,7 +540,7 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
   auto kedge = k.qmax3 ? (k.d2div ? k_edge<N, true, true> : k_edge<N, false, true>)
                        : (k.d2div ? k_edge<N, true, false> : k_edge<N, false, false>);
   if (k.visc)
-    TIMED(K_EDGE, (kedge<<<gz8, BB_Z8, 0, s>>>(d[F_TXX], d[F_TYY], d[F_TZZ], d[F_TXY], d[F_TYZ],
+    TIMED(K_EDGE, (kedge<<<gz8, bz8, 0, s>>>(d[F_TXX], d[F_TYY], d[F_TZZ], d[F_TXY], d[F_TYZ],
                                            d[F_TZX], d[F_RX], d[F_RY], d[F_RZ], d[F_JX],
                                            d[F_JY], d[F_JZ], d[F_UX], d[F_UY], d[F_UZ],
                                            d[F_QXX], d[F_QYY], d[F_QZZ], d[F_QXY], d[F_QYZ],
@@ -525,8 +559,8 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
   FluxOut fo = {d[F_MXX], d[F_MYY], d[F_MZZ], d[F_MXY], d[F_MYX], d[F_MXZ], d[F_MZX],
                 d[F_MYZ], d[F_MZY], d[F_LX1], d[F_LX2], d[F_LY1], d[F_LY2], d[F_LZ1],
                 d[F_LZ2], d[F_GX], d[F_GY], d[F_GZ], d[F_QT], d[F_EX], d[F_EY], d[F_EZ]};
-  TIMED(K_FLUX, (k_flux<N><<<gz8, BB_Z8, 0, s>>>(fi, fo, k, g)));
-  TIMED(K_FLUX_E, (k_flux_e<N><<<gy8, BB_Y8, 0, s>>>(fi, fo, k, g)));
+  TIMED(K_FLUX, (k_flux<N><<<gz8, bz8, 0, s>>>(fi, fo, k, g)));
+  TIMED(K_FLUX_E, (k_flux_e<N><<<gy8, by8, 0, s>>>(fi, fo, k, g)));
   if (k.inv_tchromo > 0.f || k.corL0 > 0.f)
     TIMED(K_COOL2, (k_cool2<NB><<<gg, bb, 0, s>>>(f[0], f[4], d[F_QT], k, g)));
   STG_CUDA_OK(cudaGetLastError());
@@ -710,7 +744,8 @@ static int launch_div(Fused& F, float* const f[8], float* q[8], float* o[8], flo
   float* oo[8];
   for (int c = 0; c < 8; ++c) oo[c] = o ? o[c] : q[c];
   const bool v4 = F.cells4 && aligned16(f, 8) && aligned16(q, 8) && aligned16(oo, 8);
-  const dim3 bb = BB_Z8, gg = v4 ? grid_for<Nb4>(F.geo, bb) : grid_for<Nb>(F.geo, bb);
+  const dim3 bb = block_for(F.geo, v4 ? 4 : 1, B_LONGZ),
+             gg = v4 ? grid_for<Nb4>(F.geo, bb) : grid_for<Nb>(F.geo, bb);
   // Momentum; mass and energy; induction (disjoint inputs, one kernel each).
   const int nk = 3;
   typedef void (*DivK)(DivIn, float*, float*, float*, float*, float*, float*, float*, float*,
@@ -757,7 +792,8 @@ int fused_rhs(Fused& F, float* const f[8], float* out[8], cudaStream_t s) {
 
 template <class N>
 static void courant_part(Fused& F, float* const f[8], cudaStream_t s) {
-  TIMED(K_COURANT, (k_courant_part<N><<<grid_cells<N>(F.geo), dim3(BX, BY, BZ), 0, s>>>(
+  const dim3 bb = block_for(F.geo, N::W, B_MIXED);
+  TIMED(K_COURANT, (k_courant_part<N><<<grid_for<N>(F.geo, bb), bb, 0, s>>>(
                        F.fld[F_UX], F.fld[F_UY], F.fld[F_UZ], f[0], f[4], f[5], f[6], f[7],
                        F.q[0], F.q[4], F.fld[F_NU], F.cmax, F.kp, F.geo)));
 }
