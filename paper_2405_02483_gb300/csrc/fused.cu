@@ -381,9 +381,10 @@ int fused_init(Fused& F, const stagger_grid& gr, const stagger_params& p) {
   }
   // Which intermediate fields this parameter set needs.
   std::vector<int> need = {F_UX, F_UY, F_UZ};
-  // The fused flux-divergence kernel keeps every flux on chip and forms J
-  // itself; k_tau still writes J and eta J for k_edge in viscous runs.
-  if (!F.fdiv || k.visc) for (int f : {F_JX, F_JY, F_JZ, F_EX, F_EY, F_EZ}) need.push_back(f);
+  // k_flux and k_fdiv form J themselves; k_tau writes J and eta J for k_edge in
+  // viscous runs.
+  if (k.visc) for (int f : {F_JX, F_JY, F_JZ}) need.push_back(f);
+  if (!F.fdiv || k.visc) for (int f : {F_EX, F_EY, F_EZ}) need.push_back(f);
   if (!F.fdiv)
     for (int f : {F_MXX, F_MYY, F_MZZ, F_MXY, F_MYX, F_MXZ, F_MZX, F_MYZ, F_MZY, F_LX1, F_LX2,
                   F_LY1, F_LY2, F_LZ1, F_LZ2, F_GX, F_GY, F_GZ, F_QT})
@@ -529,9 +530,9 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
   }
   if (k.d2div)
     TIMED(K_D2FLAG, (k_d2flag<NB><<<gg, bb, 0, s>>>(f[0], f[4], F.d2flag, k, g)));
-  // The fused flux-divergence kernel forms J itself: k_tau only for viscous runs.
+  // J for the Joule heating of k_edge; k_flux and k_fdiv form it themselves.
   auto ktau = k.d2div ? k_tau<N, true> : k_tau<N, false>;
-  if (!F.fdiv || k.visc)
+  if (k.visc)
   TIMED(K_TAU, (ktau<<<gz8, bz8, 0, s>>>(d[F_UX], d[F_UY], d[F_UZ], f[0], d[F_LFX], d[F_LFY],
                                        d[F_LFZ], d[F_NU], d[F_LNX], d[F_LNY], d[F_LNZ], f[5],
                                        f[6], f[7], d[F_TXX], d[F_TYY], d[F_TZZ], d[F_TXY],
@@ -732,13 +733,14 @@ static int launch_fdiv(Fused& F, float* const f[8], float* q[8], float* const* o
 }
 
 // Stage stg's right-hand side into q (mode 0), or with the update by its
-// beta dt (mode 1: F.bdt_dev[stg]).
+// beta dt (mode 1, or 2 in the last stage: F.bdt_dev[stg]).  parts: which of the
+// three launches (bit 0 momentum, 1 mass and energy, 2 induction).
 static int launch_div(Fused& F, float* const f[8], float* q[8], float* o[8], float alpha,
-                      int stg, int mode, cudaStream_t s, bool cfl = false) {
+                      int stg, int mode, cudaStream_t s, bool cfl = false, int parts = 7) {
   if (F.fdiv) {
     float* oo[8];
     for (int c = 0; c < 8; ++c) oo[c] = o ? o[c] : q[c];
-    return launch_fdiv(F, f, q, oo, alpha, stg, mode, s, cfl);
+    return launch_fdiv(F, f, q, oo, alpha, stg, mode ? 1 : 0, s, cfl);
   }
   DivIn di = div_in(F, f);
   float* oo[8];
@@ -747,7 +749,6 @@ static int launch_div(Fused& F, float* const f[8], float* q[8], float* o[8], flo
   const dim3 bb = block_for(F.geo, v4 ? 4 : 1, B_LONGZ),
              gg = v4 ? grid_for<Nb4>(F.geo, bb) : grid_for<Nb>(F.geo, bb);
   // Momentum; mass and energy; induction (disjoint inputs, one kernel each).
-  const int nk = 3;
   typedef void (*DivK)(DivIn, float*, float*, float*, float*, float*, float*, float*, float*,
                        float*, float*, float*, float*, float*, float*, float*, float*, float,
                        const float*, int, unsigned*, KPar, Geo);
@@ -770,7 +771,8 @@ static int launch_div(Fused& F, float* const f[8], float* q[8], float* o[8], flo
       kern[2] = v4 ? k_div<Nb4, 0xE0, false> : k_div<Nb, 0xE0, false>;
     }
   }
-  for (int i = 0; i < nk; ++i)
+  for (int i = 0; i < 3; ++i)
+    if ((parts >> i) & 1)
     TIMED(K_DIV, (kern[i]<<<gg, bb, 0, s>>>(di, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7],
                                             oo[0], oo[1], oo[2], oo[3], oo[4], oo[5], oo[6],
                                             oo[7], alpha, F.bdt_dev + stg, mode, F.cmax + 1,
@@ -832,22 +834,32 @@ int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s) {
     if (rc) return rc;
     const float alpha = (float)RK_ALPHA[stg];
     if (stg == 0 && dt <= 0) {
-      // Courant step from the state and its stage-1 derivative, then update.
-      rc = launch_div(F, st_in[0], F.q, nullptr, 0.f, 0, 0, s, cfl);
+      // The Courant step needs the state, <nu> and the mass and energy
+      // derivatives: they come first, the other six fields then take their
+      // update with their divergence, and only rho and E need one of their own
+      // (6 arrays in place of 24).  k_fdiv forms all eight at once.
+      const int first = F.fdiv ? 7 : 2;
+      rc = launch_div(F, st_in[0], F.q, nullptr, 0.f, 0, 0, s, cfl, first);
       if (rc) return rc;
       courant_to_dev(F, st_in[0], s, cfl);
+      if (!F.fdiv) {
+        rc = launch_div(F, st_in[0], F.q, const_cast<float**>(st_out[0]), 0.f, 0, 1, s, false, 5);
+        if (rc) return rc;
+      }
       Upd8 u;
-      int vec = (F.geo.n % 4) == 0;
+      int vec = (F.geo.n % 4) == 0, nu = 0;
       for (int c = 0; c < 8; ++c) {
-        u.f[c] = st_in[0][c];
-        u.q[c] = F.q[c];
-        u.o[c] = st_out[0][c];
-        vec &= (((uintptr_t)u.f[c] | (uintptr_t)u.q[c] | (uintptr_t)u.o[c]) & 15) == 0;
+        if (!F.fdiv && c != 0 && c != 4) continue;
+        u.f[nu] = st_in[0][c];
+        u.q[nu] = F.q[c];
+        u.o[nu] = st_out[0][c];
+        vec &= (((uintptr_t)u.f[nu] | (uintptr_t)u.q[nu] | (uintptr_t)u.o[nu]) & 15) == 0;
+        ++nu;
       }
       const long long work = vec ? F.geo.n / 4 : F.geo.n;
       unsigned bx = (unsigned)((work + 255) / 256);
       if (bx > 2048) bx = 2048;
-      TIMED(K_UPDATE, (k_update8<<<dim3(bx, 8), 256, 0, s>>>(u, F.bdt_dev, F.geo.n, vec)));
+      TIMED(K_UPDATE, (k_update8<<<dim3(bx, (unsigned)nu), 256, 0, s>>>(u, F.bdt_dev, F.geo.n, vec)));
       STG_CUDA_OK(cudaGetLastError());
       continue;
     }
@@ -855,7 +867,7 @@ int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s) {
       TIMED(K_MISC, (k_set_dt<<<1, 1, 0, s>>>(F.dt_dev, F.bdt_dev, dt, (float)RK_BETA[0],
                                               (float)RK_BETA[1], (float)RK_BETA[2])));
     }
-    rc = launch_div(F, st_in[stg], F.q, const_cast<float**>(st_out[stg]), alpha, stg, 1, s);
+    rc = launch_div(F, st_in[stg], F.q, const_cast<float**>(st_out[stg]), alpha, stg, stg == 2 ? 2 : 1, s);
     if (rc) return rc;
   }
   if (F.wall) wall_launch(F, f, false, s, false);

@@ -330,6 +330,24 @@ template <class V> __device__ __forceinline__ auto s_dd(V v, float ih) -> declty
   return (DA_ * (v(0) - v(-1)) + DB_ * (v(1) - v(-2)) + DC_ * (v(2) - v(-3))) * ih;
 }
 
+// s_dn and s_dd of the same taps (dn returned, the derivative in d).
+template <class V>
+__device__ __forceinline__ auto s_dn_dd(V v, float ih, decltype(v(0))& d) -> decltype(v(0)) {
+  const auto a = v(-3), b = v(-2), c = v(-1), e = v(0), f = v(1), g = v(2);
+  d = (DA_ * (e - c) + DB_ * (f - b) + DC_ * (g - a)) * ih;
+  return IA_ * (c + e) + IB_ * (b + f) + IC_ * (a + g);
+}
+
+// Ask for the cell's line of an array the kernel reads later, without a
+// register to receive it: the DRAM read of the first arrays' taps then runs
+// beside those of the later ones (512^3: k_tau 3.71 -> 3.54 ms, the three k_div
+// 5.27 -> 4.82 ms; no gain in k_flux, k_flux_e and k_edge).
+template <class N> __device__ __forceinline__ void pf(const N& n, const float* p) {
+#ifdef __CUDA_ARCH__
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p + n.c));
+#endif
+}
+
 #define LDG(p, i) __ldg((p) + (i))
 // Operand functors along one axis of a field at the thread's cell(s).
 #define AX(fp, axis) [&](int o) { return n.lda(fp, axis, o); }
@@ -780,13 +798,16 @@ __global__ void STG_LB_HI(N, STG_MINB) k_tau(
   N n;
   if (!n.init(g, k)) return;
   using T = typename N::T;
+  pf(n, ux); pf(n, uy); pf(n, uz); pf(n, lfx); pf(n, lfy); pf(n, lfz); pf(n, rd);
+  if (k.rm) {
+    pf(n, lnx); pf(n, lny); pf(n, lnz); pf(n, nu);
+  }
   T jx = s_dd(AX(bz, 1), n.jd(1, k)) - s_dd(AX(by, 2), n.jd(2, k));
   T jy = s_dd(AX(bx, 2), n.jd(2, k)) - s_dd(AX(bz, 0), n.jd(0, k));
   T jz = s_dd(AX(by, 0), n.jd(0, k)) - s_dd(AX(bx, 1), n.jd(1, k));
   n.st(Jx, jx);
   n.st(Jy, jy);
   n.st(Jz, jz);
-  if (!k.visc) return;
   const unsigned fl = D2 ? n.ldflag(flag) : 0u;
   const Strain3<T> Sd = strain_diag<D2>(n, ux, uy, uz, fl, k);
   const T sxx = Sd.a, syy = Sd.b, szz = Sd.c;
@@ -953,38 +974,45 @@ __device__ __forceinline__ void flux_mom_cell(const N& n, const FluxIn& in, cons
     if (k.visc) v -= n.ld(tau);
     return v;
   };
+  // J = curl B at the edge comes from the taps of its two B interpolations.
   {  // Ex edge (i, j-1/2, k-1/2)
-    const T uy_z = s_dn(AX(in.uy, 2)), uz_y = s_dn(AX(in.uz, 1));
-    const T bz_y = s_dn(AX(in.bz, 1)) + B0[2], by_z = s_dn(AX(in.by, 2)) + B0[1];
-    n.st(out.myz, off(1, 2, uz_y, in.qyz));
-    n.st(out.mzy, off(2, 1, uy_z, in.qyz));
-    const T jx = n.ld(in.Jx);
+    T dz, dy;
+    const T bz_y = s_dn_dd(AX(in.bz, 1), n.jd(1, k), dz) + B0[2];
+    const T by_z = s_dn_dd(AX(in.by, 2), n.jd(2, k), dy) + B0[1];
+    const T jx = dz - dy;
     n.st(out.ly2, jx * bz_y);
     n.st(out.lz1, jx * by_z);
+    const T uy_z = s_dn(AX(in.uy, 2)), uz_y = s_dn(AX(in.uz, 1));
     const T ex = -((uy_z * bz_y) - (uz_y * by_z));
     n.st(out.ex, k.visc ? ex + n.ldw(out.ex) : ex);
+    n.st(out.myz, off(1, 2, uz_y, in.qyz));
+    n.st(out.mzy, off(2, 1, uy_z, in.qyz));
   }
   {  // Ey edge (i-1/2, j, k-1/2)
-    const T uz_x = s_dn(AX(in.uz, 0)), ux_z = s_dn(AX(in.ux, 2));
-    const T bx_z = s_dn(AX(in.bx, 2)) + B0[0], bz_x = s_dn(AX(in.bz, 0)) + B0[2];
-    n.st(out.mxz, off(0, 2, uz_x, in.qzx));
-    n.st(out.mzx, off(2, 0, ux_z, in.qzx));
-    const T jy = n.ld(in.Jy);
+    T dx, dz;
+    const T bx_z = s_dn_dd(AX(in.bx, 2), n.jd(2, k), dx) + B0[0];
+    const T bz_x = s_dn_dd(AX(in.bz, 0), n.jd(0, k), dz) + B0[2];
+    const T jy = dx - dz;
     n.st(out.lx1, jy * bz_x);
     n.st(out.lz2, jy * bx_z);
+    const T uz_x = s_dn(AX(in.uz, 0)), ux_z = s_dn(AX(in.ux, 2));
     const T ey = -((uz_x * bx_z) - (ux_z * bz_x));
     n.st(out.ey, k.visc ? ey + n.ldw(out.ey) : ey);
+    n.st(out.mxz, off(0, 2, uz_x, in.qzx));
+    n.st(out.mzx, off(2, 0, ux_z, in.qzx));
   }
   {  // Ez edge (i-1/2, j-1/2, k)
-    const T ux_y = s_dn(AX(in.ux, 1)), uy_x = s_dn(AX(in.uy, 0));
-    const T by_x = s_dn(AX(in.by, 0)) + B0[1], bx_y = s_dn(AX(in.bx, 1)) + B0[0];
-    n.st(out.mxy, off(0, 1, uy_x, in.qxy));
-    n.st(out.myx, off(1, 0, ux_y, in.qxy));
-    const T jz = n.ld(in.Jz);
+    T dy, dx;
+    const T by_x = s_dn_dd(AX(in.by, 0), n.jd(0, k), dy) + B0[1];
+    const T bx_y = s_dn_dd(AX(in.bx, 1), n.jd(1, k), dx) + B0[0];
+    const T jz = dy - dx;
     n.st(out.lx2, jz * by_x);
     n.st(out.ly1, jz * bx_y);
+    const T ux_y = s_dn(AX(in.ux, 1)), uy_x = s_dn(AX(in.uy, 0));
     const T ez = -((ux_y * by_x) - (uy_x * bx_y));
     n.st(out.ez, k.visc ? ez + n.ldw(out.ez) : ez);
+    n.st(out.mxy, off(0, 1, uy_x, in.qxy));
+    n.st(out.myx, off(1, 0, ux_y, in.qxy));
   }
 }
 
@@ -1044,8 +1072,13 @@ __device__ __forceinline__ void flux_energy_cell(const N& n, const FluxIn& in,
 
 // Two launches with disjoint outputs; they share only the momenta, the
 // velocities and E as inputs, and each keeps its live values in registers.
+// Both wait on their loads (37 and 17 arrays).  k_flux holds more taps in flight
+// with 128 registers and two blocks an SM than with 80 and three (512^3: 4.13
+// against 4.98 ms, J formed from the B taps included, which saves reading its
+// three arrays); k_flux_e, whose taps are mostly one array's 6 x 6 squares, is
+// faster with three blocks (3.27 against 3.63 ms).
 template <class N>
-__global__ void STG_LB_HI(N, STG_MINB) k_flux(FluxIn in, FluxOut out, KPar k, Geo g) {
+__global__ void STG_LB(N, STG_MINB) k_flux(FluxIn in, FluxOut out, KPar k, Geo g) {
   N n;
   if (!n.init(g, k)) return;
   flux_mom_cell(n, in, out, k);
@@ -1111,7 +1144,8 @@ __device__ __forceinline__ typename N::T lnp_grad(const N& n, const float* lq, c
 
 // F(f) and the RK update: q <- alpha q + F, f_out <- f + beta dt q, for the
 // fields in the bit mask M (bit c: field c), each stored as soon as it is
-// formed.  mode 0: write F to q only; 1: also update with beta dt = *bdtp.
+// formed.  mode 0: write F to q only; 1: also update with beta dt = *bdtp; 2:
+// update without storing q (the last stage, whose q nothing reads).
 // Launched as three kernels (momentum; mass and energy; induction), whose
 // inputs are disjoint, at 4 blocks per SM: fewer live registers per launch.
 // With CR (mass and energy, the stage whose derivative sets the Courant step)
@@ -1133,7 +1167,7 @@ __device__ __forceinline__ unsigned div_cell(const N& n, const DivIn& in, float*
     if (CR && c == 0) F0 = F;
     if (CR && c == 4) F4 = F;
     const T qq = alpha != 0.f ? alpha * n.ldw(qs[c]) + F : F;
-    n.st(qs[c], qq);
+    if (mode != 2) n.st(qs[c], qq);
     if (mode) n.st(os[c], n.ld(in.f[c]) + bdt * qq);
   };
   // Stellar-atmosphere boundaries (R26): the inflow weight f of the bottom
@@ -1235,6 +1269,22 @@ __global__ void STG_LB_4(N, STG_MINB) k_div(DivIn in, float* q0, float* q1, floa
   const bool inside = n.init(g, k);
   float* qs[8] = {q0, q1, q2, q3, q4, q5, q6, q7};
   float* os[8] = {o0, o1, o2, o3, o4, o5, o6, o7};
+  if (inside) {
+    if (M & 14)
+      for (const float* p : {in.mxx, in.mxy, in.mxz, in.lx1, in.lx2, in.myx, in.myy, in.myz,
+                             in.ly1, in.ly2, in.mzx, in.mzy, in.mzz, in.lz1, in.lz2})
+        pf(n, p);
+    if (M & 17)
+      for (const float* p : {in.px, in.py, in.pz, in.gx, in.gy, in.gz, in.qt}) pf(n, p);
+    if (M & 0xE0)
+      for (const float* p : {in.Ex, in.Ey, in.Ez}) pf(n, p);
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if ((M >> c) & 1) {
+        if (mode) pf(n, in.f[c]);
+        if (alpha != 0.f) pf(n, qs[c]);
+      }
+  }
   if constexpr (!CR) {
     if (inside) div_cell<N, M, false, WB>(n, in, qs, os, alpha, bdtp, mode, k);
   } else {
