@@ -1,6 +1,5 @@
-// Op-graph executor (see graph.cuh): one launch of a primitive's forward or
-// transpose kernel (graph_kernels.cuh) per node, on one stream or as a DAG
-// over several.
+// Op-graph executor (see graph.cuh): the sweeps as batches of independent
+// nodes, one launch per dependency level (kernels in graph_kernels.cuh).
 #include <math.h>
 
 #include <stdint.h>
@@ -10,6 +9,140 @@
 #include "graph_kernels.cuh"
 
 namespace stg {
+
+// ---------------------------------------------------------------------------
+// Schedule.  A sweep is a sequence of batches of at most cap nodes that do not
+// depend on one another, each the next ready nodes in the graph's order.
+// Reverse: the cotangent of a node is the sum of what its consumers pass to it;
+// a node whose only term is the consumer's cotangent itself shares that array.
+// A cotangent's array is free again after the last batch that reads it.
+// ---------------------------------------------------------------------------
+static bool special_op(int op) { return op == G_QUENCH || op == G_PMEAN; }
+
+// Whether the term (consumer nd, role) passes nd's cotangent on unchanged.
+static bool identity_term(const GNode& nd, int role) {
+  if (role == R_COPY) return true;
+  if (nd.ep) return false;
+  if (role == R_C) return nd.pop != 2;
+  if (nd.pop == 3) return false;
+  return nd.op == G_ADD || (nd.op == G_SUB && role == R_A);
+}
+
+static void plan_sweeps(const GraphDef& G, int cap, LevelPlan& P) {
+  const int nn = (int)G.nodes.size();
+  P = LevelPlan();
+  P.flev.assign(nn, 0);   // 0: an input, or not scheduled yet
+  for (int left = nn, lo = 0; lo < nn; ++P.nflev) {
+    const int now = P.nflev + 1;
+    int took = 0;
+    for (int i = lo; i < nn && took < cap; ++i) {
+      const GNode& nd = G.nodes[i];
+      bool ready = nd.op != G_INPUT && !P.flev[i];
+      for (int o : {nd.a, nd.b, nd.c})
+        if (o >= 0 && G.nodes[o].op != G_INPUT && (!P.flev[o] || P.flev[o] == now)) ready = false;
+      if (ready) {
+        P.flev[i] = now;
+        ++took;
+      }
+    }
+    while (lo < nn && (G.nodes[lo].op == G_INPUT || P.flev[lo])) ++lo;
+    if (!took && --left < 0) break;   // (every pass takes a node: operands come first)
+  }
+  // Nodes a gradient is worth forming for: those an input reaches.
+  std::vector<char> useful(nn, 0);
+  for (int i = 0; i < nn; ++i) {
+    const GNode& nd = G.nodes[i];
+    useful[i] = nd.op == G_INPUT;
+    if (has_transpose(nd.op))
+      for (int o : {nd.a, nd.b, nd.c})
+        if (o >= 0 && useful[o]) useful[i] = 1;
+  }
+  P.terms.assign(nn, {});
+  P.rlev.assign(nn, -1);
+  P.alias.assign(nn, P.OWN);
+  P.gslot.assign(nn, -1);
+  std::vector<int> seeds(nn, 0);
+  for (int k = 0; k < 8; ++k)
+    if (useful[G.out[k]]) {
+      // (the seed of output k as a term with consumer -1 - k)
+      P.terms[G.out[k]].push_back({-1 - k, R_COPY});
+      ++seeds[G.out[k]];
+    }
+  for (int i = nn - 1; i >= 0; --i) {
+    const GNode& nd = G.nodes[i];
+    if (P.terms[i].empty() || !has_transpose(nd.op)) continue;
+    if (special_op(nd.op)) {   // its own array holds the operand's contribution
+      if (useful[nd.a]) P.terms[nd.a].push_back({i, R_COPY});
+      continue;
+    }
+    if (nd.a >= 0 && useful[nd.a]) P.terms[nd.a].push_back({i, R_A});
+    if (nd.b >= 0 && useful[nd.b]) P.terms[nd.b].push_back({i, R_B});
+    if (nd.c >= 0 && useful[nd.c]) P.terms[nd.c].push_back({i, R_C});
+  }
+  for (int i = nn - 1; i >= 0; --i) {
+    const GNode& nd = G.nodes[i];
+    if (P.terms[i].size() != 1 || nd.op == G_INPUT || special_op(nd.op)) continue;
+    const auto& t = P.terms[i][0];
+    if (t.consumer < 0 || identity_term(G.nodes[t.consumer], t.role))
+      P.alias[i] = t.consumer >= 0 && P.alias[t.consumer] != P.OWN ? P.alias[t.consumer] : t.consumer;
+  }
+  // A node with no array of its own is ready with the one it shares (a
+  // special's after its own passes, which end its batch).
+  for (int hi = nn - 1; hi >= 0;) {
+    const int now = P.nrlev;
+    int took = 0;
+    for (int i = hi; i >= 0; --i) {
+      if (P.rlev[i] >= 0 || P.terms[i].empty()) continue;
+      if (P.alias[i] != P.OWN) {
+        if (P.alias[i] < 0) P.rlev[i] = 0;
+        else if (P.rlev[P.alias[i]] >= 0) P.rlev[i] = P.rlev[P.alias[i]];
+        continue;
+      }
+      if (took == cap) continue;
+      bool ready = true;
+      for (const auto& t : P.terms[i])
+        if (t.consumer >= 0) {
+          const int r = P.alias[t.consumer] == P.OWN ? t.consumer : P.alias[t.consumer];
+          if (r >= 0 && (P.rlev[r] < 0 || P.rlev[r] == now)) ready = false;
+        }
+      if (ready) {
+        P.rlev[i] = now;
+        ++took;
+      }
+    }
+    while (hi >= 0 && (P.terms[hi].empty() || P.rlev[hi] >= 0)) --hi;
+    if (!took) break;   // (every pass takes a node: consumers come last)
+    ++P.nrlev;
+  }
+  // Arrays by liveness: root r's is read up to level last[r].
+  auto root = [&](int i) { return P.alias[i] == P.OWN ? i : P.alias[i]; };
+  std::vector<int> last(nn, -1);
+  for (int i = 0; i < nn; ++i) {
+    if (P.rlev[i] < 0 || P.alias[i] != P.OWN) continue;
+    for (const auto& t : P.terms[i])
+      if (t.consumer >= 0 && root(t.consumer) >= 0)
+        last[root(t.consumer)] = std::max(last[root(t.consumer)], P.rlev[i]);
+  }
+  std::vector<int> freel;
+  std::vector<std::pair<int, int>> live;   // (last level, slot)
+  for (int L = 0; L < P.nrlev; ++L) {
+    for (size_t q = 0; q < live.size();)
+      if (live[q].first < L) {
+        freel.push_back(live[q].second);
+        live[q] = live.back();
+        live.pop_back();
+      } else {
+        ++q;
+      }
+    for (int i = 0; i < nn; ++i) {
+      if (P.rlev[i] != L || P.alias[i] != P.OWN || G.nodes[i].op == G_INPUT) continue;
+      if (freel.empty()) freel.push_back(P.nslots++);
+      P.gslot[i] = freel.back();
+      freel.pop_back();
+      live.push_back({std::max(last[i], L), P.gslot[i]});
+    }
+  }
+}
 
 // ---------------------------------------------------------------------------
 // Executor
@@ -24,16 +157,21 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads) {
   for (auto& nd : def.nodes)
     if (nd.op != G_INPUT) ++nval;
   if (cudaMalloc(&vals, sizeof(T) * nval * g.n) != cudaSuccess) { vals = nullptr; return STAGGER_EOOM; }
-  bool has_pmean = false, has_quench = false;
+  bool has_pmean = false;
+  int nquench = 0;
+  near = true;
   for (auto& nd : def.nodes) {
     has_pmean |= nd.op == G_PMEAN;
-    has_quench |= nd.op == G_QUENCH;
+    nquench += nd.op == G_QUENCH;
+    if ((nd.op == G_SHIFT || nd.op == G_NB3) && nd.sk != 1 && nd.sk != -1) near = false;
   }
-  if (has_quench && with_grads &&
-      cudaMalloc(&qscr, sizeof(T) * 15 * (size_t)g.n) != cudaSuccess) {
-    qscr = nullptr;
-    release();
-    return STAGGER_EOOM;
+  if (nquench && with_grads) {
+    nscr = std::min(nquench, (int)QuenchBatch<T>::MAX);
+    if (cudaMalloc(&qscr, sizeof(T) * 15 * nscr * (size_t)g.n) != cudaSuccess) {
+      qscr = nullptr;
+      release();
+      return STAGGER_EOOM;
+    }
   }
   if (has_pmean && cudaMalloc(&psum, sizeof(T) * g.nz) != cudaSuccess) {
     psum = nullptr;
@@ -52,10 +190,9 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads) {
       return STAGGER_ECUDA;
     }
   }
-  // Reverse-sweep bookkeeping: gradient flags and the reused gradient arrays.
-  plan_reverse(def, rp);
+  plan_sweeps(def, FwdBatch<T>::MAX, lp);
   if (with_grads) {
-    if (cudaMalloc(&grads, sizeof(T) * (size_t)rp.nslots * g.n) != cudaSuccess) {
+    if (cudaMalloc(&grads, sizeof(T) * (size_t)std::max(1, lp.nslots) * g.n) != cudaSuccess) {
       grads = nullptr;
       release();
       return STAGGER_EOOM;
@@ -69,34 +206,7 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads) {
 }
 
 template <typename T>
-int GraphExec<T>::enable_concurrency() {
-  if (nconc) return STAGGER_OK;
-  for (int k = 0; k < GRAPH_NSTREAMS; ++k)
-    if (cudaStreamCreateWithFlags(&aux[k], cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&evjoin[k], cudaEventDisableTiming) != cudaSuccess)
-      return STAGGER_ECUDA;
-  if (cudaEventCreateWithFlags(&evfork, cudaEventDisableTiming) != cudaSuccess) return STAGGER_ECUDA;
-  evn.assign(def.nodes.size(), nullptr);
-  for (auto& e : evn)
-    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return STAGGER_ECUDA;
-  nconc = GRAPH_NSTREAMS;
-  return STAGGER_OK;
-}
-
-template <typename T>
 void GraphExec<T>::release() {
-  for (auto e : evn)
-    if (e) cudaEventDestroy(e);
-  evn.clear();
-  for (int k = 0; k < GRAPH_NSTREAMS; ++k) {
-    if (aux[k]) cudaStreamDestroy(aux[k]);
-    if (evjoin[k]) cudaEventDestroy(evjoin[k]);
-    aux[k] = nullptr;
-    evjoin[k] = nullptr;
-  }
-  if (evfork) cudaEventDestroy(evfork);
-  evfork = nullptr;
-  nconc = 0;
   if (vals) cudaFree(vals);
   if (grads) cudaFree(grads);
   if (mesh) cudaFree(mesh);
@@ -106,217 +216,188 @@ void GraphExec<T>::release() {
   ptr.clear();
 }
 
-// z extent of the launch: GBZ * GZU cells per block along z (GZU per thread).
-static inline dim3 ggrid(const Geo& g) {
-  return dim3((unsigned)((g.nx + GBX - 1) / GBX), (unsigned)((g.ny + GBY - 1) / GBY),
-              (unsigned)((g.nz + GBZ * GZU - 1) / (GBZ * GZU)));
-}
-
-// The forward and transpose kernel of each op (the op a template constant):
-// the stencil-like ops on the 3-D launch grid, the pointwise ops as flat
-// kernels (pointwise_op).
-template <typename T>
-using FwdK = void (*)(GNode, const T*, const T*, const T*, T*, const T*, Geo);
-template <typename T>
-using BwdK = void (*)(GNode, const T*, const T*, const T*, const T*, T*, T*, T*, int, int, int,
-                      Geo);
-template <typename T>
-using FwdPwK = void (*)(GNode, const T*, const T*, const T*, T*, long long, int);
-template <typename T>
-using BwdPwK = void (*)(GNode, const T*, const T*, const T*, const T*, T*, T*, T*, int, int, int,
-                        long long, int);
-
-template <typename T>
-static FwdK<T> fwd_kernel(int op) {
-  switch (op) {
-    case G_STENCIL: return g_forward<T, G_STENCIL>;
-    case G_SHIFT: return g_forward<T, G_SHIFT>;
-    case G_STBIN: return g_forward<T, G_STBIN>;
-    case G_STMUL: return g_forward<T, G_STMUL>;
-    case G_ST2: return g_forward<T, G_ST2>;
-    case G_STEXP: return g_forward<T, G_STEXP>;
-    case G_NB3: return g_forward<T, G_NB3>;
-    default: return g_forward<T, G_ZFIELD>;
-  }
-}
-
-template <typename T>
-static BwdK<T> bwd_kernel(int op) {
-  switch (op) {
-    case G_STENCIL: return g_backward<T, G_STENCIL>;
-    case G_STBIN: return g_backward<T, G_STBIN>;
-    case G_STMUL: return g_backward<T, G_STMUL>;
-    case G_ST2: return g_backward<T, G_ST2>;
-    case G_STEXP: return g_backward<T, G_STEXP>;
-    case G_NB3: return g_backward<T, G_NB3>;
-    default: return g_backward<T, G_SHIFT>;
-  }
-}
-
-template <typename T>
-static FwdK<T> fwd_kernel4(int op) {
-  switch (op) {
-    case G_STENCIL: return g_forward4<T, G_STENCIL>;
-    case G_SHIFT: return g_forward4<T, G_SHIFT>;
-    case G_STBIN: return g_forward4<T, G_STBIN>;
-    case G_STMUL: return g_forward4<T, G_STMUL>;
-    case G_ST2: return g_forward4<T, G_ST2>;
-    case G_STEXP: return g_forward4<T, G_STEXP>;
-    case G_NB3: return g_forward4<T, G_NB3>;
-    default: return g_forward4<T, G_ZFIELD>;
-  }
-}
-
-template <typename T>
-static BwdK<T> bwd_kernel4(int op) {
-  switch (op) {
-    case G_STENCIL: return g_backward4<T, G_STENCIL>;
-    case G_STBIN: return g_backward4<T, G_STBIN>;
-    case G_STMUL: return g_backward4<T, G_STMUL>;
-    case G_ST2: return g_backward4<T, G_ST2>;
-    case G_STEXP: return g_backward4<T, G_STEXP>;
-    case G_NB3: return g_backward4<T, G_NB3>;
-    default: return g_backward4<T, G_SHIFT>;
-  }
-}
-
-template <typename T>
-static FwdPwK<T> fwd_kernel_pw(int op) {
-  switch (op) {
-    case G_ADD: return g_forward_pw<T, G_ADD>;
-    case G_SUB: return g_forward_pw<T, G_SUB>;
-    case G_MUL: return g_forward_pw<T, G_MUL>;
-    case G_DIV: return g_forward_pw<T, G_DIV>;
-    case G_MAX: return g_forward_pw<T, G_MAX>;
-    case G_EXP: return g_forward_pw<T, G_EXP>;
-    case G_LOG: return g_forward_pw<T, G_LOG>;
-    case G_LOG1P: return g_forward_pw<T, G_LOG1P>;
-    case G_SQRT: return g_forward_pw<T, G_SQRT>;
-    case G_ABS: return g_forward_pw<T, G_ABS>;
-    case G_AXPB: return g_forward_pw<T, G_AXPB>;
-    case G_CLAMPMIN: return g_forward_pw<T, G_CLAMPMIN>;
-    case G_CLAMPMAX: return g_forward_pw<T, G_CLAMPMAX>;
-    case G_STEP: return g_forward_pw<T, G_STEP>;
-    default: return g_forward_pw<T, G_CONST>;
-  }
-}
-
-template <typename T>
-static BwdPwK<T> bwd_kernel_pw(int op) {
-  switch (op) {
-    case G_ADD: return g_backward_pw<T, G_ADD>;
-    case G_SUB: return g_backward_pw<T, G_SUB>;
-    case G_MUL: return g_backward_pw<T, G_MUL>;
-    case G_DIV: return g_backward_pw<T, G_DIV>;
-    case G_MAX: return g_backward_pw<T, G_MAX>;
-    case G_EXP: return g_backward_pw<T, G_EXP>;
-    case G_LOG: return g_backward_pw<T, G_LOG>;
-    case G_LOG1P: return g_backward_pw<T, G_LOG1P>;
-    case G_SQRT: return g_backward_pw<T, G_SQRT>;
-    case G_ABS: return g_backward_pw<T, G_ABS>;
-    case G_AXPB: return g_backward_pw<T, G_AXPB>;
-    case G_CLAMPMIN: return g_backward_pw<T, G_CLAMPMIN>;
-    default: return g_backward_pw<T, G_CLAMPMAX>;
-  }
-}
-
-// Flat launch of a pointwise kernel: four cells a thread when every array is
-// 16-byte aligned and n a multiple of 4.
 static inline bool al16(const void* p) { return ((uintptr_t)p & 15) == 0; }
-// The four-x-cell stencil kernels: nx a multiple of 4 and shifts of one cell
-// (the arrays' alignment is checked per launch), for the kernels they made
-// faster.  The forward STMUL, which gathers two tap arrays, measured slower
-// with four cells (FP32, 128^3, ncu launch list: 16.8 us at 64 registers
-// against 15.9 with one cell) and keeps one cell a thread; every other
-// forward (ST2 17.5 against 19.2 once its two stencils were formed one after
-// the other) and every transpose is faster with four.
-static inline bool cells4(const GNode& nd, const Geo& g, bool bwd) {
-  if (g.nx % 4 != 0) return false;
-  if ((nd.op == G_SHIFT || nd.op == G_NB3) && nd.sk != 1 && nd.sk != -1) return false;
-  return bwd || nd.op != G_STMUL;
+
+// Block shape of a sweep with w cells a thread: the widest along x among those
+// that cover the box with the fewest threads (256 threads; at nx = 64 half the
+// lanes of a 32-lane row of four-cell threads have no cell).
+static dim3 level_block(const Geo& g, int w) {
+  static const int sh[6][3] = {{32, 2, 4}, {16, 4, 4}, {8, 8, 4}, {32, 8, 1}, {16, 16, 1}, {8, 32, 1}};
+  const long long lanes = (g.nx + w - 1) / w;
+  const int* best = sh[0];
+  long long least = -1;
+  for (const auto& s : sh) {
+    const long long t = (lanes + s[0] - 1) / s[0] * s[0] * ((g.ny + s[1] - 1) / s[1] * s[1]) *
+                        ((g.nz + s[2] - 1) / s[2] * s[2]);
+    if (least < 0 || t < least) {
+      least = t;
+      best = s;
+    }
+  }
+  return dim3((unsigned)best[0], (unsigned)best[1], (unsigned)best[2]);
 }
-static inline dim3 ggrid4(const Geo& g) {
-  return dim3((unsigned)((g.nx / 4 + GBX - 1) / GBX), (unsigned)((g.ny + GBY - 1) / GBY),
-              (unsigned)((g.nz + GBZ - 1) / GBZ));
-}
-static inline unsigned pw_blocks(long long work) {
-  const long long b = (work + 255) / 256;
-  return (unsigned)(b < 8192 ? (b > 0 ? b : 1) : 8192);
+struct LevelGrid {
+  dim3 b;
+  unsigned gx, gy;
+  int nzb;
+  LevelGrid(const Geo& g, int w) : b(level_block(g, w)) {
+    gx = (unsigned)((g.nx + b.x * w - 1) / (b.x * w));
+    gy = (unsigned)((g.ny + b.y - 1) / b.y);
+    nzb = (int)((g.nz + b.z - 1) / b.z);
+  }
+  int most(int cap) const { return std::max(1, std::min(cap, 65535 / nzb)); }   // gridDim.z
+  dim3 grid(int n) const { return dim3(gx, gy, (unsigned)(nzb * n)); }
+};
+
+// Four cells a thread: rows of whole 16-byte chunks, aligned arrays, shifts of
+// one cell.
+template <typename T>
+static bool cells4(const GraphExec<T>& G, T* const* a, int n) {
+  bool ok = G.geo.nx % 4 == 0 && G.near;
+  for (int i = 0; i < n; ++i) ok = ok && al16(a[i]);
+  return ok;
 }
 
-// Fork the auxiliary streams from s (they then follow everything enqueued on
-// s so far), and join them back into s.
-template <typename T>
-static int fork_streams(GraphExec<T>& G, cudaStream_t s) {
-  STG_CUDA_OK(cudaEventRecord(G.evfork, s));
-  for (int k = 0; k < G.nconc; ++k) STG_CUDA_OK(cudaStreamWaitEvent(G.aux[k], G.evfork, 0));
-  return STAGGER_OK;
-}
-template <typename T>
-static int join_streams(GraphExec<T>& G, cudaStream_t s) {
-  for (int k = 0; k < G.nconc; ++k) {
-    STG_CUDA_OK(cudaEventRecord(G.evjoin[k], G.aux[k]));
-    STG_CUDA_OK(cudaStreamWaitEvent(s, G.evjoin[k], 0));
+template <typename T, int W>
+static int forward_w(GraphExec<T>& G, cudaStream_t s) {
+  const Geo& g = G.geo;
+  const int nn = (int)G.def.nodes.size();
+  const LevelGrid lg(g, W);
+  FwdBatch<T> b;
+  const int most = lg.most(FwdBatch<T>::MAX);
+  for (int L = 1; L <= G.lp.nflev; ++L) {
+    b.n = 0;
+    auto flush = [&] {
+      if (!b.n) return;
+      b.rn = recip32(b.n);
+      g_level_fwd<T, W><<<lg.grid(b.n), lg.b, 0, s>>>(b, G.mesh, g);
+      ++G.launches;
+      b.n = 0;
+    };
+    for (int i = 0; i < nn; ++i) {
+      const GNode& nd = G.def.nodes[i];
+      if (nd.op == G_INPUT || G.lp.flev[i] != L) continue;
+      const T* A = nd.a >= 0 ? G.ptr[nd.a] : nullptr;
+      if (nd.op == G_PMEAN) {
+        const LevelGrid l1(g, 1);
+        g_plane_sum<T><<<g.nz, 256, 0, s>>>(A, G.psum, g);
+        g_plane_bcast<T><<<l1.grid(1), l1.b, 0, s>>>(G.psum, G.ptr[i], 0, g);
+        G.launches += 2;
+        continue;
+      }
+      b.t[b.n++] = {nd, A, nd.b >= 0 ? G.ptr[nd.b] : nullptr, nd.c >= 0 ? G.ptr[nd.c] : nullptr,
+                    G.ptr[i]};
+      if (b.n == most) flush();
+    }
+    flush();
   }
+  STG_CUDA_OK(cudaGetLastError());
   return STAGGER_OK;
 }
 
 template <typename T>
 int GraphExec<T>::forward(T* const in[8], cudaStream_t s) {
-  const size_t nn = def.nodes.size();
-  for (size_t i = 0; i < nn; ++i)
+  for (size_t i = 0; i < def.nodes.size(); ++i)
     if (def.nodes[i].op == G_INPUT) ptr[i] = in[def.nodes[i].sk];
-  const dim3 gg = ggrid(geo), gb(GBX, GBY, GBZ);
-  // Concurrent form: the stream of each node (-1: an input, ready at the fork).
-  std::vector<int> sto(nconc ? nn : 0, -1);
-  int rr = 0, prev_scr = -1;
-  if (nconc && fork_streams(*this, s)) return STAGGER_ECUDA;
-  for (size_t i = 0; i < nn; ++i) {
-    const GNode& nd = def.nodes[i];
-    if (nd.op == G_INPUT) continue;
-    const T* A = nd.a >= 0 ? ptr[nd.a] : nullptr;
-    const T* B = nd.b >= 0 ? ptr[nd.b] : nullptr;
-    const T* C = nd.c >= 0 ? ptr[nd.c] : nullptr;
-    cudaStream_t st = s;
-    if (nconc) {
-      // Follow the first operand's stream (chains stay on one stream); a node
-      // without a computed operand starts the next stream in turn.
-      int k = (nd.a >= 0 && sto[nd.a] >= 0) ? sto[nd.a]
-            : (nd.b >= 0 && sto[nd.b] >= 0) ? sto[nd.b]
-            : (nd.c >= 0 && sto[nd.c] >= 0) ? sto[nd.c] : (rr++ % nconc);
-      st = aux[k];
-      for (int o : {nd.a, nd.b, nd.c})
-        if (o >= 0 && sto[o] >= 0 && sto[o] != k) STG_CUDA_OK(cudaStreamWaitEvent(st, evn[o], 0));
-      if (nd.op == G_PMEAN && prev_scr >= 0 && sto[prev_scr] != k)
-        STG_CUDA_OK(cudaStreamWaitEvent(st, evn[prev_scr], 0));   // psum is shared
-      sto[i] = k;
+  // FP64 takes one cell a thread: its pipe, not the loads, is the bound (32^3
+  // adjoint step 2.8 ms against 3.8 with four).
+  if constexpr (sizeof(T) == sizeof(float))
+    if (cells4(*this, in, 8)) return forward_w<T, 4>(*this, s);
+  return forward_w<T, 1>(*this, s);
+}
+
+// The quench nodes q[0 .. n) of a level, nscr at a time.
+template <typename T, int W>
+static void quench_rev(GraphExec<T>& G, const std::vector<int>& q, const LevelGrid& lg,
+                       cudaStream_t s) {
+  const int most = lg.most(G.nscr);
+  for (size_t q0 = 0; q0 < q.size(); q0 += most) {
+    QuenchBatch<T> b;
+      b.n = (int)std::min<size_t>(most, q.size() - q0);
+    b.rn = recip32(b.n);
+    for (int j = 0; j < b.n; ++j) {
+      const int i = q[q0 + j];
+      b.nd[j] = G.def.nodes[i];
+      b.A[j] = G.ptr[G.def.nodes[i].a];
+      b.G[j] = G.grads + (size_t)G.lp.gslot[i] * G.geo.n;
+      b.scr[j] = G.qscr + (size_t)15 * j * G.geo.n;
     }
-    if (nd.op == G_PMEAN) {
-      g_plane_sum<T><<<geo.nz, 256, 0, st>>>(A, psum, geo);
-      g_plane_bcast<T><<<gg, gb, 0, st>>>(psum, ptr[i], 0, geo);
-      launches += 2;
-      prev_scr = (int)i;
-    } else if (nd.op == G_QUENCH) {
-      if (geo.nx % 4 == 0 && al16(A) && al16(ptr[i]))
-        g_quench_f4<T><<<ggrid4(geo), gb, 0, st>>>(nd, A, ptr[i], geo);
-      else
-        g_quench_f<T><<<gg, gb, 0, st>>>(nd, A, ptr[i], geo);
-      ++launches;
-    } else {
-      if (pointwise_op(nd.op)) {
-        const int vec = geo.n % 4 == 0 && al16(A) && al16(B) && al16(C) && al16(ptr[i]);
-        fwd_kernel_pw<T>(nd.op)<<<pw_blocks(vec ? geo.n / 4 : geo.n), 256, 0, st>>>(
-            nd, A, B, C, ptr[i], geo.n, vec);
-      } else if (cells4(nd, geo, false) && al16(A) && al16(B) && al16(C) && al16(ptr[i])) {
-        fwd_kernel4<T>(nd.op)<<<ggrid4(geo), gb, 0, st>>>(nd, A, B, C, ptr[i], mesh, geo);
-      } else {
-        fwd_kernel<T>(nd.op)<<<gg, gb, 0, st>>>(nd, A, B, C, ptr[i], mesh, geo);
-      }
-      ++launches;
-    }
-    if (nconc) STG_CUDA_OK(cudaEventRecord(evn[i], st));
+    g_level_quench<T, W, 0><<<lg.grid(b.n), lg.b, 0, s>>>(b, G.geo);
+    g_level_quench<T, W, 1><<<lg.grid(b.n), lg.b, 0, s>>>(b, G.geo);
+    g_level_quench<T, W, 2><<<lg.grid(b.n), lg.b, 0, s>>>(b, G.geo);
+    G.launches += 3;
   }
-  if (nconc && join_streams(*this, s)) return STAGGER_ECUDA;
+}
+
+template <typename T, int W>
+static int backward_w(GraphExec<T>& G, T* const seed[8], T* gin[8], cudaStream_t s) {
+  const Geo& g = G.geo;
+  const LevelPlan& P = G.lp;
+  const int nn = (int)G.def.nodes.size();
+  const LevelGrid lg(g, W);
+  const int most = lg.most(RevBatch<T>::MAX);
+  // The cotangent array of node i (-1 - k: the seed of output k).
+  auto garr = [&](int i) -> T* {
+    if (i >= 0 && P.alias[i] != P.OWN) i = P.alias[i];
+    return i < 0 ? seed[-1 - i] : G.grads + (size_t)P.gslot[i] * g.n;
+  };
+  RevBatch<T> b;
+  b.n = b.nterm = 0;
+  auto flush = [&] {
+    if (!b.n) return;
+    b.rn = recip32(b.n);
+    g_level_rev<T, W><<<lg.grid(b.n), lg.b, 0, s>>>(b, g);
+    ++G.launches;
+    b.n = b.nterm = 0;
+  };
+  for (int L = 0; L < P.nrlev; ++L) {
+    // The nodes with most terms first: their blocks run longest.
+    std::vector<int> lev;
+    for (int i = 0; i < nn; ++i)
+      if (P.rlev[i] == L && P.alias[i] == P.OWN) lev.push_back(i);
+    std::stable_sort(lev.begin(), lev.end(),
+                     [&](int x, int y) { return P.terms[x].size() > P.terms[y].size(); });
+    std::vector<int> quench, pmean;
+    for (int i : lev) {
+      const GNode& nd = G.def.nodes[i];
+      if (nd.op == G_QUENCH) quench.push_back(i);
+      if (nd.op == G_PMEAN) pmean.push_back(i);
+      const auto& tm = P.terms[i];
+      T* dst = nd.op == G_INPUT ? gin[nd.sk] : garr(i);
+      // An input's sum goes onto what gin holds; a sum of more than MAX terms
+      // runs in parts.
+      for (size_t t0 = 0; t0 < tm.size(); t0 += RevBatch<T>::MAX) {
+        const int n = (int)std::min<size_t>(RevBatch<T>::MAX, tm.size() - t0);
+        if (b.n == most || b.nterm + n > RevBatch<T>::MAX) flush();
+        const int add = t0 > 0 ? ADD_FIRST
+                      : nd.op != G_INPUT ? ADD_NO
+                      : (int)tm.size() <= RevBatch<T>::MAX ? ADD_LAST : ADD_FIRST;
+        b.t[b.n++] = {dst, b.nterm, n, add};
+        for (int q = 0; q < n; ++q) {
+          const auto& t = tm[t0 + q];
+          RevTerm<T>& r = b.c[b.nterm++];
+          r = RevTerm<T>();
+          r.role = t.role;
+          r.G = garr(t.consumer);
+          if (t.consumer < 0 || t.role == R_COPY) continue;
+          r.nd = G.def.nodes[t.consumer];
+          r.A = r.nd.a >= 0 ? G.ptr[r.nd.a] : nullptr;
+          r.B = r.nd.b >= 0 ? G.ptr[r.nd.b] : nullptr;
+          r.Y = G.ptr[t.consumer];
+        }
+        if (t0 + n < tm.size()) flush();   // the next part adds to this one's result
+      }
+    }
+    flush();
+    // Their own arrays become the operand's contribution.
+    quench_rev<T, W>(G, quench, lg, s);
+    for (int i : pmean) {
+      const LevelGrid l1(g, 1);
+      g_plane_sum<T><<<g.nz, 256, 0, s>>>(garr(i), G.psum, g);
+      g_plane_bcast<T><<<l1.grid(1), l1.b, 0, s>>>(G.psum, garr(i), 0, g);
+      G.launches += 2;
+    }
+  }
   STG_CUDA_OK(cudaGetLastError());
   return STAGGER_OK;
 }
@@ -324,104 +405,14 @@ int GraphExec<T>::forward(T* const in[8], cudaStream_t s) {
 template <typename T>
 int GraphExec<T>::backward(T* const seed[8], T* gin[8], cudaStream_t s) {
   if (!grads) return STAGGER_EINVAL;
-  const size_t nn = def.nodes.size();
-  const int bs = 256;
-  const dim3 gg = ggrid(geo), gb(GBX, GBY, GBZ);
-  // Seeds are the first contribution to the outputs' gradients: copy them.
-  for (int k = 0; k < 8; ++k)
-    STG_CUDA_OK(cudaMemcpyAsync(gptr(def.out[k]), seed[k],
-                                sizeof(T) * geo.n, cudaMemcpyDeviceToDevice, s));
-  // Concurrent form: the last launch that wrote each gradient array (-1: none
-  // since the fork), and its stream.
-  std::vector<int> lastw(nconc ? nn : 0, -1), sto(nconc ? nn : 0, -1);
-  int rr = 0, prev_scr = -1;
-  if (nconc && fork_streams(*this, s)) return STAGGER_ECUDA;
-  const std::vector<char>&wa = rp.wa, &wb = rp.wb, &wc = rp.wc;
-  for (long long i = (long long)nn - 1; i >= 0; --i) {
-    const GNode& nd = def.nodes[i];
-    if (!rp.hasg[i] || !has_transpose(nd.op)) continue;
-    const T* A = nd.a >= 0 ? ptr[nd.a] : nullptr;
-    const T* B = nd.b >= 0 ? ptr[nd.b] : nullptr;
-    T* gA = nd.a >= 0 ? gptr(nd.a) : nullptr;
-    T* gB = nd.b >= 0 ? gptr(nd.b) : nullptr;
-    T* gC = nd.c >= 0 ? gptr(nd.c) : nullptr;
-    cudaStream_t st = s;
-    if (nconc) {
-      // Wait for the complete gradient of this node, for the previous writer
-      // of each gradient it adds to, for the transpose that last read an
-      // array this launch writes first, and for the previous user of the
-      // shared scratch (quench, plane mean).
-      const int own = lastw[i];
-      int k = own >= 0 ? sto[own] : (rr++ % nconc);
-      st = aux[k];
-      const bool scr = nd.op == G_QUENCH || nd.op == G_PMEAN;
-      for (int w : {own, nd.a >= 0 ? lastw[nd.a] : -1, nd.b >= 0 ? lastw[nd.b] : -1,
-                    nd.c >= 0 ? lastw[nd.c] : -1, scr ? prev_scr : -1,
-                    wa[i] ? rp.gprev[nd.a] : -1, wb[i] ? rp.gprev[nd.b] : -1,
-                    wc[i] ? rp.gprev[nd.c] : -1})
-        if (w >= 0 && sto[w] != k) STG_CUDA_OK(cudaStreamWaitEvent(st, evn[w], 0));
-      sto[i] = k;
-      if (scr) prev_scr = (int)i;
-    }
-    if (nd.op == G_PMEAN) {
-      g_plane_sum<T><<<geo.nz, 256, 0, st>>>(gptr((int)i), psum, geo);
-      g_plane_bcast<T><<<gg, gb, 0, st>>>(psum, gA, wa[i] ? 0 : 1, geo);
-      launches += 2;
-    } else if (nd.op == G_QUENCH) {
-      T* Q = qscr + (size_t)7 * geo.n;   // q and its derivatives, 4 arrays per axis slot
-      T* gi = gptr((int)i);
-      if (geo.nx % 4 == 0 && al16(A) && al16(gi) && al16(gA) && al16(qscr)) {
-        const dim3 g4 = ggrid4(geo);
-        g_quench_q4<T><<<g4, gb, 0, st>>>(nd, A, Q, geo);
-        g_quench_b1_4<T><<<g4, gb, 0, st>>>(nd, A, Q, gi, qscr, geo);
-        g_quench_b3_4<T><<<g4, gb, 0, st>>>(nd, Q, qscr, gA, wa[i], geo);
-      } else {
-        g_quench_q<T><<<gg, gb, 0, st>>>(nd, A, Q, geo);
-        g_quench_b1<T><<<gg, gb, 0, st>>>(nd, A, Q, gi, qscr, geo);
-        g_quench_b3<T><<<gg, gb, 0, st>>>(nd, Q, qscr, gA, wa[i], geo);
-      }
-      launches += 3;
-    } else {
-      T* gi = gptr((int)i);
-      if (pointwise_op(nd.op)) {
-        const int vec = geo.n % 4 == 0 && al16(A) && al16(B) && al16(ptr[i]) && al16(gi) &&
-                        al16(gA) && al16(gB) && al16(gC);
-        bwd_kernel_pw<T>(nd.op)<<<pw_blocks(vec ? geo.n / 4 : geo.n), 256, 0, st>>>(
-            nd, A, B, ptr[i], gi, gA, gB, gC, wa[i], wb[i], wc[i], geo.n, vec);
-      } else if (cells4(nd, geo, true) && al16(A) && al16(B) && al16(ptr[i]) && al16(gi) &&
-                 al16(gA) && al16(gB) && al16(gC)) {
-        bwd_kernel4<T>(nd.op)<<<ggrid4(geo), gb, 0, st>>>(nd, A, B, ptr[i], gi, gA, gB, gC,
-                                                          wa[i], wb[i], wc[i], geo);
-      } else {
-        bwd_kernel<T>(nd.op)<<<gg, gb, 0, st>>>(nd, A, B, ptr[i], gi, gA, gB, gC, wa[i], wb[i],
-                                                wc[i], geo);
-      }
-      ++launches;
-    }
-    if (nconc) {
-      STG_CUDA_OK(cudaEventRecord(evn[i], st));
-      if (nd.a >= 0) lastw[nd.a] = (int)i;
-      if (nd.b >= 0) lastw[nd.b] = (int)i;
-      if (nd.c >= 0) lastw[nd.c] = (int)i;
-    }
-  }
-  if (nconc && join_streams(*this, s)) return STAGGER_ECUDA;
-  Add8<T> ad;
-  unsigned na = 0;
-  int vec = geo.n % 4 == 0;
-  for (int k = 0; k < 8; ++k) {
-    if (!rp.hasg[def.in[k]]) continue;   // the outputs do not depend on this input
-    ad.dst[na] = gin[k];
-    ad.src[na] = gptr(def.in[k]);
-    vec &= al16(ad.dst[na]) && al16(ad.src[na]);
-    ++na;
-  }
-  if (na) {
-    g_add_into8<T><<<dim3(pw_blocks(vec ? geo.n / 4 : geo.n), na), bs, 0, s>>>(ad, geo.n, vec);
-    ++launches;
-  }
-  STG_CUDA_OK(cudaGetLastError());
-  return STAGGER_OK;
+  T* in[8];
+  int ni = 0;
+  for (size_t i = 0; i < def.nodes.size() && ni < 8; ++i)
+    if (def.nodes[i].op == G_INPUT) in[ni++] = ptr[i];
+  if constexpr (sizeof(T) == sizeof(float))
+    if (cells4(*this, seed, 8) && cells4(*this, gin, 8) && cells4(*this, in, ni))
+      return backward_w<T, 4>(*this, seed, gin, s);
+  return backward_w<T, 1>(*this, seed, gin, s);
 }
 
 template struct GraphExec<float>;

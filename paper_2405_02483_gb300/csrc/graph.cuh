@@ -54,8 +54,11 @@ struct GNode {
   int c = -1, pop = 0;
   // Float copies of the constants, for the FP32 kernels, and whether the
   // epilogue is other than the identity (set when the graph is complete).
-  float f0 = 0, f1 = 0, f2 = 0, fh2 = 0, fps = 1, fpt = 0;
+  float f0 = 0, f1 = 0, f2 = 0, fps = 1, fpt = 0;
   int ep = 0;
+  // Inverse spacings of the stencils (1 / c0, 1 / h2) and their float copies.
+  double ic0 = 1, ih2 = 1;
+  float fi0 = 1, fih2 = 1;
 };
 
 // Precision-independent description of the graph.
@@ -137,12 +140,24 @@ inline bool has_transpose(int op) {
   return op != G_INPUT && op != G_CONST && op != G_ZFIELD && op != G_STEP;
 }
 
-#ifndef GRAPH_NSTREAMS
-#define GRAPH_NSTREAMS 4
-#endif
+// The sweeps' schedule.  flev: a node's forward level (inputs 0).  The
+// reverse gathers: terms of a node are the consumers that pass it a cotangent
+// and their operand role (graph_kernels.cuh), consumer -1 - k for the seed of
+// output k; rlev its level (-1: no cotangent), alias the node (or -1 - k the
+// seed) whose array it shares (OWN: none, its array is gslot).
+struct LevelPlan {
+  static constexpr int OWN = -1000;
+  struct Term {
+    int consumer, role;
+  };
+  std::vector<int> flev, rlev, alias, gslot;
+  std::vector<std::vector<Term>> terms;
+  int nflev = 0, nrlev = 0, nslots = 0;
+};
 
-// Device executor for one precision.  Holds one value and one gradient array
-// of n cells per node (inputs point at caller memory and need none).
+// Device executor for one precision.  Holds one value array of n cells per
+// node (inputs point at caller memory and need none) and the cotangent arrays
+// of the plan, reused by liveness.
 template <typename T>
 struct GraphExec {
   GraphDef def;
@@ -150,23 +165,13 @@ struct GraphExec {
   T* vals = nullptr;     // node values (non-input nodes)
   T* mesh = nullptr;     // the mesh arrays of G_ZFIELD on the device, or null
   T* psum = nullptr;     // per-plane sums of G_PMEAN (nz), or null
-  T* qscr = nullptr;     // 15 arrays of scratch for the G_QUENCH transpose, or null
-  T* grads = nullptr;    // gradient arrays (rp.nslots, reused by liveness)
+  T* qscr = nullptr;     // scratch of the G_QUENCH transposes, nscr sets of 15 arrays, or null
+  T* grads = nullptr;    // cotangent arrays (lp.nslots)
+  int nscr = 0;
+  bool near = true;      // every shift is one cell
   std::vector<T*> ptr;   // value pointer per node
-  ReversePlan rp;        // the reverse sweep's gradient flags and arrays
-  T* gptr(int i) { return grads + (size_t)rp.gslot[i] * geo.n; }
+  LevelPlan lp;
   long long launches = 0;
-  // Concurrent sweeps: with nconc auxiliary streams each node's launch waits
-  // only on the launches it depends on (its operands' values in the forward;
-  // its own gradient and the previous writer of each gradient it adds to in
-  // the reverse; the previous user of the shared quench and plane-mean
-  // scratch), so a sweep captured into a CUDA graph becomes a DAG whose
-  // independent kernels overlap.  0: one stream, in node order.
-  int nconc = 0;
-  cudaStream_t aux[GRAPH_NSTREAMS] = {};
-  std::vector<cudaEvent_t> evn;
-  cudaEvent_t evfork = nullptr, evjoin[GRAPH_NSTREAMS] = {};
-  int enable_concurrency();
 
   int init(const GraphDef& d, const Geo& g, bool with_grads);
   void release();

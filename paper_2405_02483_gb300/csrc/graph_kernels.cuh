@@ -11,11 +11,7 @@
 
 namespace stg {
 
-// ---------------------------------------------------------------------------
-// A cell of a graph launch: 3-D grid of GB x GBY x GBZ thread blocks, so the
-// cell's (i, j, k) come from the launch and a periodic neighbour needs no
-// division.
-// ---------------------------------------------------------------------------
+// The launch shape of the one-cell kernels (threads along x, y, z).
 #ifndef GBX
 #define GBX 32
 #endif
@@ -25,38 +21,29 @@ namespace stg {
 #ifndef GBZ
 #define GBZ 4
 #endif
+#define GZU 1   // cells a thread takes along z
 
+// The cells of a thread: W consecutive x-cells i .. i + W - 1 of row (j, k), W 1
+// or 4 (4 needs nx a multiple of 4 and 16-byte aligned arrays: each tap is then
+// one 16-byte load and the index work is shared by four cells).  Every lane
+// takes the one-cell arithmetic, so the values do not depend on W.
 struct GCell {
   int i, j, k;
-  long long idx;
+  int idx;   // (a box has less than 2^31 cells)
 };
 
-__device__ __forceinline__ bool gcell(GCell& c, const Geo& g) {
-  c.i = blockIdx.x * blockDim.x + threadIdx.x;
+template <int W>
+__device__ __forceinline__ bool gcell_at(GCell& c, int kb, const Geo& g) {
+  c.i = W * (int)(blockIdx.x * blockDim.x + threadIdx.x);
   c.j = blockIdx.y * blockDim.y + threadIdx.y;
-  c.k = blockIdx.z * blockDim.z + threadIdx.z;
+  c.k = kb * (int)blockDim.z + (int)threadIdx.z;
   if (c.i >= g.nx || c.j >= g.ny || c.k >= g.nz) return false;
-  c.idx = (long long)c.k * g.sz + (long long)c.j * g.sy + c.i;
+  c.idx = c.k * (int)g.sz + c.j * (int)g.sy + c.i;
   return true;
 }
-
-// A thread of a graph launch takes GZU cells along z: its first cell from the
-// launch, then steps of the launch's z extent (gridDim.z * GBZ).  The
-// pointwise and stencil kernels compute every value before they store any,
-// so that GZU loads of each operand are in flight together.  One cell per
-// thread measured fastest on GB300 (adjoint step at 128^3: 25.3 / 26.5 / 26.7
-// / 32.4 ms with 1 / 2 / 4 / 8): the per-op kernels are small enough that
-// occupancy, not loads per thread, sets their throughput.
-#ifndef GZU
-#define GZU 1
-#endif
-
-__device__ __forceinline__ GCell gcell_at(const GCell& c0, int u, const Geo& g) {
-  GCell c = c0;
-  const int dz = u * (int)(gridDim.z * blockDim.z);
-  c.k += dz;
-  c.idx += (long long)dz * g.sz;
-  return c;
+template <int W>
+__device__ __forceinline__ bool gcell(GCell& c, const Geo& g) {
+  return gcell_at<W>(c, (int)blockIdx.z, g);
 }
 
 // A node's constant in the sweep's precision: the FP32 kernels read the
@@ -68,62 +55,166 @@ __device__ __forceinline__ T kc(double d, float f) {
   else return d;
 }
 
-// Periodic neighbour of cell c along an axis (shifted by o).
-__device__ __forceinline__ long long nbr(const GCell& c, int axis, int o, const Geo& g) {
-  if (axis == 0) return c.idx + (wrap(c.i + o, g.nx) - c.i);
-  if (axis == 1) return c.idx + (long long)(wrap(c.j + o, g.ny) - c.j) * g.sy;
-  return c.idx + (long long)(wrap(c.k + o, g.nz) - c.k) * g.sz;
-}
-
-// The values v(j) at the seven taps c - 3 .. c + 3 along an axis: plain
-// strides away from the periodic seam, wrapped indices within 3 cells of it.
-template <typename T, class V>
-__device__ __forceinline__ void taps7(V v, const GCell& c, int axis, const Geo& g, T t[7]) {
-  const long long st = axis == 0 ? 1 : axis == 1 ? g.sy : g.sz;
-  const int pos = axis == 0 ? c.i : axis == 1 ? c.j : c.k;
-  const int n = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
-  if (pos >= 3 && pos + 3 < n) {
-#pragma unroll
-    for (int o = -3; o <= 3; ++o) t[o + 3] = v(c.idx + o * st);
+// W consecutive elements i .. as 16-byte loads and stores (W = 4) or one.
+template <typename T>
+__device__ __forceinline__ void ld4(const T* p, long long i, T (&v)[4]) {
+  if constexpr (sizeof(T) == sizeof(float)) {
+    const float4 x = *reinterpret_cast<const float4*>(p + i);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
   } else {
+    const double2 x = *reinterpret_cast<const double2*>(p + i);
+    const double2 y = *reinterpret_cast<const double2*>(p + i + 2);
+    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
+  }
+}
+template <typename T>
+__device__ __forceinline__ void st4(T* p, long long i, const T (&v)[4]) {
+  if constexpr (sizeof(T) == sizeof(float)) {
+    *reinterpret_cast<float4*>(p + i) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+    *reinterpret_cast<double2*>(p + i) = make_double2(v[0], v[1]);
+    *reinterpret_cast<double2*>(p + i + 2) = make_double2(v[2], v[3]);
+  }
+}
+template <typename T, int W>
+__device__ __forceinline__ void ldw(const T* p, int i, T (&v)[W]) {
+  if constexpr (W == 4) ld4(p, i, v);
+  else v[0] = p[i];
+}
+template <typename T, int W>
+__device__ __forceinline__ void stw(T* p, int i, const T (&v)[W]) {
+  if constexpr (W == 4) st4(p, i, v);
+  else p[i] = v[0];
+}
+
+// t[o + K][l]: f at cell (i + l, j, k) + o e_axis, o = -K .. K (K <= 3):
+// plain strides away from the periodic seam, wrapped indices next to it.
+template <int K, int W, typename T>
+__device__ __forceinline__ void taps(const T* f, const GCell& c, int axis, const Geo& g,
+                                     T (&t)[2 * K + 1][W]) {
+  if (W == 4 && axis == 0) {
+    const int row = c.idx - c.i;
+    T L[W], M[W], R[W];
+    ldw<T, W>(f, row + wrap(c.i - 4, g.nx), L);
+    ldw<T, W>(f, c.idx, M);
+    ldw<T, W>(f, row + wrap(c.i + 4, g.nx), R);
 #pragma unroll
-    for (int o = -3; o <= 3; ++o) t[o + 3] = v(c.idx + (long long)(wrap(pos + o, n) - pos) * st);
+    for (int o = -K; o <= K; ++o)
+#pragma unroll
+      for (int l = 0; l < W; ++l) {
+        const int q = 4 + l + o;   // in the 12-cell window i - 4 .. i + 7
+        t[o + K][l] = q < 4 ? L[q & (W - 1)] : q < 8 ? M[(q - 4) & (W - 1)] : R[(q - 8) & (W - 1)];
+      }
+  } else {
+    const int st = axis == 0 ? 1 : axis == 1 ? (int)g.sy : (int)g.sz;
+    const int pos = axis == 0 ? c.i : axis == 1 ? c.j : c.k;
+    const int n = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
+    const bool inner = pos >= K && pos + K < n;
+#pragma unroll
+    for (int o = -K; o <= K; ++o)
+      ldw<T, W>(f, c.idx + (inner ? o : wrap(pos + o, n) - pos) * st, t[o + K]);
   }
 }
 
-// A stencil from the values at its seven taps t[0..6] = c - 3 .. c + 3: up/dn
-// are eq. (interp) to i+1/2 and i-1/2; ddup/dddn are eq. (deriv) to i+1/2 and
-// i-1/2, divided by the spacing h.
-template <typename T>
-__device__ __forceinline__ T st_comb(int kind, T h, const T t[7]) {
-  const T IA = (T)STG_IA, IB = (T)STG_IB, IC = (T)STG_IC;
-  const T DA = (T)STG_DA, DB = (T)STG_DB, DC = (T)STG_DC;
-  const T m3 = t[0], m2 = t[1], m1 = t[2], z0 = t[3], p1 = t[4], p2 = t[5], p3 = t[6];
-  switch (kind) {
-    case ST_UP: return IA * (z0 + p1) + IB * (m1 + p2) + IC * (m2 + p3);
-    case ST_DN: return IA * (m1 + z0) + IB * (m2 + p1) + IC * (m3 + p2);
-    case ST_DDUP: return (DA * (p1 - z0) + DB * (p2 - m1) + DC * (p3 - m2)) / h;
-    default: return (DA * (z0 - m1) + DB * (p1 - m2) + DC * (p2 - m3)) / h;
+// v[l]: f at cell (i + l, j, k) + o e_axis; with W = 4 along x |o| <= 3.
+template <int W, typename T>
+__device__ __forceinline__ void tap(const T* f, const GCell& c, int axis, int o, const Geo& g,
+                                    T (&v)[W]) {
+  if (W == 4 && axis == 0) {
+    T t[7][W];
+    taps<3, W>(f, c, 0, g, t);
+#pragma unroll
+    for (int l = 0; l < W; ++l)
+      v[l] = o == -1 ? t[2][l] : o == 1 ? t[4][l] : o == 0 ? t[3][l] : o == -2 ? t[1][l]
+           : o == 2 ? t[5][l] : o == -3 ? t[0][l] : t[6][l];
+  } else {
+    const int st = axis == 0 ? 1 : axis == 1 ? (int)g.sy : (int)g.sz;
+    const int pos = axis == 0 ? c.i : axis == 1 ? c.j : c.k;
+    const int n = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
+    ldw<T, W>(f, c.idx + (wrap(pos + o, n) - pos) * st, v);
   }
 }
 
-// Stencil value of f at c.
-template <typename T>
-__device__ __forceinline__ T stencil_at(const T* f, const GCell& c, int axis, int kind, T h,
-                                        const Geo& g) {
-  T t[7];
-  taps7<T>([&](long long j) { return f[j]; }, c, axis, g, t);
-  return st_comb(kind, h, t);
+// The six taps of a stencil: t[q][l] is f at cell (i + l, j, k) + (q - 2 - dn) e_axis
+// (c - 2 .. c + 3 for the upward kinds, c - 3 .. c + 2 for the downward ones).
+template <int W, typename T>
+__device__ __forceinline__ void taps6(const T* f, const GCell& c, int axis, int dn, const Geo& g,
+                                      T (&t)[6][W]) {
+  if (W == 4 && axis == 0) {
+    const int row = c.idx - c.i;
+    T w[3][W];   // the 12-cell window i - 4 .. i + 7
+    ldw<T, W>(f, row + wrap(c.i - 4, g.nx), w[0]);
+    ldw<T, W>(f, c.idx, w[1]);
+    ldw<T, W>(f, row + wrap(c.i + 4, g.nx), w[2]);
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+#pragma unroll
+      for (int l = 0; l < W; ++l) {
+        const int u = 2 + q + l, d = 1 + q + l;
+        t[q][l] = dn ? w[d / 4][d & (W - 1)] : w[u / 4][u & (W - 1)];
+      }
+  } else {
+    const int st = axis == 0 ? 1 : axis == 1 ? (int)g.sy : (int)g.sz;
+    const int pos = (axis == 0 ? c.i : axis == 1 ? c.j : c.k) - 2 - dn;
+    const int n = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
+    const int base = c.idx - (2 + dn) * st;
+    if (pos >= 0 && pos + 5 < n) {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) ldw<T, W>(f, base + q * st, t[q]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) ldw<T, W>(f, base + (wrap(pos + q, n) - pos) * st, t[q]);
+    }
+  }
 }
 
-// The same stencil of the values v(idx) of a functor at the taps.
-template <typename T, class V>
-__device__ __forceinline__ T stencil_fn(V v, const GCell& c, int axis, int kind, T h,
-                                        const Geo& g) {
-  T t[7];
-  taps7<T>(v, c, axis, g, t);
-  return st_comb(kind, h, t);
+// A stencil (kind, inverse spacing ih) from its six taps: up/dn are eq.
+// (interp) to i+1/2 and i-1/2, ddup/dddn eq. (deriv) to i+1/2 and i-1/2.  One
+// form for the four kinds, sums for the interpolations and differences for the
+// derivatives by the factor s (the kind is known at run time only, and a
+// switch over four forms was a third of the sweeps' instructions).  Times the
+// inverse spacing: a division per cell was half the work of an FP64
+// derivative on the narrow FP64 pipe.
+template <int W, typename T>
+__device__ __forceinline__ void st_comb(int kind, T ih, const T (&t)[6][W], T (&v)[W]) {
+  const bool d = kind >= ST_DDUP;
+  const T s = d ? (T)-1 : (T)1;
+  const T a = d ? (T)STG_DA : (T)STG_IA, b = d ? (T)STG_DB : (T)STG_IB, e = d ? (T)STG_DC : (T)STG_IC;
+#pragma unroll
+  for (int l = 0; l < W; ++l)
+    v[l] = (a * (t[3][l] + s * t[2][l]) + b * (t[4][l] + s * t[1][l]) + e * (t[5][l] + s * t[0][l])) * ih;
 }
+__device__ __forceinline__ int st_down(int kind) { return kind & 1; }   // ST_DN, ST_DDDN
+// A node's first and second stencil's inverse spacing.
+template <typename T> __device__ __forceinline__ T ih1(const GNode& nd) { return kc<T>(nd.ic0, nd.fi0); }
+template <typename T> __device__ __forceinline__ T ih2(const GNode& nd) { return kc<T>(nd.ih2, nd.fih2); }
+
+// The stencil (kind, axis, inverse spacing) of f at the thread's cells.
+template <int W, typename T>
+__device__ __forceinline__ void stencil(const T* f, const GCell& c, int axis, int kind, T ih,
+                                        const Geo& g, T (&v)[W]) {
+  T t[6][W];
+  taps6<W>(f, c, axis, st_down(kind), g, t);
+  st_comb<W>(kind, ih, t, v);
+}
+// The stencil of the product f (h - s): one tap array live, the product
+// formed as its second factor arrives.
+template <int W, typename T>
+__device__ __forceinline__ void stencil_mul(const T* f, const T* h, T s, const GCell& c, int axis,
+                                            int kind, T ih, const Geo& g, T (&v)[W]) {
+  T t[6][W];
+  taps6<W>(f, c, axis, st_down(kind), g, t);
+  {
+    T u[6][W];
+    taps6<W>(h, c, axis, st_down(kind), g, u);
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+#pragma unroll
+      for (int l = 0; l < W; ++l) t[q][l] = t[q][l] * (u[q][l] - s);
+  }
+  st_comb<W>(kind, ih, t, v);
+}
+
 // Transposed kind and sign of a stencil: up^T = dn, dn^T = up, ddup^T =
 // -dddn, dddn^T = -ddup (periodic summation by parts).
 __device__ __forceinline__ int st_transpose(int kind) {
@@ -176,10 +267,10 @@ __device__ __forceinline__ T q_val(T vm, T v0, T vp, T iq, T eps, T* dq) {
     T wim, wi0, woi, wop;
     max_w(am, a0, wim, wi0);
     max_w(inner, ap, woi, wop);
-    // a2 / den^2 as q / den: den^2 underflows in FP32 where T and D2 T are
+    // a2 / den^2 as q times 1 / den: den^2 underflows in FP32 where T and D2 T are
     // both zero (den = 1e-30), and 0 / 0 would poison the cotangent.
-    const T qd = qdiv(q, den);
-    const T dq_da2 = qdiv((T)1, den) - iq * qd;
+    const T rd = qdiv((T)1, den), qd = q * rd;
+    const T dq_da2 = rd - iq * qd;
     const T dq_dM = -qd;
     const T sd = sgn(d2);
     dq[0] = dq_da2 * sd + dq_dM * (cM * (woi * wim)) * sgn(vm);
@@ -188,13 +279,6 @@ __device__ __forceinline__ T q_val(T vm, T v0, T vp, T iq, T eps, T* dq) {
   }
   return q;
 }
-template <typename T>
-__device__ __forceinline__ T q_at(const T* A, const GCell& c, int ax, int s, T iq, T eps,
-                                  const Geo& g, T* dq) {
-  return q_val(A[nbr(c, ax, s - 1, g)], A[nbr(c, ax, s, g)], A[nbr(c, ax, s + 1, g)], iq, eps,
-               dq);
-}
-
 // fac at c, and (when wq) the weights of the three q of each axis in fac:
 // wq[3 t + p + 1] for axis t and position p.  qf(t, ax, s) is q at
 // c + s e_ax (axis slot t): formed from T, or read from the transpose's
@@ -231,89 +315,87 @@ __device__ __forceinline__ T quench_fac(QF qf, int a0, int a1, T* wq) {
 // Transpose, q pass (per cell z, per axis slot t): q(z) and its derivatives
 // with respect to T at z - 1, z, z + 1, into Q[(4 t + 0 .. 3) n + z], formed
 // once here instead of at every tap of the two passes that follow.
-template <typename T>
-__global__ void g_quench_q(GNode nd, const T* A, T* Q, Geo g) {
-  GCell c0;
-  if (!gcell(c0, g)) return;
+template <typename T, int W>
+__device__ __forceinline__ void quench_q(const GNode& nd, const T* A, T* Q, const GCell& c,
+                                         const Geo& g) {
   const T iq = (T)1 / kc<T>(nd.c0, nd.f0), eps = kc<T>(nd.c2, nd.f2);
-  for (int u = 0; u < GZU; ++u) {
-    const GCell c = gcell_at(c0, u, g);
-    if (c.k >= g.nz) break;
-    for (int t = 0; t < 2; ++t) {
-      const int ax = t == 0 ? nd.axis : nd.sk;
-      if (ax < 0) continue;
+  for (int t = 0; t < 2; ++t) {
+    const int ax = t == 0 ? nd.axis : nd.sk;
+    if (ax < 0) continue;
+    T ta[3][W], q[W], d0[W], d1[W], d2[W];
+    taps<1, W>(A, c, ax, g, ta);
+#pragma unroll
+    for (int l = 0; l < W; ++l) {
       T dq[3];
-      const T q = q_at(A, c, ax, 0, iq, eps, g, dq);
-      Q[(long long)(4 * t) * g.n + c.idx] = q;
-      for (int k = 0; k < 3; ++k) Q[(long long)(4 * t + 1 + k) * g.n + c.idx] = dq[k];
+      q[l] = q_val(ta[0][l], ta[1][l], ta[2][l], iq, eps, dq);
+      d0[l] = dq[0];
+      d1[l] = dq[1];
+      d2[l] = dq[2];
     }
+    stw<T, W>(Q + (long long)(4 * t) * g.n, c.idx, q);
+    stw<T, W>(Q + (long long)(4 * t + 1) * g.n, c.idx, d0);
+    stw<T, W>(Q + (long long)(4 * t + 2) * g.n, c.idx, d1);
+    stw<T, W>(Q + (long long)(4 * t + 3) * g.n, c.idx, d2);
   }
 }
 
 // Transpose, first pass (per output cell y): S0 = gbar C (the product's own
 // term) and S[1 + 3 t + p + 1] = gbar T dC/dfac dfac/dq, the cotangent each
 // q of axis t at position p receives from y.
-template <typename T>
-__global__ void g_quench_b1(GNode nd, const T* A, const T* Q, const T* gout, T* S, Geo g) {
-  GCell c0;
-  if (!gcell(c0, g)) return;
+template <typename T, int W>
+__device__ __forceinline__ void quench_b1(const GNode& nd, const T* A, const T* Q, const T* gout,
+                                          T* S, const GCell& c, const Geo& g) {
   const T qlim = kc<T>(nd.c1, nd.f1);
-  for (int u = 0; u < GZU; ++u) {
-    const GCell c = gcell_at(c0, u, g);
-    if (c.k >= g.nz) break;
+  T tq[2][3][W];   // q at offsets -1 .. 1 along each axis slot
+  taps<1, W>(Q, c, nd.axis, g, tq[0]);
+  if (nd.sk >= 0) taps<1, W>(Q + 4 * g.n, c, nd.sk, g, tq[1]);
+  T a[W], gg[W], s0[W], sw[6][W];
+  ldw<T, W>(A, c.idx, a);
+  ldw<T, W>(gout, c.idx, gg);
+#pragma unroll
+  for (int l = 0; l < W; ++l) {
     T wq[6];
-    const T fac = quench_fac<T>(
-        [&](int t, int ax, int s) { return Q[(long long)(4 * t) * g.n + nbr(c, ax, s, g)]; },
-        nd.axis, nd.sk, wq);
-    const T gg = gout[c.idx];
+    const T fac = quench_fac<T>([&](int t, int, int s) { return tq[t][s + 1][l]; }, nd.axis,
+                                nd.sk, wq);
     const T C = fac > qlim ? qlim : fac;
     const T dC = fac <= qlim ? (T)1 : (T)0;
-    const T base = gg * A[c.idx] * dC;
-    S[c.idx] = gg * C;
-    for (int j = 0; j < 6; ++j) S[(long long)(1 + j) * g.n + c.idx] = base * wq[j];
+    const T base = gg[l] * a[l] * dC;
+    s0[l] = gg[l] * C;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) sw[j][l] = base * wq[j];
   }
+  stw<T, W>(S, c.idx, s0);
+#pragma unroll
+  for (int j = 0; j < 6; ++j)
+    if (j < 3 || nd.sk >= 0) stw<T, W>(S + (long long)(1 + j) * g.n, c.idx, sw[j]);
 }
 
 // Transpose, second pass (per input cell x): Tbar(x) = S0(x) + the sum over
 // the axes and the three q positions z = x + r e_a whose stencils hold x of
-// qbar(z) dq(z)/dT(x), qbar(z) = sum_p S[.. p](z - p e_a).
-template <typename T>
-__global__ void g_quench_b3(GNode nd, const T* Q, const T* S, T* gA, int wA, Geo g) {
-  GCell c0;
-  if (!gcell(c0, g)) return;
-  for (int u = 0; u < GZU; ++u) {
-    const GCell c = gcell_at(c0, u, g);
-    if (c.k >= g.nz) break;
-    T acc = S[c.idx];
-    for (int t = 0; t < 2; ++t) {
-      const int ax = t == 0 ? nd.axis : nd.sk;
-      if (ax < 0) continue;
-      for (int r = -1; r <= 1; ++r) {
+// qbar(z) dq(z)/dT(x), qbar(z) = sum_p S[.. p](z - p e_a).  Reads Q and S only.
+template <typename T, int W>
+__device__ __forceinline__ void quench_b3(const GNode& nd, const T* Q, const T* S, const GCell& c,
+                                          const Geo& g, T (&acc)[W]) {
+  ldw<T, W>(S, c.idx, acc);
+  for (int t = 0; t < 2; ++t) {
+    const int ax = t == 0 ? nd.axis : nd.sk;
+    if (ax < 0) continue;
+    T ts[3][5][W];   // S of q position p = -1 .. 1 at offsets -2 .. 2
+#pragma unroll
+    for (int p = 0; p < 3; ++p) taps<2, W>(S + (long long)(1 + 3 * t + p) * g.n, c, ax, g, ts[p]);
+    T td[3][W];      // d q(z) / d T at its tap 1 - r, z at offsets r = -1 .. 1
+#pragma unroll
+    for (int r = -1; r <= 1; ++r)
+      tap<W>(Q + (long long)(4 * t + 2 - r) * g.n, c, ax, r, g, td[r + 1]);
+#pragma unroll
+    for (int r = -1; r <= 1; ++r)
+#pragma unroll
+      for (int l = 0; l < W; ++l) {
         T qbar = 0;
-        for (int p = -1; p <= 1; ++p)
-          qbar += S[(long long)(1 + 3 * t + p + 1) * g.n + nbr(c, ax, r - p, g)];
-        // d q(z) / d T(x), z = x + r e_ax: the derivative at z's tap 1 - r.
-        acc += qbar * Q[(long long)(4 * t + 2 - r) * g.n + nbr(c, ax, r, g)];
+#pragma unroll
+        for (int p = -1; p <= 1; ++p) qbar += ts[p + 1][r - p + 2][l];
+        acc[l] += qbar * td[r + 1][l];
       }
-    }
-    gA[c.idx] = wA ? acc : gA[c.idx] + acc;
-  }
-}
-
-// Quench forward (G_QUENCH): out = T min(fac, qlim).
-template <typename T>
-__global__ void g_quench_f(GNode nd, const T* A, T* out, Geo g) {
-  GCell c0;
-  if (!gcell(c0, g)) return;
-  for (int u = 0; u < GZU; ++u) {
-    const GCell c = gcell_at(c0, u, g);
-    if (c.k >= g.nz) break;
-    const T iq = (T)1 / kc<T>(nd.c0, nd.f0), qlim = kc<T>(nd.c1, nd.f1);
-    const T eps = kc<T>(nd.c2, nd.f2);
-    const T fac = quench_fac<T>(
-        [&](int, int ax, int s) { return q_at(A, c, ax, s, iq, eps, g, (T*)nullptr); }, nd.axis,
-        nd.sk, (T*)nullptr);
-    out[c.idx] = A[c.idx] * (fac > qlim ? qlim : fac);
   }
 }
 
@@ -325,40 +407,14 @@ __device__ __forceinline__ T stbin_val(const GNode& nd, T st, T b) {
   return nd.side ? b - st : st - b;     // G_SUB
 }
 
-template <typename T>
-__device__ __forceinline__ T fwd_value(int op, const GNode& nd, const T* A, const T* B,
-                                       const T* mesh, const GCell& c, const Geo& g) {
-  const long long idx = c.idx;
-  switch (op) {
-    case G_STENCIL: return stencil_at(A, c, nd.axis, nd.sk, kc<T>(nd.c0, nd.f0), g);
-    case G_STBIN:
-      return stbin_val(nd, stencil_at(A, c, nd.axis, nd.sk, kc<T>(nd.c0, nd.f0), g), B[idx]);
-    case G_STMUL:
-      return stencil_fn<T>([&](long long j) { return A[j] * B[j]; }, c, nd.axis, nd.sk,
-                           kc<T>(nd.c0, nd.f0), g);
-    case G_STEXP: return exp(stencil_at(A, c, nd.axis, nd.sk, kc<T>(nd.c0, nd.f0), g));
-    case G_NB3: {
-      const T m = A[nbr(c, nd.axis, nd.sk, g)], z = A[idx], p = A[nbr(c, nd.axis, -nd.sk, g)];
-      if (nd.iop == G_ADD) return (m + z) + p;
-      const T in = m >= z ? m : z;
-      return in >= p ? in : p;
-    }
-    case G_ST2: {
-      const T s1 = stencil_at(A, c, nd.axis, nd.sk, kc<T>(nd.c0, nd.f0), g);
-      const T s2 = stencil_at(B, c, nd.axis2, nd.sk2, kc<T>(nd.h2, nd.fh2), g);
-      return nd.iop == G_ADD ? s1 + s2 : s1 - s2;
-    }
-    case G_SHIFT: return A[nbr(c, nd.axis, nd.sk, g)];
-    default: return mesh[(long long)nd.sk * g.nz + c.k];   // G_ZFIELD
-  }
-}
-
 // The ops whose value at a cell reads only that cell of their operands: they
 // run as flat kernels over the arrays (g_forward_pw, g_backward_pw).
 __host__ __device__ __forceinline__ bool pointwise_op(int op) {
-  return op == G_ADD || op == G_SUB || op == G_MUL || op == G_DIV || op == G_MAX ||
-         op == G_EXP || op == G_LOG || op == G_LOG1P || op == G_SQRT || op == G_ABS ||
-         op == G_AXPB || op == G_CLAMPMIN || op == G_CLAMPMAX || op == G_STEP || op == G_CONST;
+  constexpr unsigned mask = 1u << G_ADD | 1u << G_SUB | 1u << G_MUL | 1u << G_DIV | 1u << G_MAX |
+                            1u << G_EXP | 1u << G_LOG | 1u << G_LOG1P | 1u << G_SQRT |
+                            1u << G_ABS | 1u << G_AXPB | 1u << G_CLAMPMIN | 1u << G_CLAMPMAX |
+                            1u << G_STEP | 1u << G_CONST;
+  return (mask >> op) & 1u;
 }
 
 // A pointwise op's value from its operands' values a, b at the cell.
@@ -390,154 +446,91 @@ __device__ __forceinline__ T finish(const GNode& nd, T v, T cv) {
   return nd.ep ? kc<T>(nd.ps, nd.fps) * v + kc<T>(nd.pt, nd.fpt) : v;
 }
 
-// Four consecutive elements i .. i + 3 as 16-byte loads and stores (i a
-// multiple of 4, the array 16-byte aligned).
-template <typename T>
-__device__ __forceinline__ void ld4(const T* p, long long i, T (&v)[4]) {
-  if constexpr (sizeof(T) == sizeof(float)) {
-    const float4 x = *reinterpret_cast<const float4*>(p + i);
-    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-  } else {
-    const double2 x = *reinterpret_cast<const double2*>(p + i);
-    const double2 y = *reinterpret_cast<const double2*>(p + i + 2);
-    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
-  }
-}
-template <typename T>
-__device__ __forceinline__ void st4(T* p, long long i, const T (&v)[4]) {
-  if constexpr (sizeof(T) == sizeof(float)) {
-    *reinterpret_cast<float4*>(p + i) = make_float4(v[0], v[1], v[2], v[3]);
-  } else {
-    *reinterpret_cast<double2*>(p + i) = make_double2(v[0], v[1]);
-    *reinterpret_cast<double2*>(p + i + 2) = make_double2(v[2], v[3]);
-  }
-}
-
-// Pointwise forward over n cells: with vec (every array 16-byte aligned and n
-// a multiple of 4) four cells a thread through 16-byte accesses, which keeps
-// enough bytes in flight per SM; else one cell at a time.  Grid-stride.
-template <typename T, int OP>
-__global__ void g_forward_pw(GNode nd, const T* A, const T* B, const T* C, T* out, long long n,
-                             int vec) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (vec) {
-    for (; t < n / 4; t += stride) {
-      const long long i = 4 * t;
-      T a[4] = {0, 0, 0, 0}, b[4] = {0, 0, 0, 0}, cv[4] = {0, 0, 0, 0}, r[4];
-      if (A) ld4(A, i, a);
-      if (B) ld4(B, i, b);
-      if (nd.pop) ld4(C, i, cv);
+// The value of a node (every op but G_INPUT and G_PMEAN) at the thread's cells.
+template <typename T, int W>
+__device__ __forceinline__ void node_value(int op, const GNode& nd, const T* A, const T* B,
+                                           const T* mesh, const GCell& c, const Geo& g,
+                                           T (&r)[W]) {
+  if (pointwise_op(op)) {
+    T a[W] = {}, b[W] = {};
+    if (A) ldw<T, W>(A, c.idx, a);
+    if (B) ldw<T, W>(B, c.idx, b);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) r[k] = finish(nd, pw_value(OP, nd, a[k], b[k]), cv[k]);
-      st4(out, i, r);
+    for (int l = 0; l < W; ++l) r[l] = pw_value(op, nd, a[l], b[l]);
+    return;
+  }
+  switch (op) {
+    case G_STENCIL: stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, r); break;
+    case G_STEXP:
+      stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, r);
+#pragma unroll
+      for (int l = 0; l < W; ++l) r[l] = exp(r[l]);
+      break;
+    case G_STBIN: {
+      T b[W];
+      stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, r);
+      ldw<T, W>(B, c.idx, b);
+#pragma unroll
+      for (int l = 0; l < W; ++l) r[l] = stbin_val(nd, r[l], b[l]);
+      break;
     }
-  } else {
-    for (; t < n; t += stride) {
-      const T a = A ? A[t] : (T)0, b = B ? B[t] : (T)0, cv = nd.pop ? C[t] : (T)0;
-      out[t] = finish(nd, pw_value(OP, nd, a, b), cv);
+    case G_STMUL: stencil_mul<W>(A, B, (T)0, c, nd.axis, nd.sk, ih1<T>(nd), g, r); break;
+    case G_ST2: {   // one after the other: one tap array live
+      T s2[W];
+      stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, r);
+      stencil<W>(B, c, nd.axis2, nd.sk2, ih2<T>(nd), g, s2);
+#pragma unroll
+      for (int l = 0; l < W; ++l) r[l] = nd.iop == G_ADD ? r[l] + s2[l] : r[l] - s2[l];
+      break;
+    }
+    case G_NB3: {
+      T m[W], z[W], p[W];
+      tap<W>(A, c, nd.axis, nd.sk, g, m);
+      ldw<T, W>(A, c.idx, z);
+      tap<W>(A, c, nd.axis, -nd.sk, g, p);
+#pragma unroll
+      for (int l = 0; l < W; ++l) {
+        const T in = m[l] >= z[l] ? m[l] : z[l];
+        r[l] = nd.iop == G_ADD ? (m[l] + z[l]) + p[l] : in >= p[l] ? in : p[l];
+      }
+      break;
+    }
+    case G_SHIFT: tap<W>(A, c, nd.axis, nd.sk, g, r); break;
+    case G_QUENCH: {   // out = T min(fac, qlim)
+      const T iq = (T)1 / kc<T>(nd.c0, nd.f0), qlim = kc<T>(nd.c1, nd.f1);
+      const T eps = kc<T>(nd.c2, nd.f2);
+      T ta[2][5][W];   // T at offsets -2 .. 2 along each axis slot
+      taps<2, W>(A, c, nd.axis, g, ta[0]);
+      if (nd.sk >= 0) taps<2, W>(A, c, nd.sk, g, ta[1]);
+#pragma unroll
+      for (int l = 0; l < W; ++l) {
+        const T fac = quench_fac<T>(
+            [&](int t, int, int s) {
+              return q_val(ta[t][s + 1][l], ta[t][s + 2][l], ta[t][s + 3][l], iq, eps, (T*)nullptr);
+            },
+            nd.axis, nd.sk, (T*)nullptr);
+        r[l] = ta[0][2][l] * (fac > qlim ? qlim : fac);
+      }
+      break;
+    }
+    default: {   // G_ZFIELD
+      const T z = mesh[(long long)nd.sk * g.nz + c.k];
+#pragma unroll
+      for (int l = 0; l < W; ++l) r[l] = z;
     }
   }
 }
-
-// Every node but the pointwise ones, G_QUENCH (g_quench_f) and G_PMEAN; one
-// instance per op.
-template <typename T, int OP>
-__global__ void g_forward(GNode nd, const T* A, const T* B, const T* C, T* out, const T* mesh,
-                          Geo g) {
-  GCell c0;
-  if (!gcell(c0, g)) return;
-  T r[GZU];
+// ... with its folded sum and epilogue, stored.
+template <typename T, int W>
+__device__ __forceinline__ void node_forward(int op, const GNode& nd, const T* A, const T* B,
+                                             const T* C, T* out, const T* mesh, const GCell& c,
+                                             const Geo& g) {
+  T r[W], cv[W] = {};
+  node_value<T, W>(op, nd, A, B, mesh, c, g, r);
+  if (nd.pop) ldw<T, W>(C, c.idx, cv);
 #pragma unroll
-  for (int u = 0; u < GZU; ++u) {
-    const GCell c = gcell_at(c0, u, g);
-    if (c.k < g.nz)
-      r[u] = finish(nd, fwd_value(OP, nd, A, B, mesh, c, g), nd.pop ? C[c.idx] : (T)0);
-  }
-#pragma unroll
-  for (int u = 0; u < GZU; ++u) {
-    const GCell c = gcell_at(c0, u, g);
-    if (c.k < g.nz) out[c.idx] = r[u];
-  }
-}
-
-// Transpose kernels.  Pointwise rules follow the usual subgradient choices:
-// |x|' = sign(x) with sign(0) = 0; clamp passes the gradient where the bound
-// holds with equality; max(a, b) splits it evenly on ties.
-template <typename T>
-__device__ __forceinline__ void bwd_value(int op, const GNode& nd, const T* A, const T* B,
-                                          const T* out, const T* gout, const GCell& c,
-                                          const Geo& g, T& ca, T& cb) {
-  const long long idx = c.idx;
-  ca = 0;
-  cb = 0;
-  if (op == G_STENCIL) {
-    // Gather form of the transpose: up^T = dn, dn^T = up, ddup^T = -dddn,
-    // dddn^T = -ddup (periodic summation by parts).
-    int kind = nd.sk;
-    T v = stencil_at(gout, c, nd.axis, st_transpose(kind), kc<T>(nd.c0, nd.f0), g);
-    ca = st_negates(kind) ? -v : v;
-  } else if (op == G_STBIN) {
-    // y = st(a) (op) b: the stencil's transpose of the cotangent of st(a),
-    // which is g (add), -+g (sub) or g b (mul) at each tap.
-    const int tk = st_transpose(nd.sk);
-    const T sg = st_negates(nd.sk) ? (T)-1 : (T)1;
-    const T gg = gout[idx];
-    if (nd.iop == G_MUL) {
-      ca = sg * stencil_fn<T>([&](long long j) { return gout[j] * B[j]; }, c, nd.axis, tk,
-                              kc<T>(nd.c0, nd.f0), g);
-      cb = gg * stencil_at(A, c, nd.axis, nd.sk, kc<T>(nd.c0, nd.f0), g);
-    } else {
-      const T v = sg * stencil_at(gout, c, nd.axis, tk, kc<T>(nd.c0, nd.f0), g);
-      const bool neg_st = nd.iop == G_SUB && nd.side;    // b - st
-      const bool neg_b = nd.iop == G_SUB && !nd.side;    // st - b
-      ca = neg_st ? -v : v;
-      cb = neg_b ? -gg : gg;
-    }
-  } else if (op == G_STMUL) {
-    // y = st(a b): the transposed stencil of g, times the other factor.
-    T v = stencil_at(gout, c, nd.axis, st_transpose(nd.sk), kc<T>(nd.c0, nd.f0), g);
-    if (st_negates(nd.sk)) v = -v;
-    ca = v * B[idx];
-    cb = v * A[idx];
-  } else if (op == G_STEXP) {
-    // y = ps exp(st(a)) + pt: the stencil's transpose of g (y - pt), the
-    // epilogue's factor included (it is in y).
-    const T pt = kc<T>(nd.pt, nd.fpt);
-    T v = stencil_fn<T>([&](long long j) { return gout[j] * (out[j] - pt); }, c, nd.axis,
-                        st_transpose(nd.sk), kc<T>(nd.c0, nd.f0), g);
-    ca = st_negates(nd.sk) ? -v : v;
-  } else if (op == G_NB3) {
-    // Gather over the three outputs y = x - o, x, x + o (o = sk) that read x
-    // as their a(y + o), a(y), a(y - o); a max passes g by the primitive
-    // nodes' rule (an even split on a tie, the inner pair first).
-    const int ax = nd.axis, o = nd.sk;
-    const T gm = gout[nbr(c, ax, -o, g)], g0 = gout[idx], gp = gout[nbr(c, ax, o, g)];
-    if (nd.iop == G_ADD) {
-      ca = (gm + g0) + gp;
-    } else {
-      const T a0 = A[idx], am = A[nbr(c, ax, -o, g)], am2 = A[nbr(c, ax, -2 * o, g)];
-      const T ap = A[nbr(c, ax, o, g)], ap2 = A[nbr(c, ax, 2 * o, g)];
-      T wm, wz, wi, wp;
-      max_w(a0, am, wm, wz);   // y = x - o: (a0 op am) op am2, x in the inner first slot
-      max_w(a0 >= am ? a0 : am, am2, wi, wp);
-      T acc = gm * (wi * wm);
-      max_w(ap, a0, wm, wz);   // y = x: (ap op a0) op am, x in the inner second slot
-      max_w(ap >= a0 ? ap : a0, am, wi, wp);
-      acc += g0 * (wi * wz);
-      max_w(ap2, ap, wm, wz);  // y = x + o: (ap2 op ap) op a0, x the outer second slot
-      max_w(ap2 >= ap ? ap2 : ap, a0, wi, wp);
-      ca = acc + gp * wp;
-    }
-  } else if (op == G_ST2) {
-    // y = st1(a) +- st2(b): each stencil's transpose of the cotangent.
-    const T v1 = stencil_at(gout, c, nd.axis, st_transpose(nd.sk), kc<T>(nd.c0, nd.f0), g);
-    const T v2 = stencil_at(gout, c, nd.axis2, st_transpose(nd.sk2), kc<T>(nd.h2, nd.fh2), g);
-    ca = st_negates(nd.sk) ? -v1 : v1;
-    cb = (st_negates(nd.sk2) != (nd.iop == G_SUB)) ? -v2 : v2;
-  } else {   // G_SHIFT
-    ca = gout[nbr(c, nd.axis, -nd.sk, g)];
-  }
+  for (int l = 0; l < W; ++l) r[l] = finish(nd, r[l], cv[l]);
+  stw<T, W>(out, c.idx, r);
 }
 
 // A pointwise op's cotangents of a and b from y = its value and gg = y's
@@ -572,550 +565,393 @@ __device__ __forceinline__ void pw_grad(int op, const GNode& nd, T a, T b, T y, 
   }
 }
 
-// Pointwise transpose over n cells (the layout of g_forward_pw): the
-// cotangents, scaled by the folded sum's sign and the epilogue's factor, are
-// written (first contribution) or added into gA, gB, gC; a and b may be the
-// same node (a's contribution first).
-template <typename T, int OP>
-__device__ __forceinline__ void pw_back_cell(const GNode& nd, T a, T b, T y, T gg, T sv, T sc,
-                                             T& ca, T& cb, T& cc) {
-  pw_grad(OP, nd, a, b, y, gg, ca, cb);
-  if ((nd.ep && OP != G_EXP) || nd.pop == 3) {
-    ca *= sv;
-    cb *= sv;
-  }
-  cc = sc * gg;
-}
-
-template <typename T, int OP>
-__global__ void g_backward_pw(GNode nd, const T* A, const T* B, const T* out, const T* gout,
-                              T* gA, T* gB, T* gC, int wA, int wB, int wC, long long n, int vec) {
-  const bool same = gA != nullptr && gA == gB;
+// What a node (operands' values A, B, its own value Y, its cotangent G) passes
+// to one of its operands: role 0 to a, 1 to b, 2 to the folded sum's c, 3 G
+// itself (an identity, or an array that already holds the contribution).
+// Pointwise rules follow the usual subgradient choices: |x|' = sign(x) with
+// sign(0) = 0; clamp passes the gradient where the bound holds with equality;
+// max(a, b) splits it evenly on ties.
+enum { R_A = 0, R_B, R_C, R_COPY };
+template <typename T, int W>
+__device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T* A, const T* B,
+                                     const T* Y, const T* G, const GCell& c, const Geo& g,
+                                     T (&v)[W]) {
+  // The factors of the epilogue and the folded sum: every transpose is linear
+  // in G, and c's cotangent is +-ps G at the cell.
   const T sv = kc<T>(nd.ps, nd.fps) * (nd.pop == 3 ? (T)-1 : (T)1);
-  const T sc = kc<T>(nd.ps, nd.fps) * (nd.pop == 2 ? (T)-1 : (T)1);
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  auto put = [](int w, T v, T old) { return w ? v : old + v; };   // first write, or add
-  if (vec) {
-    for (; t < n / 4; t += stride) {
-      const long long i = 4 * t;
-      T a[4] = {0, 0, 0, 0}, b[4] = {0, 0, 0, 0}, y[4], gg[4], ca[4], cb[4], cc[4];
-      T oa[4] = {0, 0, 0, 0}, ob[4] = {0, 0, 0, 0}, oc[4] = {0, 0, 0, 0};
-      if (A) ld4(A, i, a);
-      if (B) ld4(B, i, b);
-      ld4(out, i, y);
-      ld4(gout, i, gg);
-      if (gA && !wA) ld4((const T*)gA, i, oa);
-      if (gB && !wB && !same) ld4((const T*)gB, i, ob);
-      if (gC && !wC) ld4((const T*)gC, i, oc);
+  if (role >= R_C) {
+    const T sc = role == R_C ? kc<T>(nd.ps, nd.fps) * (nd.pop == 2 ? (T)-1 : (T)1) : (T)1;
+    ldw<T, W>(G, c.idx, v);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        pw_back_cell<T, OP>(nd, a[k], b[k], y[k], gg[k], sv, sc, ca[k], cb[k], cc[k]);
-        if (same) {
-          oa[k] = put(wB, cb[k], put(wA, ca[k], oa[k]));
-        } else {
-          oa[k] = put(wA, ca[k], oa[k]);
-          ob[k] = put(wB, cb[k], ob[k]);
-        }
-        oc[k] = put(wC, cc[k], oc[k]);
-      }
-      if (gA) st4(gA, i, oa);
-      if (gB && !same) st4(gB, i, ob);
-      if (gC) st4(gC, i, oc);
+    for (int l = 0; l < W; ++l) v[l] = sc * v[l];
+    return;
+  }
+  if (pointwise_op(op)) {
+    T a[W] = {}, b[W] = {}, y[W], gg[W];
+    if (A) ldw<T, W>(A, c.idx, a);
+    if (B) ldw<T, W>(B, c.idx, b);
+    ldw<T, W>(Y, c.idx, y);
+    ldw<T, W>(G, c.idx, gg);
+#pragma unroll
+    for (int l = 0; l < W; ++l) {
+      T ca, cb;
+      pw_grad(op, nd, a[l], b[l], y[l], gg[l], ca, cb);
+      v[l] = role == R_A ? ca : cb;
     }
   } else {
-    for (; t < n; t += stride) {
-      T ca, cb, cc;
-      pw_back_cell<T, OP>(nd, A ? A[t] : (T)0, B ? B[t] : (T)0, out[t], gout[t], sv, sc, ca, cb,
-                          cc);
-      if (same) {
-        gA[t] = put(wB, cb, put(wA, ca, wA ? (T)0 : gA[t]));
+    const int tk = st_transpose(nd.sk);
+    bool ng = st_negates(nd.sk);
+    if (op == G_STBIN && nd.iop == G_MUL) {
+      // y = st(a) b
+      if (role == R_A) {
+        stencil_mul<W>(G, B, (T)0, c, nd.axis, tk, ih1<T>(nd), g, v);
       } else {
-        if (gA) gA[t] = put(wA, ca, wA ? (T)0 : gA[t]);
-        if (gB) gB[t] = put(wB, cb, wB ? (T)0 : gB[t]);
+        T gg[W];
+        stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, v);
+        ldw<T, W>(G, c.idx, gg);
+#pragma unroll
+        for (int l = 0; l < W; ++l) v[l] = gg[l] * v[l];
+        ng = false;
       }
-      if (gC) gC[t] = put(wC, cc, wC ? (T)0 : gC[t]);
+    } else if (op == G_STBIN && role == R_B) {
+      ldw<T, W>(G, c.idx, v);
+      ng = nd.iop == G_SUB && !nd.side;                    // st - b
+    } else if (op == G_STEXP) {
+      // y = ps exp(st(a)) + pt: the stencil's transpose of g (y - pt), the
+      // epilogue's factor included (it is in y).
+      stencil_mul<W>(G, Y, kc<T>(nd.pt, nd.fpt), c, nd.axis, tk, ih1<T>(nd), g, v);
+    } else if (op == G_NB3) {
+      // Gather over the three outputs y = x - o, x, x + o (o = sk) that read x
+      // as their a(y + o), a(y), a(y - o); a max passes g by the primitive
+      // nodes' rule (an even split on a tie, the inner pair first).
+      const int ax = nd.axis, o = nd.sk;
+      T gm[W], g0[W], gp[W];
+      tap<W>(G, c, ax, -o, g, gm);
+      ldw<T, W>(G, c.idx, g0);
+      tap<W>(G, c, ax, o, g, gp);
+      if (nd.iop == G_ADD) {
+#pragma unroll
+        for (int l = 0; l < W; ++l) v[l] = (gm[l] + g0[l]) + gp[l];
+      } else {
+        T a0[W], am[W], am2[W], ap[W], ap2[W];
+        ldw<T, W>(A, c.idx, a0);
+        tap<W>(A, c, ax, -o, g, am);
+        tap<W>(A, c, ax, -2 * o, g, am2);
+        tap<W>(A, c, ax, o, g, ap);
+        tap<W>(A, c, ax, 2 * o, g, ap2);
+#pragma unroll
+        for (int l = 0; l < W; ++l) {
+          T wm, wz, wi, wp;
+          max_w(a0[l], am[l], wm, wz);   // y = x - o: (a0 op am) op am2, x in the inner first slot
+          max_w(a0[l] >= am[l] ? a0[l] : am[l], am2[l], wi, wp);
+          T acc = gm[l] * (wi * wm);
+          max_w(ap[l], a0[l], wm, wz);   // y = x: (ap op a0) op am, x in the inner second slot
+          max_w(ap[l] >= a0[l] ? ap[l] : a0[l], am[l], wi, wp);
+          acc += g0[l] * (wi * wz);
+          max_w(ap2[l], ap[l], wm, wz);  // y = x + o: (ap2 op ap) op a0, x the outer second slot
+          max_w(ap2[l] >= ap[l] ? ap2[l] : ap[l], a0[l], wi, wp);
+          v[l] = acc + gp[l] * wp;
+        }
+      }
+      ng = false;
+    } else if (op == G_SHIFT) {
+      tap<W>(G, c, nd.axis, -nd.sk, g, v);
+      ng = false;
+    } else if (op == G_ST2 && role == R_B) {
+      // y = st1(a) +- st2(b)
+      stencil<W>(G, c, nd.axis2, st_transpose(nd.sk2), ih2<T>(nd), g, v);
+      ng = st_negates(nd.sk2) != (nd.iop == G_SUB);
+    } else {
+      // The transposed stencil of G: STENCIL, ST2 and STBIN (a sum) to a; STMUL,
+      // y = st(a b), times the other factor.
+      stencil<W>(G, c, nd.axis, tk, ih1<T>(nd), g, v);
+      if (op == G_STBIN && nd.iop == G_SUB && nd.side) ng = !ng;   // b - st
+      if (op == G_STMUL) {
+        T f[W];
+        ldw<T, W>(role == R_A ? B : A, c.idx, f);
+#pragma unroll
+        for (int l = 0; l < W; ++l) v[l] = (ng ? -v[l] : v[l]) * f[l];
+        ng = false;
+      }
     }
+    if (ng) {
+#pragma unroll
+      for (int l = 0; l < W; ++l) v[l] = -v[l];
+    }
+  }
+  // exp's transposes take the epilogue's factor from their own value.
+  if ((nd.ep && op != G_EXP && op != G_STEXP) || nd.pop == 3) {
+#pragma unroll
+    for (int l = 0; l < W; ++l) v[l] *= sv;
   }
 }
 
-// The first contribution a gradient receives in the reverse sweep writes it
-// (wA, wB); later ones accumulate.  a and b may be the same node: a's
-// contribution is applied first, as two sequential updates would.
+// ---------------------------------------------------------------------------
+// The sweeps' kernels.  A launch runs a batch of nodes that do not depend on
+// one another, their blocks interleaved along the launch's z extent (tasks of
+// one batch share operands); block-uniform switches pick the op.  A node alone
+// is a few microseconds of work (8 MB at 128^3), much of it the launch, its ramp
+// and its tail: one launch a node took 9.5 ms for an adjoint step at 128^3 and
+// 3.4 ms at 64^3 (on four streams), batches of 24 take 7.3 and 1.45 ms, batches
+// of 6 7.5 and 1.5.  The reverse gathers: the thread sums what every consumer
+// passes to the node's cells and stores once, where a sweep by consumer reads
+// and rewrites the gradient for each of them.
+// ---------------------------------------------------------------------------
+// x / n as the high word of x times recip32(n), exact for x < 65536, n <= 64.
+inline unsigned recip32(int n) { return n == 1 ? 0u : 0xffffffffu / (unsigned)n + 1u; }
+template <typename T>
+struct FwdTask {
+  GNode nd;
+  const T *A, *B, *C;
+  T* out;
+};
+template <typename T>
+struct FwdBatch {
+  static constexpr int MAX = 24;
+  int n;         // tasks
+  unsigned rn;   // recip32(n)
+  FwdTask<T> t[MAX];
+};
+template <typename T>
+struct RevTerm {
+  GNode nd;
+  int role;
+  const T *A, *B, *Y, *G;
+};
+// What becomes of dst's old value: replaced, the start of the sum (a sum in
+// parts), or added to the sum (the caller's input cotangents).
+enum { ADD_NO = 0, ADD_FIRST, ADD_LAST };
+template <typename T>
+struct RevTask {
+  T* dst;
+  int first, n, add;   // its terms
+};
+template <typename T>
+struct RevBatch {
+  static constexpr int MAX = 32;
+  int n, nterm;
+  unsigned rn;
+  RevTask<T> t[MAX];
+  RevTerm<T> c[MAX];
+};
+template <typename T>
+struct QuenchBatch {
+  static constexpr int MAX = 3;
+  int n;
+  unsigned rn;
+  GNode nd[MAX];
+  const T* A[MAX];
+  T* G[MAX];        // the node's cotangent, replaced by its operand's contribution
+  T* scr[MAX];      // 15 arrays each: S (7), Q (8)
+};
+
+// Both sweeps wait on their loads and on instruction issue (a stencil of four
+// cells is 6 loads, 28 operations and about as many for its indices), so warps
+// count: at 128^3 the FP32 adjoint takes 8.27 ms at 4 blocks an SM (64
+// registers), 7.57 at 5 and 7.34 at 6 (40); two planes a thread 7.54.  FP64 is
+// bound by its own pipe.
+#define STG_GRAPH_LB(T) __launch_bounds__(256, sizeof(T) == 4 ? 6 : 2)
+
+#ifdef __CUDACC__
+// f(integral constant) for the op of a task or term (uniform over the block).
+template <int OP> struct OpC { static constexpr int value = OP; };
+template <class F>
+__device__ __forceinline__ void for_op(int op, F f) {
+  switch (op) {
+#define STG_OP(X) case X: f(OpC<X>()); break;
+    STG_OP(G_STENCIL) STG_OP(G_STBIN) STG_OP(G_STMUL) STG_OP(G_ST2) STG_OP(G_STEXP) STG_OP(G_NB3)
+    STG_OP(G_SHIFT) STG_OP(G_ADD) STG_OP(G_SUB) STG_OP(G_MUL) STG_OP(G_DIV) STG_OP(G_MAX)
+    STG_OP(G_EXP) STG_OP(G_LOG) STG_OP(G_LOG1P) STG_OP(G_SQRT) STG_OP(G_ABS) STG_OP(G_AXPB)
+    STG_OP(G_CLAMPMIN) STG_OP(G_CLAMPMAX) STG_OP(G_STEP) STG_OP(G_CONST) STG_OP(G_QUENCH)
+    default: f(OpC<G_ZFIELD>()); break;
+#undef STG_OP
+  }
+}
+
+template <typename T, int W>
+__global__ void STG_GRAPH_LB(T) g_level_fwd(const __grid_constant__ FwdBatch<T> b, const T* mesh,
+                                            Geo g) {
+  const int kb = b.n == 1 ? (int)blockIdx.z : (int)__umulhi(blockIdx.z, b.rn);
+  GCell c;
+  if (!gcell_at<W>(c, kb, g)) return;
+  const FwdTask<T>& t = b.t[(int)blockIdx.z - kb * b.n];
+  for_op(t.nd.op, [&](auto op) {
+    node_forward<T, W>(decltype(op)::value, t.nd, t.A, t.B, t.C, t.out, mesh, c, g);
+  });
+}
+
+template <typename T, int W>
+__global__ void STG_GRAPH_LB(T) g_level_rev(const __grid_constant__ RevBatch<T> b, Geo g) {
+  const int kb = b.n == 1 ? (int)blockIdx.z : (int)__umulhi(blockIdx.z, b.rn);
+  GCell c;
+  if (!gcell_at<W>(c, kb, g)) return;
+  const RevTask<T>& t = b.t[(int)blockIdx.z - kb * b.n];
+  T acc[W];
+  if (t.add == ADD_FIRST) ldw<T, W>((const T*)t.dst, c.idx, acc);
+  for (int q = 0; q < t.n; ++q) {
+    const RevTerm<T>& r = b.c[t.first + q];
+    T v[W];
+    for_op(r.nd.op, [&](auto op) {
+      pull<T, W>(decltype(op)::value, r.role, r.nd, r.A, r.B, r.Y, r.G, c, g, v);
+    });
+#pragma unroll
+    for (int l = 0; l < W; ++l) acc[l] = q == 0 && t.add != ADD_FIRST ? v[l] : acc[l] + v[l];
+  }
+  if (t.add == ADD_LAST) {
+    T o[W];
+    ldw<T, W>((const T*)t.dst, c.idx, o);
+#pragma unroll
+    for (int l = 0; l < W; ++l) acc[l] = o[l] + acc[l];
+  }
+  stw<T, W>(t.dst, c.idx, acc);
+}
+
+// The quench's transpose: PASS 0 q and its derivatives, 1 the cotangents the q
+// receive, 2 the operand's contribution over the node's own cotangent.
+template <typename T, int W, int PASS>
+__global__ void __launch_bounds__(256) g_level_quench(const __grid_constant__ QuenchBatch<T> b,
+                                                      Geo g) {
+  const int kb = b.n == 1 ? (int)blockIdx.z : (int)__umulhi(blockIdx.z, b.rn);
+  const int ti = (int)blockIdx.z - kb * b.n;
+  GCell c;
+  if (!gcell_at<W>(c, kb, g)) return;
+  const GNode& nd = b.nd[ti];
+  T* S = b.scr[ti];
+  T* Q = S + 7 * g.n;
+  if (PASS == 0) quench_q<T, W>(nd, b.A[ti], Q, c, g);
+  if (PASS == 1) quench_b1<T, W>(nd, b.A[ti], Q, b.G[ti], S, c, g);
+  if (PASS == 2) {
+    T acc[W];
+    quench_b3<T, W>(nd, Q, S, c, g, acc);
+    stw<T, W>(b.G[ti], c.idx, acc);
+  }
+}
+#endif  // __CUDACC__
+
+// ---------------------------------------------------------------------------
+// One node per launch (op a template constant), the reverse by consumer: the
+// form the host build runs against the graph of one node per primitive.
+// ---------------------------------------------------------------------------
+template <typename T, int OP>
+__global__ void g_forward(GNode nd, const T* A, const T* B, const T* C, T* out, const T* mesh,
+                          Geo g) {
+  GCell c;
+  if (gcell<1>(c, g)) node_forward<T, 1>(OP, nd, A, B, C, out, mesh, c, g);
+}
+template <typename T, int OP>
+__global__ void g_forward4(GNode nd, const T* A, const T* B, const T* C, T* out, const T* mesh,
+                           Geo g) {
+  GCell c;
+  if (gcell<4>(c, g)) node_forward<T, 4>(OP, nd, A, B, C, out, mesh, c, g);
+}
+// A flat launch over n cells, four at a time with vec.
+template <typename T, int OP>
+__global__ void g_forward_pw(GNode nd, const T* A, const T* B, const T* C, T* out, long long n,
+                             int vec) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  const Geo g{};
+  GCell c{};
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < (vec ? n / 4 : n);
+       t += stride) {
+    c.idx = vec ? 4 * t : t;
+    if (vec) node_forward<T, 4>(OP, nd, A, B, C, out, nullptr, c, g);
+    else node_forward<T, 1>(OP, nd, A, B, C, out, nullptr, c, g);
+  }
+}
+// The operands' contributions, a's first; the first a gradient receives
+// writes it (wA, wB, wC), later ones add.
+template <typename T, int W>
+__device__ __forceinline__ void push_cell(int op, const GNode& nd, const T* A, const T* B,
+                                          const T* out, const T* gout, T* gA, T* gB, T* gC, int wA,
+                                          int wB, int wC, const GCell& c, const Geo& g) {
+  T* dst[3] = {gA, gB, gC};
+  const int w[3] = {wA, wB, wC};
+  for (int r = 0; r < 3; ++r) {
+    if (!dst[r]) continue;
+    T v[W], o[W];
+    pull<T, W>(op, r, nd, A, B, out, gout, c, g, v);
+    if (!w[r]) {
+      ldw<T, W>((const T*)dst[r], c.idx, o);
+      for (int l = 0; l < W; ++l) v[l] = o[l] + v[l];
+    }
+    stw<T, W>(dst[r], c.idx, v);
+  }
+}
 template <typename T, int OP>
 __global__ void g_backward(GNode nd, const T* A, const T* B, const T* out, const T* gout,
                            T* gA, T* gB, T* gC, int wA, int wB, int wC, Geo g) {
-  GCell c0;
-  if (!gcell(c0, g)) return;
-  const bool same = gA != nullptr && gA == gB;
-  // The factors of the epilogue and the folded sum: every transpose is linear
-  // in gout, and C's cotangent is +-ps gout at the cell (C is neither a nor b).
-  const T sv = kc<T>(nd.ps, nd.fps) * (nd.pop == 3 ? (T)-1 : (T)1);
-  const T sc = kc<T>(nd.ps, nd.fps) * (nd.pop == 2 ? (T)-1 : (T)1);
-  T ca[GZU], cb[GZU], oa[GZU], ob[GZU];
-#pragma unroll
-  for (int u = 0; u < GZU; ++u) {
-    const GCell c = gcell_at(c0, u, g);
-    if (c.k < g.nz) {
-      bwd_value(OP, nd, A, B, out, gout, c, g, ca[u], cb[u]);
-      // exp's transposes take the epilogue's factor from their own value.
-      if ((nd.ep && OP != G_EXP && OP != G_STEXP) || nd.pop == 3) {
-        ca[u] *= sv;
-        cb[u] *= sv;
-      }
-      oa[u] = (gA && !wA) ? gA[c.idx] : (T)0;
-      ob[u] = (gB && !wB && !same) ? gB[c.idx] : (T)0;
-      if (gC) {
-        const T v = sc * gout[c.idx];
-        gC[c.idx] = wC ? v : gC[c.idx] + v;
-      }
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < GZU; ++u) {
-    const GCell c = gcell_at(c0, u, g);
-    if (c.k < g.nz) {
-      if (same) {
-        T v = wA ? ca[u] : oa[u] + ca[u];
-        gA[c.idx] = wB ? cb[u] : v + cb[u];
-      } else {
-        if (gA) gA[c.idx] = wA ? ca[u] : oa[u] + ca[u];
-        if (gB) gB[c.idx] = wB ? cb[u] : ob[u] + cb[u];
-      }
-    }
-  }
+  GCell c;
+  if (gcell<1>(c, g)) push_cell<T, 1>(OP, nd, A, B, out, gout, gA, gB, gC, wA, wB, wC, c, g);
 }
-
-// ---------------------------------------------------------------------------
-// The same stencil-type kernels with four consecutive x-cells a thread (nx a
-// multiple of 4, every array 16-byte aligned): each tap is one 16-byte load,
-// the x taps come from the aligned 4-cell chunks left of, at and right of the
-// thread's cells, and the per-thread index work is shared by four cells (the
-// one-cell kernels are bound by their instruction issue).  Every lane takes
-// the one-cell arithmetic, so the values are the same bit for bit.  SHIFT and
-// NB3 here take offsets of one cell.
-// ---------------------------------------------------------------------------
-struct GCell4 {
-  int i0, j, k;   // i0: the first of the four x-cells
-  long long idx;  // index of cell i0
-};
-
-__device__ __forceinline__ bool gcell4(GCell4& c, const Geo& g) {
-  c.i0 = 4 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  c.j = blockIdx.y * blockDim.y + threadIdx.y;
-  c.k = blockIdx.z * blockDim.z + threadIdx.z;
-  if (c.i0 >= g.nx || c.j >= g.ny || c.k >= g.nz) return false;
-  c.idx = (long long)c.k * g.sz + (long long)c.j * g.sy + c.i0;
-  return true;
-}
-
-// t[o + K][l]: f at cell (i0 + l, j, k) + o e_axis, o = -K .. K (K <= 3).
-template <int K, typename T>
-__device__ __forceinline__ void tapsx4(const T* f, const GCell4& c, int axis, const Geo& g,
-                                       T t[2 * K + 1][4]) {
-  if (axis == 0) {
-    const long long row = c.idx - c.i0;
-    T L[4], M[4], R[4];
-    ld4(f, row + wrap(c.i0 - 4, g.nx), L);
-    ld4(f, c.idx, M);
-    ld4(f, row + wrap(c.i0 + 4, g.nx), R);
-#pragma unroll
-    for (int o = -K; o <= K; ++o)
-#pragma unroll
-      for (int l = 0; l < 4; ++l) {
-        const int q = 4 + l + o;   // in the 12-cell window i0 - 4 .. i0 + 7
-        t[o + K][l] = q < 4 ? L[q] : q < 8 ? M[q - 4] : R[q - 8];
-      }
-  } else {
-    const long long st = axis == 1 ? g.sy : g.sz;
-    const int pos = axis == 1 ? c.j : c.k, n = axis == 1 ? g.ny : g.nz;
-    const bool inner = pos >= K && pos + K < n;
-#pragma unroll
-    for (int o = -K; o <= K; ++o)
-      ld4(f, c.idx + (inner ? o * st : (long long)(wrap(pos + o, n) - pos) * st), t[o + K]);
-  }
-}
-template <typename T>
-__device__ __forceinline__ void taps7x4(const T* f, const GCell4& c, int axis, const Geo& g,
-                                        T t[7][4]) {
-  tapsx4<3>(f, c, axis, g, t);
-}
-
-// v[l]: f at cell (i0 + l, j, k) + o e_axis, one offset o in -1 .. 1.
-template <typename T>
-__device__ __forceinline__ void tap1x4(const T* f, const GCell4& c, int axis, int o,
-                                       const Geo& g, T (&v)[4]) {
-  if (axis == 0) {
-    T t[3][4];
-    tapsx4<1>(f, c, 0, g, t);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) v[l] = o < 0 ? t[0][l] : o > 0 ? t[2][l] : t[1][l];
-  } else {
-    const long long st = axis == 1 ? g.sy : g.sz;
-    const int pos = axis == 1 ? c.j : c.k, n = axis == 1 ? g.ny : g.nz;
-    ld4(f, c.idx + (long long)(wrap(pos + o, n) - pos) * st, v);
-  }
-}
-
-// Lane l's seven taps as one array.
-template <typename T>
-__device__ __forceinline__ void lane7(const T t[7][4], int l, T u[7]) {
-#pragma unroll
-  for (int o = 0; o < 7; ++o) u[o] = t[o][l];
-}
-// The tap at offset s = +-1 (or +-2 with d2) of lane l.
-template <typename T>
-__device__ __forceinline__ T tap1(const T t[7][4], int s, int l) {
-  return s > 0 ? t[4][l] : t[2][l];
-}
-template <typename T>
-__device__ __forceinline__ T tap2(const T t[7][4], int s, int l) {
-  return s > 0 ? t[5][l] : t[1][l];
-}
-
-// FP32: at most 64 registers (4 blocks per SM): the transposes that gather
-// two or three tap arrays spill about 100 bytes then, yet run faster than at
-// 76-84 registers and 3 blocks (STBIN of a product 38 -> 21 us, STEXP 23 -> 16
-// us at 128^3); the forward kernels taken with four cells stay under 64
-// anyway.  FP64 (twice the registers a value) keeps the compiler's choice.
 template <typename T, int OP>
-__global__ void __launch_bounds__(GBX * GBY * GBZ, sizeof(T) == 4 ? 4 : 1)
-    g_forward4(GNode nd, const T* A, const T* B, const T* C, T* out, const T* mesh, Geo g) {
-  GCell4 c;
-  if (!gcell4(c, g)) return;
-  const T h = kc<T>(nd.c0, nd.f0);
-  T r[4];
-  if (OP == G_ZFIELD) {
-    const T z = mesh[(long long)nd.sk * g.nz + c.k];
-#pragma unroll
-    for (int l = 0; l < 4; ++l) r[l] = z;
-  } else if (OP == G_STMUL) {
-    // The product formed as B's taps arrive: one tap array live.
-    T ta[7][4];
-    taps7x4(A, c, nd.axis, g, ta);
-    {
-      T tb[7][4];
-      taps7x4(B, c, nd.axis, g, tb);
-#pragma unroll
-      for (int o = 0; o < 7; ++o)
-#pragma unroll
-        for (int l = 0; l < 4; ++l) ta[o][l] = ta[o][l] * tb[o][l];
-    }
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      T u[7];
-      lane7(ta, l, u);
-      r[l] = st_comb(nd.sk, h, u);
-    }
-  } else if (OP == G_ST2) {
-    // The two stencils one after the other: one tap array live.
-    T s1[4];
-    {
-      T ta[7][4];
-      taps7x4(A, c, nd.axis, g, ta);
-#pragma unroll
-      for (int l = 0; l < 4; ++l) {
-        T u[7];
-        lane7(ta, l, u);
-        s1[l] = st_comb(nd.sk, h, u);
-      }
-    }
-    T tb[7][4];
-    taps7x4(B, c, nd.axis2, g, tb);
-    const T h2 = kc<T>(nd.h2, nd.fh2);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      T v[7];
-      lane7(tb, l, v);
-      const T s2 = st_comb(nd.sk2, h2, v);
-      r[l] = nd.iop == G_ADD ? s1[l] + s2 : s1[l] - s2;
-    }
-  } else {
-    T t[7][4];
-    taps7x4(A, c, nd.axis, g, t);
-    T b[4] = {0, 0, 0, 0};
-    if (OP == G_STBIN) ld4(B, c.idx, b);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      if (OP == G_SHIFT) {
-        r[l] = tap1(t, nd.sk, l);
-      } else if (OP == G_NB3) {
-        const T m = tap1(t, nd.sk, l), z = t[3][l], p = tap1(t, -nd.sk, l);
-        if (nd.iop == G_ADD) {
-          r[l] = (m + z) + p;
-        } else {
-          const T in = m >= z ? m : z;
-          r[l] = in >= p ? in : p;
-        }
-      } else {
-        T u[7];
-        lane7(t, l, u);
-        const T st = st_comb(nd.sk, h, u);
-        r[l] = OP == G_STEXP ? exp(st) : OP == G_STBIN ? stbin_val(nd, st, b[l]) : st;
-      }
-    }
-  }
-  T cv[4] = {0, 0, 0, 0};
-  if (nd.pop) ld4(C, c.idx, cv);
-#pragma unroll
-  for (int l = 0; l < 4; ++l) r[l] = finish(nd, r[l], cv[l]);
-  st4(out, c.idx, r);
+__global__ void g_backward4(GNode nd, const T* A, const T* B, const T* out, const T* gout, T* gA,
+                            T* gB, T* gC, int wA, int wB, int wC, Geo g) {
+  GCell c;
+  if (gcell<4>(c, g)) push_cell<T, 4>(OP, nd, A, B, out, gout, gA, gB, gC, wA, wB, wC, c, g);
 }
-
 template <typename T, int OP>
-__global__ void __launch_bounds__(GBX * GBY * GBZ, sizeof(T) == 4 ? 4 : 1)
-    g_backward4(GNode nd, const T* A, const T* B, const T* out, const T* gout, T* gA, T* gB,
-                T* gC, int wA, int wB, int wC, Geo g) {
-  GCell4 c;
-  if (!gcell4(c, g)) return;
-  const T h = kc<T>(nd.c0, nd.f0);
-  const int tk = st_transpose(nd.sk);
-  const bool ng = st_negates(nd.sk);
-  T ca[4] = {0, 0, 0, 0}, cb[4] = {0, 0, 0, 0}, gg[4];
-  ld4(gout, c.idx, gg);
-  if (OP == G_ST2) {
-    T t1[7][4], t2[7][4];
-    taps7x4(gout, c, nd.axis, g, t1);
-    taps7x4(gout, c, nd.axis2, g, t2);
-    const T h2 = kc<T>(nd.h2, nd.fh2);
-    const bool n2 = st_negates(nd.sk2) != (nd.iop == G_SUB);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      T u[7], v[7];
-      lane7(t1, l, u);
-      lane7(t2, l, v);
-      const T v1 = st_comb(tk, h, u), v2 = st_comb(st_transpose(nd.sk2), h2, v);
-      ca[l] = ng ? -v1 : v1;
-      cb[l] = n2 ? -v2 : v2;
-    }
-  } else if (OP == G_NB3) {
-    T tg[7][4], ta[7][4];
-    taps7x4(gout, c, nd.axis, g, tg);
-    if (nd.iop != G_ADD) taps7x4(A, c, nd.axis, g, ta);
-    const int o = nd.sk;
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const T gm = tap1(tg, -o, l), g0 = tg[3][l], gp = tap1(tg, o, l);
-      if (nd.iop == G_ADD) {
-        ca[l] = (gm + g0) + gp;
-      } else {
-        const T a0 = ta[3][l], am = tap1(ta, -o, l), am2 = tap2(ta, -o, l);
-        const T ap = tap1(ta, o, l), ap2 = tap2(ta, o, l);
-        T wm, wz, wi, wp;
-        max_w(a0, am, wm, wz);
-        max_w(a0 >= am ? a0 : am, am2, wi, wp);
-        T acc = gm * (wi * wm);
-        max_w(ap, a0, wm, wz);
-        max_w(ap >= a0 ? ap : a0, am, wi, wp);
-        acc += g0 * (wi * wz);
-        max_w(ap2, ap, wm, wz);
-        max_w(ap2 >= ap ? ap2 : ap, a0, wi, wp);
-        ca[l] = acc + gp * wp;
-      }
-    }
-  } else if (OP == G_SHIFT) {
-    T tg[7][4];
-    taps7x4(gout, c, nd.axis, g, tg);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) ca[l] = tap1(tg, -nd.sk, l);
-  } else {
-    // STENCIL, STBIN, STMUL, STEXP: the transposed stencil of gout, or of
-    // gout times B (STBIN with a product) or times y - pt (STEXP).
-    // One tap array live at a time (the product formed as its factor
-    // arrives), then, for STBIN of a product, the stencil of A for cb.
-    const bool prod = (OP == G_STBIN && nd.iop == G_MUL) || OP == G_STEXP;
-    {
-      T tg[7][4];
-      taps7x4(gout, c, nd.axis, g, tg);
-      if (prod) {
-        T tb[7][4];
-        taps7x4(OP == G_STEXP ? out : B, c, nd.axis, g, tb);
-        const T pt = kc<T>(nd.pt, nd.fpt);
-#pragma unroll
-        for (int q = 0; q < 7; ++q)
-#pragma unroll
-          for (int l = 0; l < 4; ++l)
-            tg[q][l] = OP == G_STEXP ? tg[q][l] * (tb[q][l] - pt) : tg[q][l] * tb[q][l];
-      }
-      T a[4] = {0, 0, 0, 0}, b[4] = {0, 0, 0, 0};
-      if (OP == G_STMUL) {
-        ld4(A, c.idx, a);
-        ld4(B, c.idx, b);
-      }
-#pragma unroll
-      for (int l = 0; l < 4; ++l) {
-        T u[7];
-        lane7(tg, l, u);
-        T v = st_comb(tk, h, u);
-        if (ng) v = -v;
-        if (OP == G_STBIN) {
-          if (nd.iop == G_MUL) {
-            ca[l] = v;
-          } else {
-            ca[l] = (nd.iop == G_SUB && nd.side) ? -v : v;
-            cb[l] = (nd.iop == G_SUB && !nd.side) ? -gg[l] : gg[l];
-          }
-        } else if (OP == G_STMUL) {
-          ca[l] = v * b[l];
-          cb[l] = v * a[l];
-        } else {
-          ca[l] = v;
-        }
-      }
-    }
-    if (OP == G_STBIN && nd.iop == G_MUL) {
-      T ta[7][4];
-      taps7x4(A, c, nd.axis, g, ta);
-#pragma unroll
-      for (int l = 0; l < 4; ++l) {
-        T w[7];
-        lane7(ta, l, w);
-        cb[l] = gg[l] * st_comb(nd.sk, h, w);
-      }
-    }
+__global__ void g_backward_pw(GNode nd, const T* A, const T* B, const T* out, const T* gout,
+                              T* gA, T* gB, T* gC, int wA, int wB, int wC, long long n, int vec) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  const Geo g{};
+  GCell c{};
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < (vec ? n / 4 : n);
+       t += stride) {
+    c.idx = vec ? 4 * t : t;
+    if (vec) push_cell<T, 4>(OP, nd, A, B, out, gout, gA, gB, gC, wA, wB, wC, c, g);
+    else push_cell<T, 1>(OP, nd, A, B, out, gout, gA, gB, gC, wA, wB, wC, c, g);
   }
-  const bool same = gA != nullptr && gA == gB;
-  const T sv = kc<T>(nd.ps, nd.fps) * (nd.pop == 3 ? (T)-1 : (T)1);
-  const T sc = kc<T>(nd.ps, nd.fps) * (nd.pop == 2 ? (T)-1 : (T)1);
-  if ((nd.ep && OP != G_STEXP) || nd.pop == 3) {
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      ca[l] *= sv;
-      cb[l] *= sv;
-    }
-  }
-  auto put = [](int w, T v, T old) { return w ? v : old + v; };   // first write, or add
-  T oa[4] = {0, 0, 0, 0}, ob[4] = {0, 0, 0, 0}, oc[4] = {0, 0, 0, 0};
-  if (gA && !wA) ld4((const T*)gA, c.idx, oa);
-  if (gB && !wB && !same) ld4((const T*)gB, c.idx, ob);
-  if (gC && !wC) ld4((const T*)gC, c.idx, oc);
-#pragma unroll
-  for (int l = 0; l < 4; ++l) {
-    if (same) {
-      oa[l] = put(wB, cb[l], put(wA, ca[l], oa[l]));
-    } else {
-      oa[l] = put(wA, ca[l], oa[l]);
-      ob[l] = put(wB, cb[l], ob[l]);
-    }
-    oc[l] = put(wC, sc * gg[l], oc[l]);
-  }
-  if (gA) st4(gA, c.idx, oa);
-  if (gB && !same) st4(gB, c.idx, ob);
-  if (gC) st4(gC, c.idx, oc);
 }
-
-// The quench's kernels with four x-cells a thread (the same per-lane
-// arithmetic as g_quench_f, g_quench_q, g_quench_b1 and g_quench_b3).
+template <typename T>
+__global__ void g_quench_f(GNode nd, const T* A, T* out, Geo g) {
+  GCell c;
+  if (gcell<1>(c, g)) node_forward<T, 1>(G_QUENCH, nd, A, nullptr, nullptr, out, nullptr, c, g);
+}
 template <typename T>
 __global__ void g_quench_f4(GNode nd, const T* A, T* out, Geo g) {
-  GCell4 c;
-  if (!gcell4(c, g)) return;
-  const T iq = (T)1 / kc<T>(nd.c0, nd.f0), qlim = kc<T>(nd.c1, nd.f1);
-  const T eps = kc<T>(nd.c2, nd.f2);
-  T ta[2][5][4];   // T at offsets -2 .. 2 along each axis slot
-  tapsx4<2>(A, c, nd.axis, g, ta[0]);
-  if (nd.sk >= 0) tapsx4<2>(A, c, nd.sk, g, ta[1]);
-  T r[4];
-#pragma unroll
-  for (int l = 0; l < 4; ++l) {
-    const T fac = quench_fac<T>(
-        [&](int t, int, int s) {
-          return q_val(ta[t][s + 1][l], ta[t][s + 2][l], ta[t][s + 3][l], iq, eps, (T*)nullptr);
-        },
-        nd.axis, nd.sk, (T*)nullptr);
-    r[l] = ta[0][2][l] * (fac > qlim ? qlim : fac);
-  }
-  st4(out, c.idx, r);
+  GCell c;
+  if (gcell<4>(c, g)) node_forward<T, 4>(G_QUENCH, nd, A, nullptr, nullptr, out, nullptr, c, g);
 }
-
+template <typename T>
+__global__ void g_quench_q(GNode nd, const T* A, T* Q, Geo g) {
+  GCell c;
+  if (gcell<1>(c, g)) quench_q<T, 1>(nd, A, Q, c, g);
+}
 template <typename T>
 __global__ void g_quench_q4(GNode nd, const T* A, T* Q, Geo g) {
-  GCell4 c;
-  if (!gcell4(c, g)) return;
-  const T iq = (T)1 / kc<T>(nd.c0, nd.f0), eps = kc<T>(nd.c2, nd.f2);
-  for (int t = 0; t < 2; ++t) {
-    const int ax = t == 0 ? nd.axis : nd.sk;
-    if (ax < 0) continue;
-    T ta[3][4];
-    tapsx4<1>(A, c, ax, g, ta);
-    T q[4], d0[4], d1[4], d2[4];
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      T dq[3];
-      q[l] = q_val(ta[0][l], ta[1][l], ta[2][l], iq, eps, dq);
-      d0[l] = dq[0];
-      d1[l] = dq[1];
-      d2[l] = dq[2];
-    }
-    st4(Q + (long long)(4 * t) * g.n, c.idx, q);
-    st4(Q + (long long)(4 * t + 1) * g.n, c.idx, d0);
-    st4(Q + (long long)(4 * t + 2) * g.n, c.idx, d1);
-    st4(Q + (long long)(4 * t + 3) * g.n, c.idx, d2);
-  }
+  GCell c;
+  if (gcell<4>(c, g)) quench_q<T, 4>(nd, A, Q, c, g);
 }
-
+template <typename T>
+__global__ void g_quench_b1(GNode nd, const T* A, const T* Q, const T* gout, T* S, Geo g) {
+  GCell c;
+  if (gcell<1>(c, g)) quench_b1<T, 1>(nd, A, Q, gout, S, c, g);
+}
 template <typename T>
 __global__ void g_quench_b1_4(GNode nd, const T* A, const T* Q, const T* gout, T* S, Geo g) {
-  GCell4 c;
-  if (!gcell4(c, g)) return;
-  const T qlim = kc<T>(nd.c1, nd.f1);
-  T tq[2][3][4];   // q at offsets -1 .. 1 along each axis slot
-  tapsx4<1>(Q, c, nd.axis, g, tq[0]);
-  if (nd.sk >= 0) tapsx4<1>(Q + 4 * g.n, c, nd.sk, g, tq[1]);
-  T a[4], gg[4];
-  ld4(A, c.idx, a);
-  ld4(gout, c.idx, gg);
-  T s0[4], sw[6][4];
-#pragma unroll
-  for (int l = 0; l < 4; ++l) {
-    T wq[6];
-    const T fac = quench_fac<T>([&](int t, int, int s) { return tq[t][s + 1][l]; }, nd.axis,
-                                nd.sk, wq);
-    const T C = fac > qlim ? qlim : fac;
-    const T dC = fac <= qlim ? (T)1 : (T)0;
-    const T base = gg[l] * a[l] * dC;
-    s0[l] = gg[l] * C;
-#pragma unroll
-    for (int j = 0; j < 6; ++j) sw[j][l] = base * wq[j];
-  }
-  st4(S, c.idx, s0);
-#pragma unroll
-  for (int j = 0; j < 6; ++j) st4(S + (long long)(1 + j) * g.n, c.idx, sw[j]);
+  GCell c;
+  if (gcell<4>(c, g)) quench_b1<T, 4>(nd, A, Q, gout, S, c, g);
 }
-
+template <typename T, int W>
+__device__ __forceinline__ void quench_put(const GNode& nd, const T* Q, const T* S, T* gA, int wA,
+                                           const GCell& c, const Geo& g) {
+  T acc[W], o[W];
+  quench_b3<T, W>(nd, Q, S, c, g, acc);
+  if (!wA) {
+    ldw<T, W>((const T*)gA, c.idx, o);
+    for (int l = 0; l < W; ++l) acc[l] = o[l] + acc[l];
+  }
+  stw<T, W>(gA, c.idx, acc);
+}
+template <typename T>
+__global__ void g_quench_b3(GNode nd, const T* Q, const T* S, T* gA, int wA, Geo g) {
+  GCell c;
+  if (gcell<1>(c, g)) quench_put<T, 1>(nd, Q, S, gA, wA, c, g);
+}
 template <typename T>
 __global__ void g_quench_b3_4(GNode nd, const T* Q, const T* S, T* gA, int wA, Geo g) {
-  GCell4 c;
-  if (!gcell4(c, g)) return;
-  T acc[4];
-  ld4(S, c.idx, acc);
-  for (int t = 0; t < 2; ++t) {
-    const int ax = t == 0 ? nd.axis : nd.sk;
-    if (ax < 0) continue;
-    T ts[3][5][4];   // S of q position p = -1 .. 1 at offsets -2 .. 2
-#pragma unroll
-    for (int p = 0; p < 3; ++p) tapsx4<2>(S + (long long)(1 + 3 * t + p) * g.n, c, ax, g, ts[p]);
-    T td[3][4];   // d q(z) / d T at its tap 1 - r, z at offsets r = -1 .. 1
-#pragma unroll
-    for (int r = -1; r <= 1; ++r)
-      tap1x4(Q + (long long)(4 * t + 2 - r) * g.n, c, ax, r, g, td[r + 1]);
-#pragma unroll
-    for (int r = -1; r <= 1; ++r)
-#pragma unroll
-      for (int l = 0; l < 4; ++l) {
-        T qbar = 0;
-#pragma unroll
-        for (int p = -1; p <= 1; ++p) qbar += ts[p + 1][r - p + 2][l];
-        acc[l] += qbar * td[r + 1][l];
-      }
-  }
-  if (!wA) {
-    T o[4];
-    ld4((const T*)gA, c.idx, o);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) acc[l] = o[l] + acc[l];
-  }
-  st4(gA, c.idx, acc);
+  GCell c;
+  if (gcell<4>(c, g)) quench_put<T, 4>(nd, Q, S, gA, wA, c, g);
 }
 
 // Horizontal-plane mean (G_PMEAN): one block per z sums its plane in a fixed
@@ -1139,40 +975,10 @@ __global__ void g_plane_sum(const T* A, T* psum, Geo g) {
 
 template <typename T>
 __global__ void g_plane_bcast(const T* psum, T* out, int add, Geo g) {
-  GCell c0;
-  if (!gcell(c0, g)) return;
-  for (int u = 0; u < GZU; ++u) {
-    const GCell c = gcell_at(c0, u, g);
-    if (c.k >= g.nz) break;
-    const T v = psum[c.k] / (T)((double)g.nx * g.ny);
-    out[c.idx] = add ? out[c.idx] + v : v;
-  }
-}
-
-// dst[k] += src[k] for up to eight arrays in one launch (blockIdx.y = k).
-template <typename T>
-struct Add8 {
-  T* dst[8];
-  const T* src[8];
-};
-template <typename T>
-__global__ void g_add_into8(Add8<T> p, long long n, int vec) {
-  T* dst = p.dst[blockIdx.y];
-  const T* src = p.src[blockIdx.y];
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (vec) {   // four elements a thread through 16-byte accesses
-    for (; t < n / 4; t += stride) {
-      T a[4], b[4];
-      ld4((const T*)dst, 4 * t, a);
-      ld4(src, 4 * t, b);
-#pragma unroll
-      for (int l = 0; l < 4; ++l) a[l] += b[l];
-      st4(dst, 4 * t, a);
-    }
-  } else {
-    for (; t < n; t += stride) dst[t] += src[t];
-  }
+  GCell c;
+  if (!gcell<1>(c, g)) return;
+  const T v = psum[c.k] / (T)((double)g.nx * g.ny);
+  out[c.idx] = add ? out[c.idx] + v : v;
 }
 
 }  // namespace stg
