@@ -63,6 +63,7 @@ struct KPar {
   // plane's B_x, B_y fluctuations (one plane each).
   float oinv_tpot;
   const float *bpx, *bpy;
+  int nsm;              // SMs of the device, for the prefetch lookahead (0: off)
 };
 
 // Fields of the fused path, one contiguous device array each.

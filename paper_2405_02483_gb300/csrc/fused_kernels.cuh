@@ -26,6 +26,7 @@
 #define STG_LB(N, minb) __launch_bounds__(BX * BY * BZ, (N::W == 4 ? STG_MINB4 : (minb)))
 #define STG_LB_HI(N, minb) __launch_bounds__(BX * BY * BZ, (N::W == 4 ? STG_MINB4_HI : (minb)))
 #define STG_LB_4(N, minb) __launch_bounds__(BX * BY * BZ, (N::W == 4 ? 4 : (minb)))
+#define STG_LB_N(N, blocks, minb) __launch_bounds__(BX * BY * BZ, (N::W == 4 ? (blocks) : (minb)))
 
 namespace stg {
 
@@ -58,6 +59,35 @@ struct F4 {
     v[0] = a; v[1] = b; v[2] = c; v[3] = d;
   }
 };
+// On the device sums, products and multiply-adds run as packed pairs (one issue
+// slot for two lanes, the same rounding; fewer spills): 512^3 k_edge 4.27 -> 4.17
+// ms, k_flux 4.13 -> 4.11, k_tau 3.54 -> 3.57.
+#ifdef __CUDA_ARCH__
+#define STG_F4_PACKED(name, fn)                                                    \
+  __device__ __forceinline__ F4 name(const F4& a, const F4& b) {                   \
+    const float2 x = fn(make_float2(a.v[0], a.v[1]), make_float2(b.v[0], b.v[1])), \
+                 y = fn(make_float2(a.v[2], a.v[3]), make_float2(b.v[2], b.v[3])); \
+    return F4(x.x, x.y, y.x, y.y);                                                 \
+  }
+STG_F4_PACKED(operator+, __fadd2_rn)
+STG_F4_PACKED(operator*, __fmul2_rn)
+#undef STG_F4_PACKED
+// s a + b
+__device__ __forceinline__ F4 fma1(float s, const F4& a, const F4& b) {
+  const float2 t = make_float2(s, s);
+  const float2 x = __ffma2_rn(t, make_float2(a.v[0], a.v[1]), make_float2(b.v[0], b.v[1])),
+               y = __ffma2_rn(t, make_float2(a.v[2], a.v[3]), make_float2(b.v[2], b.v[3]));
+  return F4(x.x, x.y, y.x, y.y);
+}
+__device__ __forceinline__ F4 fma1(const F4& s, const F4& a, const F4& b) {
+  const float2 x = __ffma2_rn(make_float2(s.v[0], s.v[1]), make_float2(a.v[0], a.v[1]),
+                              make_float2(b.v[0], b.v[1])),
+               y = __ffma2_rn(make_float2(s.v[2], s.v[3]), make_float2(a.v[2], a.v[3]),
+                              make_float2(b.v[2], b.v[3]));
+  return F4(x.x, x.y, y.x, y.y);
+}
+__device__ __forceinline__ F4 operator-(const F4& a, const F4& b) { return fma1(-1.f, b, a); }
+#else
 #define STG_F4_BIN(op)                                                        \
   __device__ __forceinline__ F4 operator op(const F4& a, const F4& b) {       \
     return F4(a.v[0] op b.v[0], a.v[1] op b.v[1], a.v[2] op b.v[2], a.v[3] op b.v[3]); \
@@ -65,8 +95,13 @@ struct F4 {
 STG_F4_BIN(+)
 STG_F4_BIN(-)
 STG_F4_BIN(*)
-STG_F4_BIN(/)
 #undef STG_F4_BIN
+__device__ __forceinline__ F4 fma1(const F4& s, const F4& a, const F4& b) { return s * a + b; }
+#endif
+__device__ __forceinline__ float fma1(float s, float a, float b) { return s * a + b; }
+__device__ __forceinline__ F4 operator/(const F4& a, const F4& b) {
+  return F4(a.v[0] / b.v[0], a.v[1] / b.v[1], a.v[2] / b.v[2], a.v[3] / b.v[3]);
+}
 __device__ __forceinline__ F4 operator-(const F4& a) { return F4(-a.v[0], -a.v[1], -a.v[2], -a.v[3]); }
 __device__ __forceinline__ F4& operator+=(F4& a, const F4& b) { return a = a + b; }
 __device__ __forceinline__ F4& operator-=(F4& a, const F4& b) { return a = a - b; }
@@ -318,24 +353,24 @@ using Nb4Z = ZCell<Nb4>;
 // eq. (interp) to i+1/2 / i-1/2 and eq. (deriv) to i+1/2 / i-1/2, on a
 // functor v(o) giving the operand at offset o along the stencil axis.
 template <class V> __device__ __forceinline__ auto s_up(V v) -> decltype(v(0)) {
-  return IA_ * (v(0) + v(1)) + IB_ * (v(-1) + v(2)) + IC_ * (v(-2) + v(3));
+  return fma1(IC_, v(-2) + v(3), fma1(IB_, v(-1) + v(2), IA_ * (v(0) + v(1))));
 }
 template <class V> __device__ __forceinline__ auto s_dn(V v) -> decltype(v(0)) {
-  return IA_ * (v(-1) + v(0)) + IB_ * (v(-2) + v(1)) + IC_ * (v(-3) + v(2));
+  return fma1(IC_, v(-3) + v(2), fma1(IB_, v(-2) + v(1), IA_ * (v(-1) + v(0))));
 }
 template <class V> __device__ __forceinline__ auto s_du(V v, float ih) -> decltype(v(0)) {
-  return (DA_ * (v(1) - v(0)) + DB_ * (v(2) - v(-1)) + DC_ * (v(3) - v(-2))) * ih;
+  return fma1(DC_, v(3) - v(-2), fma1(DB_, v(2) - v(-1), DA_ * (v(1) - v(0)))) * ih;
 }
 template <class V> __device__ __forceinline__ auto s_dd(V v, float ih) -> decltype(v(0)) {
-  return (DA_ * (v(0) - v(-1)) + DB_ * (v(1) - v(-2)) + DC_ * (v(2) - v(-3))) * ih;
+  return fma1(DC_, v(2) - v(-3), fma1(DB_, v(1) - v(-2), DA_ * (v(0) - v(-1)))) * ih;
 }
 
 // s_dn and s_dd of the same taps (dn returned, the derivative in d).
 template <class V>
 __device__ __forceinline__ auto s_dn_dd(V v, float ih, decltype(v(0))& d) -> decltype(v(0)) {
   const auto a = v(-3), b = v(-2), c = v(-1), e = v(0), f = v(1), g = v(2);
-  d = (DA_ * (e - c) + DB_ * (f - b) + DC_ * (g - a)) * ih;
-  return IA_ * (c + e) + IB_ * (b + f) + IC_ * (a + g);
+  d = fma1(DC_, g - a, fma1(DB_, f - b, DA_ * (e - c))) * ih;
+  return fma1(IC_, a + g, fma1(IB_, b + f, IA_ * (c + e)));
 }
 
 // Ask for the cell's line of an array the kernel reads later, without a
@@ -345,6 +380,34 @@ __device__ __forceinline__ auto s_dn_dd(V v, float ih, decltype(v(0))& d) -> dec
 template <class N> __device__ __forceinline__ void pf(const N& n, const float* p) {
 #ifdef __CUDA_ARCH__
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p + n.c));
+#endif
+}
+
+// Cell of this thread's place in the thread block that is launched `blocks`
+// later (about the one that follows this one on the SM when blocks is what the
+// GPU holds), for one thread of each 128-byte line; -1 for the others, past the
+// grid, and with blocks 0.  A kernel of few arrays that brings those lines into
+// L2 hides its DRAM latency (512^3: k_vel, with 5 blocks an SM, 933 -> 820 us,
+// 588 from 772 in ideal runs; k_nu_raw 1045 -> 1002); the kernels of 15 and more
+// arrays got slower by it (k_flux 4.2 -> 4.6 ms and more).
+template <class N>
+__device__ __forceinline__ int ahead_cell(const Geo& g, int blocks) {
+#ifdef __CUDA_ARCH__
+  if (!blocks || (N::W * threadIdx.x) % 32) return -1;
+  const unsigned lb = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x + blocks;
+  const unsigned r = lb / gridDim.x, bx = lb - r * gridDim.x, bz = r / gridDim.y,
+                 by = r - bz * gridDim.y;
+  const int i = N::W * (bx * blockDim.x + threadIdx.x), j = by * blockDim.y + threadIdx.y,
+            kz = bz * blockDim.z + threadIdx.z;
+  if (i >= g.nx || j >= g.ny || kz >= g.nz) return -1;
+  return kz * (int)g.sz + j * (int)g.sy + i;
+#else
+  return -1;
+#endif
+}
+__device__ __forceinline__ void pf_at(int c, const float* p) {
+#ifdef __CUDA_ARCH__
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p + c));
 #endif
 }
 
@@ -392,7 +455,7 @@ __global__ void k_lr_ed(const float* __restrict__ rd, const float* __restrict__ 
 // u_d = p_d / rho_face with rho_face = dens(dn_d ls); the face values dn_d ls
 // are also stored (lf, may be null) for the edge densities of the stresses.
 template <class N>
-__global__ void STG_LB(N, STG_MINB) k_vel(
+__global__ void STG_LB_N(N, 5, STG_MINB) k_vel(
     const float* __restrict__ ls, const float* __restrict__ px, const float* __restrict__ py,
     const float* __restrict__ pz, float* __restrict__ ux, float* __restrict__ uy,
     float* __restrict__ uz, float* __restrict__ lfx, float* __restrict__ lfy,
@@ -400,6 +463,9 @@ __global__ void STG_LB(N, STG_MINB) k_vel(
   N n;
   if (!n.init(g, k)) return;
   using T = typename N::T;
+  const int ac = ahead_cell<N>(g, 5 * k.nsm);
+  if (ac >= 0)
+    for (const float* p : {ls, px, py, pz}) pf_at(ac, p);
   const T lx = s_dn(AX(ls, 0)), ly = s_dn(AX(ls, 1)), lz = s_dn(AX(ls, 2));
   n.st(ux, fdiv(n.ld(px) + k.pref[0], dens(lx, k)));
   n.st(uy, fdiv(n.ld(py) + k.pref[1], dens(ly, k)));
@@ -538,6 +604,9 @@ __global__ void __launch_bounds__(BX * BY * BZ, N::W == 4 ? (SMAG ? STG_MINB4 : 
     unsigned* cw, KPar k, Geo g) {
   N n;
   const bool in = n.init(g, k);
+  const int ac = in ? ahead_cell<N>(g, 4 * k.nsm) : -1;
+  if (ac >= 0)
+    for (const float* p : {ux, uy, uz, rd, Ed, bx, by, bz}) pf_at(ac, p);
   if constexpr (!CW) {
     if (in) nu_raw_cell<SMAG, false>(n, ux, uy, uz, rd, Ed, bx, by, bz, sqxy, sqyz, sqzx, nv, k);
   } else {
@@ -698,7 +767,7 @@ __global__ void __launch_bounds__(32 * NUZ_TY) k_nu_maxsmooth(const float* __res
 
 // ln<nu> interpolated to the three faces (first half of the edge values).
 template <class N>
-__global__ void STG_LB(N, STG_MINB) k_nu_faces(
+__global__ void STG_LB_N(N, 6, STG_MINB) k_nu_faces(
     const float* __restrict__ lnu, float* __restrict__ lx, float* __restrict__ ly,
     float* __restrict__ lz, Geo g) {
   N n;
@@ -861,11 +930,11 @@ __device__ __forceinline__ typename N::T quench1(const float* __restrict__ f, co
     T m = -1.f;
 #pragma unroll
     for (int o = 0; o < 3; ++o) {
-      T d2 = (v[o + 2] - 2.f * v[o + 1]) + v[o];
+      T d2 = fma1(T(-2.f), v[o + 1], v[o + 2]) + v[o];
       T a2 = fabsf(d2);
       const T M3 = fmaxf(fmaxf(av[o], av[o + 1]), av[o + 2]);
-      const T M = QM3 ? M3 : av[o + 1] + k.qeps * M3;
-      T q = fdiv(a2, (M + a2 * k.inv_qmax) + 1e-30f);
+      const T M = QM3 ? M3 : fma1(T(k.qeps), M3, av[o + 1]);
+      T q = fdiv(a2, fma1(T(k.inv_qmax), a2, M) + T(1e-30f));
       m = fmaxf(m, q);
     }
     fac = fmaxf(fac, m);
