@@ -59,35 +59,6 @@ struct F4 {
     v[0] = a; v[1] = b; v[2] = c; v[3] = d;
   }
 };
-// On the device sums, products and multiply-adds run as packed pairs (one issue
-// slot for two lanes, the same rounding; fewer spills): 512^3 k_edge 4.27 -> 4.17
-// ms, k_flux 4.13 -> 4.11, k_tau 3.54 -> 3.57.
-#ifdef __CUDA_ARCH__
-#define STG_F4_PACKED(name, fn)                                                    \
-  __device__ __forceinline__ F4 name(const F4& a, const F4& b) {                   \
-    const float2 x = fn(make_float2(a.v[0], a.v[1]), make_float2(b.v[0], b.v[1])), \
-                 y = fn(make_float2(a.v[2], a.v[3]), make_float2(b.v[2], b.v[3])); \
-    return F4(x.x, x.y, y.x, y.y);                                                 \
-  }
-STG_F4_PACKED(operator+, __fadd2_rn)
-STG_F4_PACKED(operator*, __fmul2_rn)
-#undef STG_F4_PACKED
-// s a + b
-__device__ __forceinline__ F4 fma1(float s, const F4& a, const F4& b) {
-  const float2 t = make_float2(s, s);
-  const float2 x = __ffma2_rn(t, make_float2(a.v[0], a.v[1]), make_float2(b.v[0], b.v[1])),
-               y = __ffma2_rn(t, make_float2(a.v[2], a.v[3]), make_float2(b.v[2], b.v[3]));
-  return F4(x.x, x.y, y.x, y.y);
-}
-__device__ __forceinline__ F4 fma1(const F4& s, const F4& a, const F4& b) {
-  const float2 x = __ffma2_rn(make_float2(s.v[0], s.v[1]), make_float2(a.v[0], a.v[1]),
-                              make_float2(b.v[0], b.v[1])),
-               y = __ffma2_rn(make_float2(s.v[2], s.v[3]), make_float2(a.v[2], a.v[3]),
-                              make_float2(b.v[2], b.v[3]));
-  return F4(x.x, x.y, y.x, y.y);
-}
-__device__ __forceinline__ F4 operator-(const F4& a, const F4& b) { return fma1(-1.f, b, a); }
-#else
 #define STG_F4_BIN(op)                                                        \
   __device__ __forceinline__ F4 operator op(const F4& a, const F4& b) {       \
     return F4(a.v[0] op b.v[0], a.v[1] op b.v[1], a.v[2] op b.v[2], a.v[3] op b.v[3]); \
@@ -95,13 +66,8 @@ __device__ __forceinline__ F4 operator-(const F4& a, const F4& b) { return fma1(
 STG_F4_BIN(+)
 STG_F4_BIN(-)
 STG_F4_BIN(*)
+STG_F4_BIN(/)
 #undef STG_F4_BIN
-__device__ __forceinline__ F4 fma1(const F4& s, const F4& a, const F4& b) { return s * a + b; }
-#endif
-__device__ __forceinline__ float fma1(float s, float a, float b) { return s * a + b; }
-__device__ __forceinline__ F4 operator/(const F4& a, const F4& b) {
-  return F4(a.v[0] / b.v[0], a.v[1] / b.v[1], a.v[2] / b.v[2], a.v[3] / b.v[3]);
-}
 __device__ __forceinline__ F4 operator-(const F4& a) { return F4(-a.v[0], -a.v[1], -a.v[2], -a.v[3]); }
 __device__ __forceinline__ F4& operator+=(F4& a, const F4& b) { return a = a + b; }
 __device__ __forceinline__ F4& operator-=(F4& a, const F4& b) { return a = a - b; }
@@ -353,24 +319,24 @@ using Nb4Z = ZCell<Nb4>;
 // eq. (interp) to i+1/2 / i-1/2 and eq. (deriv) to i+1/2 / i-1/2, on a
 // functor v(o) giving the operand at offset o along the stencil axis.
 template <class V> __device__ __forceinline__ auto s_up(V v) -> decltype(v(0)) {
-  return fma1(IC_, v(-2) + v(3), fma1(IB_, v(-1) + v(2), IA_ * (v(0) + v(1))));
+  return IA_ * (v(0) + v(1)) + IB_ * (v(-1) + v(2)) + IC_ * (v(-2) + v(3));
 }
 template <class V> __device__ __forceinline__ auto s_dn(V v) -> decltype(v(0)) {
-  return fma1(IC_, v(-3) + v(2), fma1(IB_, v(-2) + v(1), IA_ * (v(-1) + v(0))));
+  return IA_ * (v(-1) + v(0)) + IB_ * (v(-2) + v(1)) + IC_ * (v(-3) + v(2));
 }
 template <class V> __device__ __forceinline__ auto s_du(V v, float ih) -> decltype(v(0)) {
-  return fma1(DC_, v(3) - v(-2), fma1(DB_, v(2) - v(-1), DA_ * (v(1) - v(0)))) * ih;
+  return (DA_ * (v(1) - v(0)) + DB_ * (v(2) - v(-1)) + DC_ * (v(3) - v(-2))) * ih;
 }
 template <class V> __device__ __forceinline__ auto s_dd(V v, float ih) -> decltype(v(0)) {
-  return fma1(DC_, v(2) - v(-3), fma1(DB_, v(1) - v(-2), DA_ * (v(0) - v(-1)))) * ih;
+  return (DA_ * (v(0) - v(-1)) + DB_ * (v(1) - v(-2)) + DC_ * (v(2) - v(-3))) * ih;
 }
 
 // s_dn and s_dd of the same taps (dn returned, the derivative in d).
 template <class V>
 __device__ __forceinline__ auto s_dn_dd(V v, float ih, decltype(v(0))& d) -> decltype(v(0)) {
   const auto a = v(-3), b = v(-2), c = v(-1), e = v(0), f = v(1), g = v(2);
-  d = fma1(DC_, g - a, fma1(DB_, f - b, DA_ * (e - c))) * ih;
-  return fma1(IC_, a + g, fma1(IB_, b + f, IA_ * (c + e)));
+  d = (DA_ * (e - c) + DB_ * (f - b) + DC_ * (g - a)) * ih;
+  return IA_ * (c + e) + IB_ * (b + f) + IC_ * (a + g);
 }
 
 // Ask for the cell's line of an array the kernel reads later, without a
@@ -930,11 +896,11 @@ __device__ __forceinline__ typename N::T quench1(const float* __restrict__ f, co
     T m = -1.f;
 #pragma unroll
     for (int o = 0; o < 3; ++o) {
-      T d2 = fma1(T(-2.f), v[o + 1], v[o + 2]) + v[o];
+      T d2 = (v[o + 2] - 2.f * v[o + 1]) + v[o];
       T a2 = fabsf(d2);
       const T M3 = fmaxf(fmaxf(av[o], av[o + 1]), av[o + 2]);
-      const T M = QM3 ? M3 : fma1(T(k.qeps), M3, av[o + 1]);
-      T q = fdiv(a2, fma1(T(k.inv_qmax), a2, M) + T(1e-30f));
+      const T M = QM3 ? M3 : av[o + 1] + k.qeps * M3;
+      T q = fdiv(a2, (M + a2 * k.inv_qmax) + 1e-30f);
       m = fmaxf(m, q);
     }
     fac = fmaxf(fac, m);
