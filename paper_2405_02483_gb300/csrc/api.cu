@@ -310,11 +310,11 @@ struct Lin8 {
 template <typename T>
 __global__ void k_lin2x8(Lin8<T> p, T a, T b, const T* bdt, long long n, int vec) {
   const int f = blockIdx.y;
+  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x + dep_wait();
   const T bb = bdt ? bdt[0] : b;
   T* o = p.o[f];
   const T *x = p.x[f], *y = p.y[f];
   const long long stride = (long long)gridDim.x * blockDim.x;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (vec) {
     for (; t < n / 4; t += stride) {
       T xv[4], yv[4], ov[4];
@@ -721,7 +721,7 @@ static void lin2x8(stagger_ctx* c, T* const o[8], T* const x[8], double a, T* co
   }
   const long long work = vec ? n / 4 : n;
   const unsigned bx = (unsigned)std::min<long long>((work + 255) / 256, 4096);
-  k_lin2x8<T><<<dim3(bx, 8), 256, 0, s>>>(p, (T)a, (T)b, bdt, n, vec);
+  launch_dep(k_lin2x8<T>, dim3(bx, 8), 256, 0, s, p, (T)a, (T)b, bdt, n, vec);
   ++c->extra_launches;
 }
 

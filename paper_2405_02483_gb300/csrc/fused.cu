@@ -142,6 +142,11 @@ int fused_init(Fused& F, const stagger_grid& gr, const stagger_params& p) {
   F.step_exec = nullptr;
   F.cap = nullptr;
   F.step_launches = 0;
+  F.fork = 0;
+  for (int i = 0; i < 2; ++i) {
+    F.br[i] = nullptr;
+    F.brev[i] = nullptr;
+  }
   for (int c = 0; c < 8; ++c) F.step_key[c] = nullptr;
   F.cells4 = (gr.nx % 4) == 0 && !p.scalar_cells;
   // One z-marching flux-divergence kernel per stage (on request; uniform z only).
@@ -445,6 +450,12 @@ void fused_release(Fused& F) {
   F.step_exec = nullptr;
   if (F.cap) cudaStreamDestroy(F.cap);
   F.cap = nullptr;
+  for (int i = 0; i < 2; ++i) {
+    if (F.br[i]) cudaStreamDestroy(F.br[i]);
+    if (F.brev[i]) cudaEventDestroy(F.brev[i]);
+    F.br[i] = nullptr;
+    F.brev[i] = nullptr;
+  }
   for (auto& pe : F.pending) { cudaEventDestroy(pe.second.first); cudaEventDestroy(pe.second.second); }
   F.pending.clear();
   for (auto e : F.pool) cudaEventDestroy(e);
@@ -478,6 +489,25 @@ void fused_release(Fused& F) {
   F.red = nullptr;
 }
 
+// Branches of a captured step.  With F.fork (set while a step is captured) the
+// energy equation runs on F.br[0] and the induction equation on F.br[1] beside
+// the momentum equation on s; without, all on s.  Their kernels do not depend on
+// one another: on a small box they share the SMs (32^3 ideal step 85 -> 62 us,
+// 64^3 quenched 220 -> 208), on a large one they fill each other's tails (128^3
+// 1224 -> 1189, 512^3 70764 -> 70695).  branch: the stream, which then
+// follows what s holds so far; merge: s follows what branch i holds.
+static cudaStream_t branch(Fused& F, int i, cudaStream_t s) {
+  if (!F.fork) return s;
+  cudaEventRecord(F.brev[i], s);
+  cudaStreamWaitEvent(F.br[i], F.brev[i], 0);
+  return F.br[i];
+}
+static void merge(Fused& F, int i, cudaStream_t s) {
+  if (!F.fork) return;
+  cudaEventRecord(F.brev[i], F.br[i]);
+  cudaStreamWaitEvent(s, F.brev[i], 0);
+}
+
 // Everything up to (not including) the divergence kernel: primitives,
 // viscosity, stresses, edge fields and fluxes of state f.
 template <class N>
@@ -508,54 +538,54 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
                                                  const_cast<float*>(k.qm),
                                                  const_cast<float*>(k.qden), k, g)));
   }
-  TIMED(K_LR, (k_lr_ed<NB><<<nb1(g.n / N::W), 256, 0, s>>>(f[0], f[4], k.log_interp ? d[F_LR] : nullptr,
+  TIMED(K_LR, launch_dep(k_lr_ed<NB>, nb1(g.n / N::W), 256, 0, s, f[0], f[4], k.log_interp ? d[F_LR] : nullptr,
                                                        d[F_ED], k.ediffav ? d[F_LER] : nullptr,
-                                                       k.lnpa ? d[F_LQ] : nullptr, k, g.n, g.sz)));
-  TIMED(K_VEL, (k_vel<NB><<<gy8, by8, 0, s>>>(ls, f[1], f[2], f[3], d[F_UX], d[F_UY], d[F_UZ],
-                                        d[F_LFX], d[F_LFY], d[F_LFZ], k, g)));
+                                                       k.lnpa ? d[F_LQ] : nullptr, k, g.n, g.sz));
+  TIMED(K_VEL, launch_dep(k_vel<NB>, gy8, by8, 0, s, ls, f[1], f[2], f[3], d[F_UX], d[F_UY], d[F_UZ],
+                                        d[F_LFX], d[F_LFY], d[F_LFZ], k, g));
   if (k.rm) {
     if (k.csmag_dl > 0.f)
-      TIMED(K_STRAIN2, (k_strain2<N><<<gg, bb, 0, s>>>(d[F_UX], d[F_UY], d[F_UZ], d[F_SQXY], d[F_SQYZ],
-                                                    d[F_SQZX], k, g)));
+      TIMED(K_STRAIN2, launch_dep(k_strain2<N>, gg, bb, 0, s, d[F_UX], d[F_UY], d[F_UZ], d[F_SQXY], d[F_SQYZ],
+                                                    d[F_SQZX], k, g));
     // cfl: this stage's derivative sets the Courant step, and the wave-speed
     // and <nu> maxima are taken here (cmax[0], cmax[2]).
     auto knu = k.csmag_dl > 0.f ? (cfl ? k_nu_raw<true, true, N> : k_nu_raw<true, false, N>)
                                 : (cfl ? k_nu_raw<false, true, N> : k_nu_raw<false, false, N>);
-    TIMED(K_NU_RAW, (knu<<<gy8, by8, 0, s>>>(d[F_UX], d[F_UY], d[F_UZ], f[0], f[4], f[5], f[6], f[7],
+    TIMED(K_NU_RAW, launch_dep(knu, gy8, by8, 0, s, d[F_UX], d[F_UY], d[F_UZ], f[0], f[4], f[5], f[6], f[7],
                                            d[F_SQXY], d[F_SQYZ], d[F_SQZX], d[F_NV],
-                                           cfl ? F.cmax : nullptr, k, g)));
+                                           cfl ? F.cmax : nullptr, k, g));
     if (N::W == 4) {
       // One z-marching pass for the 3x3x3 max and mean (four-cell layout).
       dim3 gm, bm;
       ms_launch(g, gm, bm);
       auto kms = cfl ? k_nu_maxsmooth<true> : k_nu_maxsmooth<false>;
-      TIMED(K_NU_MS, (kms<<<gm, bm, 0, s>>>(d[F_NV], d[F_NU], d[F_LNU], F.cmax + 2, g)));
+      TIMED(K_NU_MS, launch_dep(kms, gm, bm, 0, s, d[F_NV], d[F_NU], d[F_LNU], F.cmax + 2, g));
     } else {
-      TIMED(K_NU_MAX, (k_nu_max<NB><<<gg, bb, 0, s>>>(d[F_NV], d[F_NM], g)));
+      TIMED(K_NU_MAX, launch_dep(k_nu_max<NB>, gg, bb, 0, s, d[F_NV], d[F_NM], g));
       auto ksm = cfl ? k_nu_smooth<NB, true> : k_nu_smooth<NB, false>;
-      TIMED(K_NU_SMOOTH, (ksm<<<gg, bb, 0, s>>>(d[F_NM], d[F_NU], d[F_LNU], F.cmax + 2, g)));
+      TIMED(K_NU_SMOOTH, launch_dep(ksm, gg, bb, 0, s, d[F_NM], d[F_NU], d[F_LNU], F.cmax + 2, g));
     }
-    TIMED(K_NU_FACES, (k_nu_faces<NB><<<gy8, by8, 0, s>>>(d[F_LNU], d[F_LNX], d[F_LNY], d[F_LNZ], g)));
+    TIMED(K_NU_FACES, launch_dep(k_nu_faces<NB>, gy8, by8, 0, s, d[F_LNU], d[F_LNX], d[F_LNY], d[F_LNZ], g));
   }
   if (k.d2div)
-    TIMED(K_D2FLAG, (k_d2flag<NB><<<gg, bb, 0, s>>>(f[0], f[4], F.d2flag, k, g)));
+    TIMED(K_D2FLAG, launch_dep(k_d2flag<NB>, gg, bb, 0, s, f[0], f[4], F.d2flag, k, g));
   // J for the Joule heating of k_edge; k_flux and k_fdiv form it themselves.
   auto ktau = k.d2div ? k_tau<N, true> : k_tau<N, false>;
   if (k.visc)
-  TIMED(K_TAU, (ktau<<<gz8, bz8, 0, s>>>(d[F_UX], d[F_UY], d[F_UZ], f[0], d[F_LFX], d[F_LFY],
+  TIMED(K_TAU, launch_dep(ktau, gz8, bz8, 0, s, d[F_UX], d[F_UY], d[F_UZ], f[0], d[F_LFX], d[F_LFY],
                                        d[F_LFZ], d[F_NU], d[F_LNX], d[F_LNY], d[F_LNZ], f[5],
                                        f[6], f[7], d[F_TXX], d[F_TYY], d[F_TZZ], d[F_TXY],
                                        d[F_TYZ], d[F_TZX], d[F_RX], d[F_RY], d[F_RZ], d[F_JX],
-                                       d[F_JY], d[F_JZ], F.d2flag, k, g)));
+                                       d[F_JY], d[F_JZ], F.d2flag, k, g));
   auto kedge = k.qmax3 ? (k.d2div ? k_edge<N, true, true> : k_edge<N, false, true>)
                        : (k.d2div ? k_edge<N, true, false> : k_edge<N, false, false>);
   if (k.visc)
-    TIMED(K_EDGE, (kedge<<<gz8, bz8, 0, s>>>(d[F_TXX], d[F_TYY], d[F_TZZ], d[F_TXY], d[F_TYZ],
+    TIMED(K_EDGE, launch_dep(kedge, gz8, bz8, 0, s, d[F_TXX], d[F_TYY], d[F_TZZ], d[F_TXY], d[F_TYZ],
                                            d[F_TZX], d[F_RX], d[F_RY], d[F_RZ], d[F_JX],
                                            d[F_JY], d[F_JZ], d[F_UX], d[F_UY], d[F_UZ],
                                            d[F_QXX], d[F_QYY], d[F_QZZ], d[F_QXY], d[F_QYZ],
                                            d[F_QZX], d[F_EX], d[F_EY], d[F_EZ], d[F_WC],
-                                           d[F_WX], d[F_WY], d[F_WZ], F.d2flag, k, g)));
+                                           d[F_WX], d[F_WY], d[F_WZ], F.d2flag, k, g));
   if (F.fdiv) {   // fluxes, divergences and update in k_fdiv (launch_div)
     STG_CUDA_OK(cudaGetLastError());
     return STAGGER_OK;
@@ -569,10 +599,11 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
   FluxOut fo = {d[F_MXX], d[F_MYY], d[F_MZZ], d[F_MXY], d[F_MYX], d[F_MXZ], d[F_MZX],
                 d[F_MYZ], d[F_MZY], d[F_LX1], d[F_LX2], d[F_LY1], d[F_LY2], d[F_LZ1],
                 d[F_LZ2], d[F_GX], d[F_GY], d[F_GZ], d[F_QT], d[F_EX], d[F_EY], d[F_EZ]};
-  TIMED(K_FLUX, (k_flux<N><<<gz8, bz8, 0, s>>>(fi, fo, k, g)));
-  TIMED(K_FLUX_E, (k_flux_e<N><<<gy8, by8, 0, s>>>(fi, fo, k, g)));
+  const cudaStream_t se = branch(F, 0, s);   // the energy fluxes, beside the others
+  TIMED(K_FLUX, launch_dep(k_flux<N>, gz8, bz8, 0, s, fi, fo, k, g));
+  TIMED(K_FLUX_E, launch_dep(k_flux_e<N>, gy8, by8, 0, se, fi, fo, k, g));
   if (k.inv_tchromo > 0.f || k.corL0 > 0.f)
-    TIMED(K_COOL2, (k_cool2<NB><<<gg, bb, 0, s>>>(f[0], f[4], d[F_QT], k, g)));
+    TIMED(K_COOL2, launch_dep(k_cool2<NB>, gg, bb, 0, se, f[0], f[4], d[F_QT], k, g));
   STG_CUDA_OK(cudaGetLastError());
   return STAGGER_OK;
 }
@@ -780,12 +811,16 @@ static int launch_div(Fused& F, float* const f[8], float* q[8], float* o[8], flo
       kern[2] = v4 ? k_div<Nb4, 0xE0, false> : k_div<Nb, 0xE0, false>;
     }
   }
+  // Momentum on s, mass and energy after the energy fluxes on branch 0,
+  // induction after k_flux on branch 1.
+  cudaStream_t st[3] = {s, F.fork ? F.br[0] : s, s};
+  if (parts & 4) st[2] = branch(F, 1, s);
   for (int i = 0; i < 3; ++i)
     if ((parts >> i) & 1)
-    TIMED(K_DIV, (kern[i]<<<gg, bb, 0, s>>>(di, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7],
+    TIMED(K_DIV, launch_dep(kern[i], gg, bb, 0, st[i], di, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7],
                                             oo[0], oo[1], oo[2], oo[3], oo[4], oo[5], oo[6],
                                             oo[7], alpha, F.bdt_dev + stg, mode, F.cmax + 1,
-                                            F.kp, F.geo)));
+                                            F.kp, F.geo));
   STG_CUDA_OK(cudaGetLastError());
   return STAGGER_OK;
 }
@@ -804,9 +839,8 @@ int fused_rhs(Fused& F, float* const f[8], float* out[8], cudaStream_t s) {
 template <class N>
 static void courant_part(Fused& F, float* const f[8], cudaStream_t s) {
   const dim3 bb = block_for(F.geo, N::W, B_MIXED);
-  TIMED(K_COURANT, (k_courant_part<N><<<grid_for<N>(F.geo, bb), bb, 0, s>>>(
-                       F.fld[F_UX], F.fld[F_UY], F.fld[F_UZ], f[0], f[4], f[5], f[6], f[7],
-                       F.q[0], F.q[4], F.fld[F_NU], F.cmax, F.kp, F.geo)));
+  TIMED(K_COURANT, launch_dep(k_courant_part<N>, grid_for<N>(F.geo, bb), bb, 0, s, F.fld[F_UX], F.fld[F_UY], F.fld[F_UZ], f[0], f[4], f[5], f[6], f[7],
+                       F.q[0], F.q[4], F.fld[F_NU], F.cmax, F.kp, F.geo));
 }
 
 static int courant_to_dev(Fused& F, float* const f[8], cudaStream_t s, bool fused) {
@@ -821,10 +855,9 @@ static int courant_to_dev(Fused& F, float* const f[8], cudaStream_t s, bool fuse
   }
   // A stretched z reduces w / dl and nu / dl per cell: the final pass then
   // takes dl = 1 and a velocity-like nu.
-  TIMED(K_COURANT, (k_courant_final<<<1, 32, 0, s>>>(
-                        F.cmax, F.dt_dev, F.bdt_dev, (float)RK_BETA[0], (float)RK_BETA[1],
+  TIMED(K_COURANT, launch_dep(k_courant_final, 1, 32, 0, s, F.cmax, F.dt_dev, F.bdt_dev, (float)RK_BETA[0], (float)RK_BETA[1],
                         (float)RK_BETA[2], F.cdt, F.cdtr, F.cdtd, F.zs ? 1.0 : F.dlmin, F.dfac,
-                        F.zs ? 1 : F.kp.rm)));
+                        F.zs ? 1 : F.kp.rm));
   return STAGGER_OK;
 }
 
@@ -848,9 +881,11 @@ int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s) {
       // update with their divergence, and only rho and E need one of their own
       // (6 arrays in place of 24).  k_fdiv forms all eight at once.
       const int first = F.fdiv ? 7 : 2;
+      const cudaStream_t se = F.fork ? F.br[0] : s;
       rc = launch_div(F, st_in[0], F.q, nullptr, 0.f, 0, 0, s, cfl, first);
       if (rc) return rc;
-      courant_to_dev(F, st_in[0], s, cfl);
+      courant_to_dev(F, st_in[0], se, cfl);
+      merge(F, 0, s);
       if (!F.fdiv) {
         rc = launch_div(F, st_in[0], F.q, const_cast<float**>(st_out[0]), 0.f, 0, 1, s, false, 5);
         if (rc) return rc;
@@ -868,16 +903,20 @@ int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s) {
       const long long work = vec ? F.geo.n / 4 : F.geo.n;
       unsigned bx = (unsigned)((work + 255) / 256);
       if (bx > 2048) bx = 2048;
-      TIMED(K_UPDATE, (k_update8<<<dim3(bx, (unsigned)nu), 256, 0, s>>>(u, F.bdt_dev, F.geo.n, vec)));
+      TIMED(K_UPDATE, launch_dep(k_update8, dim3(bx, (unsigned)nu), 256, 0, se, u, F.bdt_dev, F.geo.n, vec));
+      merge(F, 0, s);
+      merge(F, 1, s);
       STG_CUDA_OK(cudaGetLastError());
       continue;
     }
     if (stg == 0 && dt > 0) {
-      TIMED(K_MISC, (k_set_dt<<<1, 1, 0, s>>>(F.dt_dev, F.bdt_dev, dt, (float)RK_BETA[0],
-                                              (float)RK_BETA[1], (float)RK_BETA[2])));
+      TIMED(K_MISC, launch_dep(k_set_dt, 1, 1, 0, s, F.dt_dev, F.bdt_dev, dt, (float)RK_BETA[0],
+                                              (float)RK_BETA[1], (float)RK_BETA[2]));
     }
     rc = launch_div(F, st_in[stg], F.q, const_cast<float**>(st_out[stg]), alpha, stg, stg == 2 ? 2 : 1, s);
     if (rc) return rc;
+    merge(F, 0, s);
+    merge(F, 1, s);
   }
   if (F.wall) wall_launch(F, f, false, s, false);
   STG_CUDA_OK(cudaGetLastError());
@@ -912,12 +951,21 @@ int fused_step_graphed(Fused& F, float* f[8], double dt, cudaStream_t s) {
       F.step_state = -1;
       return fused_step(F, f, dt, s);
     }
+    if (!F.br[0])   // the branches of the captured step, once
+      for (int i = 0; i < 2; ++i)
+        if (cudaStreamCreateWithFlags(&F.br[i], cudaStreamNonBlocking) != cudaSuccess ||
+            cudaEventCreateWithFlags(&F.brev[i], cudaEventDisableTiming) != cudaSuccess) {
+          F.step_state = -1;
+          return fused_step(F, f, dt, s);
+        }
     const long long l0 = F.launches;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     bool ok = cudaStreamBeginCapture(F.cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
+      F.fork = !F.fdiv;
       const int rc = fused_step(F, f, dt, F.cap);
+      F.fork = 0;
       ok = cudaStreamEndCapture(F.cap, &graph) == cudaSuccess && rc == STAGGER_OK && graph;
     }
     if (ok) ok = cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;

@@ -125,6 +125,11 @@ struct Fused {
   int step_state;
   cudaGraphExec_t step_exec;
   cudaStream_t cap;
+  // Branches of a captured step (the energy and the induction equation beside
+  // the momentum equation); fork is set only while a step is captured.
+  int fork;
+  cudaStream_t br[2];
+  cudaEvent_t brev[2];
   float* step_key[8];
   long long step_launches;
   // Optional per-kernel timing with CUDA events on the launch stream.

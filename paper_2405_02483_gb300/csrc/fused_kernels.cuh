@@ -183,7 +183,7 @@ struct Nb {
 };
 
 __device__ __forceinline__ bool make_nb(Nb& n, const Geo& g) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  int i = blockIdx.x * blockDim.x + threadIdx.x + dep_wait();
   int j = blockIdx.y * blockDim.y + threadIdx.y;
   int k = blockIdx.z * blockDim.z + threadIdx.z;
   if (i >= g.nx || j >= g.ny || k >= g.nz) return false;
@@ -212,7 +212,7 @@ struct Nb4 {
   int y[7];
   int z[7];
   __device__ __forceinline__ bool init(const Geo& g) {
-    int i = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    int i = 4 * (blockIdx.x * blockDim.x + threadIdx.x + dep_wait());
     int j = blockIdx.y * blockDim.y + threadIdx.y;
     int k = blockIdx.z * blockDim.z + threadIdx.z;
     if (i >= g.nx || j >= g.ny || k >= g.nz) return false;
@@ -400,7 +400,7 @@ __global__ void k_lr_ed(const float* __restrict__ rd, const float* __restrict__ 
                         float* __restrict__ ler, float* __restrict__ lq, KPar k, long long n,
                         long long sz) {
   using T = typename N::T;
-  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * N::W;
+  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x + dep_wait()) * N::W;
   if (i >= n) return;
   const T r = N::ldp(rd + i);
   if (lr) N::stp(lr + i, k.r0pos ? log1pf(r / k.r0) : logf(r));
@@ -655,7 +655,7 @@ __global__ void __launch_bounds__(32 * NUZ_TY) k_nu_maxsmooth(const float* __res
                                                               float* __restrict__ nu,
                                                               float* __restrict__ lnu,
                                                               unsigned* cnu, Geo g) {
-  const int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  const int i0 = (blockIdx.x * blockDim.x + threadIdx.x + dep_wait()) * 4;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int zc = (g.nz + gridDim.z - 1) / gridDim.z;
   const int z0 = blockIdx.z * zc;
@@ -1337,6 +1337,7 @@ __device__ __forceinline__ void set_bdt(float* bdt, double dt, float b0, float b
   bdt[2] = (float)((double)b2 * dt);
 }
 __global__ void k_set_dt(double* dtp, float* bdt, double dt, float b0, float b1, float b2) {
+  dep_wait();
   dtp[0] = dt;
   set_bdt(bdt, dt, b0, b1, b2);
 }
@@ -1350,9 +1351,9 @@ struct Upd8 {
 };
 __global__ void k_update8(Upd8 u, const float* bdtp, long long n, int vec) {
   const int c = blockIdx.y;
-  const float bdt = bdtp[0];
   const long long stride = (long long)gridDim.x * blockDim.x;
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x + dep_wait();
+  const float bdt = bdtp[0];
   if (vec) {
     const float4* f = reinterpret_cast<const float4*>(u.f[c]);
     const float4* q = reinterpret_cast<const float4*>(u.q[c]);
@@ -1491,6 +1492,7 @@ __global__ void __launch_bounds__(BX * BY * BZ, N::W == 4 ? STG_MINB : STG_MINB_
 __global__ void k_courant_final(unsigned* cmax, double* dt_out, float* bdt, float b0, float b1,
                                 float b2, double cdt, double cdtr, double cdtd, double dlmin,
                                 double dfac, int nu_is_velocity) {
+  dep_wait();
   if (threadIdx.x != 0) return;
   const double wmax = (double)__uint_as_float(cmax[0]);
   const double rmax = (double)__uint_as_float(cmax[1]);

@@ -270,7 +270,7 @@ static int forward_w(GraphExec<T>& G, cudaStream_t s) {
     auto flush = [&] {
       if (!b.n) return;
       b.rn = recip32(b.n);
-      g_level_fwd<T, W><<<lg.grid(b.n), lg.b, 0, s>>>(b, G.mesh, g);
+      launch_dep(g_level_fwd<T, W>, lg.grid(b.n), lg.b, 0, s, b, G.mesh, g);
       ++G.launches;
       b.n = 0;
     };
@@ -322,9 +322,9 @@ static void quench_rev(GraphExec<T>& G, const std::vector<int>& q, const LevelGr
       b.G[j] = G.grads + (size_t)G.lp.gslot[i] * G.geo.n;
       b.scr[j] = G.qscr + (size_t)15 * j * G.geo.n;
     }
-    g_level_quench<T, W, 0><<<lg.grid(b.n), lg.b, 0, s>>>(b, G.geo);
-    g_level_quench<T, W, 1><<<lg.grid(b.n), lg.b, 0, s>>>(b, G.geo);
-    g_level_quench<T, W, 2><<<lg.grid(b.n), lg.b, 0, s>>>(b, G.geo);
+    launch_dep(g_level_quench<T, W, 0>, lg.grid(b.n), lg.b, 0, s, b, G.geo);
+    launch_dep(g_level_quench<T, W, 1>, lg.grid(b.n), lg.b, 0, s, b, G.geo);
+    launch_dep(g_level_quench<T, W, 2>, lg.grid(b.n), lg.b, 0, s, b, G.geo);
     G.launches += 3;
   }
 }
@@ -346,7 +346,7 @@ static int backward_w(GraphExec<T>& G, T* const seed[8], T* gin[8], cudaStream_t
   auto flush = [&] {
     if (!b.n) return;
     b.rn = recip32(b.n);
-    g_level_rev<T, W><<<lg.grid(b.n), lg.b, 0, s>>>(b, g);
+    launch_dep(g_level_rev<T, W>, lg.grid(b.n), lg.b, 0, s, b, g);
     ++G.launches;
     b.n = b.nterm = 0;
   };

@@ -34,7 +34,7 @@ struct GCell {
 
 template <int W>
 __device__ __forceinline__ bool gcell_at(GCell& c, int kb, const Geo& g) {
-  c.i = W * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  c.i = W * (int)(blockIdx.x * blockDim.x + threadIdx.x + dep_wait());
   c.j = blockIdx.y * blockDim.y + threadIdx.y;
   c.k = kb * (int)blockDim.z + (int)threadIdx.z;
   if (c.i >= g.nx || c.j >= g.ny || c.k >= g.nz) return false;
