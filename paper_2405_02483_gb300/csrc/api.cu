@@ -685,9 +685,9 @@ template <typename T>
 static int ensure_work(stagger_ctx* c) {
   T*& w = work_of<T>(c);
   if (w) return STAGGER_OK;
-  // f1, f2, q, fbar, qbar, and the fixed state, cotangent-in and cotangent-out
-  // buffers of the captured adjoint (8 arrays each).
-  if (cudaMalloc(&w, sizeof(T) * 64 * (size_t)c->geo.n) != cudaSuccess) {
+  // f1, f2, q, qbar, and the fixed state and cotangent buffers of the captured
+  // adjoint (8 arrays each).
+  if (cudaMalloc(&w, sizeof(T) * 48 * (size_t)c->geo.n) != cudaSuccess) {
     w = nullptr;
     return STAGGER_EOOM;
   }
@@ -801,50 +801,62 @@ int stage_rhs<double>(stagger_ctx* c, GraphExec<double>* G, double* const f[8], 
 }
 
 // Adjoint of one fixed-dt step (see stagger_step_adjoint).
-// The adjoint of one step on its workspace, with dt read from c->dtp: the
-// body that the adjoint replays as a captured CUDA graph (see below).
+// The adjoint of one step on its workspace, with dt read from c->dtp: fb holds
+// the cotangent of the step's output and receives that of its input.  The
+// adjoint replays it as a captured CUDA graph (see below).
 template <typename T>
-static int adjoint_body(stagger_ctx* c, T* const f0[8], T* const lam_in[8], T* lam_out[8],
-                        cudaStream_t s) {
+static int adjoint_body(stagger_ctx* c, T* const f0[8], T* fb[8], cudaStream_t s) {
   GraphExec<T>* G = graph_of<T>(c);
   T* w = work_of<T>(c);
   const long long n = c->geo.n;
-  T *f1[8], *f2[8], *q[8], *fb[8], *qb[8];
+  T *f1[8], *f2[8], *q[8], *qb[8], *F[8];
   for (int k = 0; k < 8; ++k) {
     f1[k] = w + (size_t)(0 + k) * n;
     f2[k] = w + (size_t)(8 + k) * n;
     q[k] = w + (size_t)(16 + k) * n;
-    fb[k] = w + (size_t)(24 + k) * n;
-    qb[k] = w + (size_t)(32 + k) * n;
+    qb[k] = w + (size_t)(24 + k) * n;
   }
   const double* A = RK_ALPHA;
   int rc;
-  // Recompute the stage states f1, f2 (eqs. (ddt), (tupdate)); the FP32
-  // path takes F from the fused kernels, FP64 from the graph.
-  if ((rc = stage_rhs<T>(c, G, f0, fb, s))) return rc;
-  lin2x8<T>(c, q, fb, 1.0, fb, 0.0, -1, s);
-  lin2x8<T>(c, f1, f0, 1.0, q, 0.0, 0, s);
-  if ((rc = stage_rhs<T>(c, G, f1, fb, s))) return rc;
-  lin2x8<T>(c, q, q, A[1], fb, 1.0, -1, s);
-  lin2x8<T>(c, f2, f1, 1.0, q, 0.0, 1, s);
-  // Reverse sweep: fbar_3 = lam; qbar_3 = beta_3 dt fbar.
-  lin2x8<T>(c, fb, lam_in, 1.0, lam_in, 0.0, -1, s);
-  lin2x8<T>(c, qb, fb, 0.0, fb, 0.0, 2, s);
+  // The stage states f1, f2 (eqs. (ddt), (tupdate)).  With three sets of node
+  // values each stage is evaluated once, by the graph, and keeps its values for
+  // the reverse; with one, the FP32 path takes F from the fused kernels, FP64
+  // from the graph, and the reverse evaluates each stage again.
+  const bool keep = G->nsets == 3;
   T* const* stages[3] = {f0, f1, f2};
+  for (int st = 0; st < 2; ++st) {
+    if (keep) {
+      if ((rc = G->forward(stages[st], s, st))) return rc;
+      if (st == 0)   // q of stage 1 is F, which its set keeps
+        for (int k = 0; k < 8; ++k) F[k] = G->output(k);
+    } else {
+      if ((rc = stage_rhs<T>(c, G, stages[st], st ? qb : q, s))) return rc;
+      if (st == 0)
+        for (int k = 0; k < 8; ++k) F[k] = q[k];
+    }
+    if (st == 1) {
+      T* F1[8];
+      for (int k = 0; k < 8; ++k) F1[k] = keep ? G->output(k) : qb[k];
+      lin2x8<T>(c, q, F, A[1], F1, 1.0, -1, s);
+    }
+    lin2x8<T>(c, st ? f2 : f1, stages[st], 1.0, st ? q : F, 0.0, st, s);
+  }
+  // Reverse sweep: qbar_3 = beta_3 dt fbar.
+  lin2x8<T>(c, qb, fb, 0.0, fb, 0.0, 2, s);
   for (int st = 2; st >= 0; --st) {
-    if ((rc = G->forward(stages[st], s))) return rc;
+    if (keep && st < 2) G->use(st, stages[st]);
+    else if ((rc = G->forward(stages[st], s, keep ? st : 0))) return rc;
     if ((rc = G->backward(qb, fb, s))) return rc;     // fbar += J(f_st)^T qbar
     if (st > 0)                                         // qbar_{st} = alpha qbar + beta dt fbar
       lin2x8<T>(c, qb, qb, A[st], fb, 0.0, st - 1, s);
   }
-  lin2x8<T>(c, lam_out, fb, 1.0, fb, 0.0, -1, s);
   STG_CUDA_OK(cudaGetLastError());
   return STAGGER_OK;
 }
 
 // Adjoint of one fixed-dt step (see stagger_step_adjoint).  The first call
 // captures adjoint_body on fixed workspace buffers into a CUDA graph (about
-// 4000 launches); every call copies the state and cotangent in, replays the
+// 220 launches); every call copies the state and cotangent in, replays the
 // graph on the caller's stream, and copies the result out.  If capture is not
 // available the body is launched directly (the same kernels).
 template <typename T>
@@ -867,11 +879,10 @@ static int graph_step_adjoint(stagger_ctx* c, T* const f0[8], double dt, T* cons
   const int pi = sizeof(T) == sizeof(float) ? 0 : 1;
   const long long n = c->geo.n;
   T* w = work_of<T>(c);
-  T *f0c[8], *lin[8], *lout[8];
+  T *f0c[8], *fb[8];
   for (int k = 0; k < 8; ++k) {
-    f0c[k] = w + (size_t)(40 + k) * n;
-    lin[k] = w + (size_t)(48 + k) * n;
-    lout[k] = w + (size_t)(56 + k) * n;
+    f0c[k] = w + (size_t)(32 + k) * n;
+    fb[k] = w + (size_t)(40 + k) * n;
   }
   if (c->adj_state[pi] == 0) {
     c->adj_state[pi] = -1;
@@ -881,7 +892,7 @@ static int graph_step_adjoint(stagger_ctx* c, T* const f0[8], double dt, T* cons
       const long long before = stagger_launch_count(c);
       cudaGraph_t graph = nullptr;
       if (cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-        const int brc = adjoint_body<T>(c, f0c, lin, lout, c->cap);
+        const int brc = adjoint_body<T>(c, f0c, fb, c->cap);
         const cudaError_t ec = cudaStreamEndCapture(c->cap, &graph);
         if (brc == STAGGER_OK && ec == cudaSuccess && graph &&
             cudaGraphInstantiate(&c->adj_exec[pi], graph, 0) == cudaSuccess)
@@ -895,16 +906,20 @@ static int graph_step_adjoint(stagger_ctx* c, T* const f0[8], double dt, T* cons
       c->fused.timing = timing;
     }
   }
-  if (c->adj_state[pi] != 1) return adjoint_body<T>(c, f0, lam_in, lam_out, s);
   const size_t bytes = sizeof(T) * (size_t)n;
   for (int k = 0; k < 8; ++k) {
-    STG_CUDA_OK(cudaMemcpyAsync(f0c[k], f0[k], bytes, cudaMemcpyDeviceToDevice, s));
-    STG_CUDA_OK(cudaMemcpyAsync(lin[k], lam_in[k], bytes, cudaMemcpyDeviceToDevice, s));
+    STG_CUDA_OK(cudaMemcpyAsync(fb[k], lam_in[k], bytes, cudaMemcpyDeviceToDevice, s));
+    if (c->adj_state[pi] == 1)
+      STG_CUDA_OK(cudaMemcpyAsync(f0c[k], f0[k], bytes, cudaMemcpyDeviceToDevice, s));
   }
-  STG_CUDA_OK(cudaGraphLaunch(c->adj_exec[pi], s));
-  c->extra_launches += c->adj_launches[pi];
+  if (c->adj_state[pi] == 1) {
+    STG_CUDA_OK(cudaGraphLaunch(c->adj_exec[pi], s));
+    c->extra_launches += c->adj_launches[pi];
+  } else if ((rc = adjoint_body<T>(c, f0, fb, s))) {
+    return rc;
+  }
   for (int k = 0; k < 8; ++k)
-    STG_CUDA_OK(cudaMemcpyAsync(lam_out[k], lout[k], bytes, cudaMemcpyDeviceToDevice, s));
+    STG_CUDA_OK(cudaMemcpyAsync(lam_out[k], fb[k], bytes, cudaMemcpyDeviceToDevice, s));
   return STAGGER_OK;
 }
 

@@ -156,7 +156,20 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads) {
   size_t nval = 0;
   for (auto& nd : def.nodes)
     if (nd.op != G_INPUT) ++nval;
-  if (cudaMalloc(&vals, sizeof(T) * nval * g.n) != cudaSuccess) { vals = nullptr; return STAGGER_EOOM; }
+  // FP64: values of all three stages where they take no more than 8 GiB (the
+  // quenched physics to 128^3), so that the adjoint evaluates each stage once.
+  // FP32 takes its stage states from the fused kernels, whose results differ from
+  // the graph's by rounding, and keeps one set.
+  nsets = sizeof(T) == sizeof(double) && with_grads &&
+                  3.0 * sizeof(T) * nval * g.n <= 8.0 * (1ull << 30) ? 3 : 1;
+  if (cudaMalloc(&vals, sizeof(T) * nsets * nval * g.n) != cudaSuccess) {
+    cudaGetLastError();
+    nsets = 1;
+    if (cudaMalloc(&vals, sizeof(T) * nval * g.n) != cudaSuccess) {
+      vals = nullptr;
+      return STAGGER_EOOM;
+    }
+  }
   bool has_pmean = false;
   int nquench = 0;
   near = true;
@@ -198,11 +211,18 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads) {
       return STAGGER_EOOM;
     }
   }
+  nvals = nval;
   ptr.assign(nn, nullptr);
-  size_t v = 0;
-  for (size_t i = 0; i < nn; ++i)
-    if (def.nodes[i].op != G_INPUT) ptr[i] = vals + (v++) * g.n;
+  T* none[8] = {};
+  use(0, none);
   return STAGGER_OK;
+}
+
+template <typename T>
+void GraphExec<T>::use(int set, T* const in[8]) {
+  size_t v = (size_t)set * nvals;
+  for (size_t i = 0; i < def.nodes.size(); ++i)
+    ptr[i] = def.nodes[i].op == G_INPUT ? in[def.nodes[i].sk] : vals + (v++) * geo.n;
 }
 
 template <typename T>
@@ -296,9 +316,8 @@ static int forward_w(GraphExec<T>& G, cudaStream_t s) {
 }
 
 template <typename T>
-int GraphExec<T>::forward(T* const in[8], cudaStream_t s) {
-  for (size_t i = 0; i < def.nodes.size(); ++i)
-    if (def.nodes[i].op == G_INPUT) ptr[i] = in[def.nodes[i].sk];
+int GraphExec<T>::forward(T* const in[8], cudaStream_t s, int set) {
+  use(set, in);
   // FP64 takes one cell a thread: its pipe, not the loads, is the bound (32^3
   // adjoint step 2.8 ms against 3.8 with four).
   if constexpr (sizeof(T) == sizeof(float))

@@ -162,7 +162,9 @@ template <typename T>
 struct GraphExec {
   GraphDef def;
   Geo geo;
-  T* vals = nullptr;     // node values (non-input nodes)
+  T* vals = nullptr;     // node values (nvals non-input nodes), nsets sets
+  size_t nvals = 0;
+  int nsets = 1;
   T* mesh = nullptr;     // the mesh arrays of G_ZFIELD on the device, or null
   T* psum = nullptr;     // per-plane sums of G_PMEAN (nz), or null
   T* qscr = nullptr;     // scratch of the G_QUENCH transposes, nscr sets of 15 arrays, or null
@@ -175,10 +177,12 @@ struct GraphExec {
 
   int init(const GraphDef& d, const Geo& g, bool with_grads);
   void release();
-  // Evaluate every node; inputs are the 8 stored deviation arrays.
-  int forward(T* const in[8], cudaStream_t s);
-  // Reverse sweep: seed the 8 output gradients, accumulate into gin[8]
-  // (+=).  forward() must have run on the same inputs.
+  // The values of a set, evaluated on the inputs in.
+  void use(int set, T* const in[8]);
+  // Evaluate every node into a set; inputs are the 8 stored deviation arrays.
+  int forward(T* const in[8], cudaStream_t s, int set = 0);
+  // Reverse sweep over the set in use: seed the 8 output gradients, accumulate
+  // into gin[8] (+=).
   int backward(T* const seed[8], T* gin[8], cudaStream_t s);
   T* output(int k) { return ptr[def.out[k]]; }
 };
