@@ -14,6 +14,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "fused_kernels.cuh"
@@ -489,6 +490,26 @@ void fused_release(Fused& F) {
   F.red = nullptr;
 }
 
+// Lanes along x of k_flux_e4's blocks (32, 16 or 8, the rest rows), those that
+// cover the plane with the fewest threads; 0 (k_flux_e) where they are a quarter
+// more than the cells need (planes of few rows), and on boxes of less than two
+// blocks an SM (64^3 step 213 us with k_flux_e4, 208 without; 80^3 389, 393).
+static int flux_e4_lanes(const Geo& g) {
+  if (g.n < 2LL * 152 * 4 * BX * BY * BZ) return 0;
+  const long long l4 = g.nx / 4;
+  long long least = 0;
+  int best = 0;
+  for (int lx : {32, 16, 8}) {
+    const long long ly = BX * BY * BZ / lx;
+    const long long t = (l4 + lx - 1) / lx * lx * (((long long)g.ny + ly - 1) / ly * ly);
+    if (!best || t < least) {
+      least = t;
+      best = lx;
+    }
+  }
+  return least <= l4 * g.ny + l4 * g.ny / 4 ? best : 0;
+}
+
 // Branches of a captured step.  With F.fork (set while a step is captured) the
 // energy equation runs on F.br[0] and the induction equation on F.br[1] beside
 // the momentum equation on s; without, all on s.  Their kernels do not depend on
@@ -601,7 +622,16 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
                 d[F_LZ2], d[F_GX], d[F_GY], d[F_GZ], d[F_QT], d[F_EX], d[F_EY], d[F_EZ]};
   const cudaStream_t se = branch(F, 0, s);   // the energy fluxes, beside the others
   TIMED(K_FLUX, launch_dep(k_flux<N>, gz8, bz8, 0, s, fi, fo, k, g));
-  TIMED(K_FLUX_E, launch_dep(k_flux_e<N>, gy8, by8, 0, se, fi, fo, k, g));
+  const int lx = std::is_same<N, Nb4>::value && k.visc ? flux_e4_lanes(g) : 0;
+  if (lx) {
+    const int ly = BX * BY * BZ / lx;
+    const dim3 ge((unsigned)((g.nx / 4 + lx - 1) / lx), (unsigned)((g.ny + ly - 1) / ly),
+                  (unsigned)g.nz);
+    auto kf = lx == 32 ? k_flux_e4<32> : lx == 16 ? k_flux_e4<16> : k_flux_e4<8>;
+    TIMED(K_FLUX_E, launch_dep(kf, ge, dim3((unsigned)lx, (unsigned)ly), 0, se, fi, fo, k, g));
+  } else {
+    TIMED(K_FLUX_E, launch_dep(k_flux_e<N>, gy8, by8, 0, se, fi, fo, k, g));
+  }
   if (k.inv_tchromo > 0.f || k.corL0 > 0.f)
     TIMED(K_COOL2, launch_dep(k_cool2<NB>, gg, bb, 0, se, f[0], f[4], d[F_QT], k, g));
   STG_CUDA_OK(cudaGetLastError());
