@@ -137,7 +137,41 @@ static bool aligned16(float* const* a, int n) {
   return (u & 15) == 0;
 }
 
+// The kernels' box from the caller's and F.pad (off where a padded array would
+// pass 2^31 elements).
+static void pad_geo(Fused& F) {
+  const long long pitch = Nb4P::pitch(F.geo.nx);
+  if (pitch * F.geo.ny * F.geo.nz >= (1LL << 31)) F.pad = 0;
+  F.kgeo = F.geo;
+  if (!F.pad) return;
+  F.kgeo.sy = pitch;
+  F.kgeo.sz = pitch * F.geo.ny;
+  F.kgeo.n = F.kgeo.sz * F.geo.nz;
+}
+
+// An array of the kernels' box.  Padded rows start 4 ghost columns before a
+// 128-byte line, so that the cells themselves start on one.
+static const int PAD_OFF = 28;
+static float* new_array(const Fused& F) {
+  float* a = nullptr;
+  const int off = F.pad ? PAD_OFF : 0;
+  if (cudaMalloc(&a, sizeof(float) * ((size_t)F.kgeo.n + off)) != cudaSuccess) return nullptr;
+  return a + off;
+}
+static void free_array(const Fused& F, float*& a) {
+  if (a) cudaFree(a - (F.pad ? PAD_OFF : 0));
+  a = nullptr;
+}
+
+static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& p, int pad);
 int fused_init(Fused& F, const stagger_grid& gr, const stagger_params& p) {
+  // Without room for the padded copies the one-cell kernels run on the caller's rows.
+  const int rc = fused_init_t(F, gr, p, 1);
+  if (rc != STAGGER_EOOM || !F.pad) return rc;
+  cudaGetLastError();
+  return fused_init_t(F, gr, p, 0);
+}
+static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& p, int pad) {
   F.geo = make_geo(gr.nx, gr.ny, gr.nz);
   F.step_state = 0;
   F.step_exec = nullptr;
@@ -150,6 +184,15 @@ int fused_init(Fused& F, const stagger_grid& gr, const stagger_params& p) {
   }
   for (int c = 0; c < 8; ++c) F.step_key[c] = nullptr;
   F.cells4 = (gr.nx % 4) == 0 && !p.scalar_cells;
+  // Rows of no multiple of four cells: the stages run on padded copies of the
+  // state with four cells a thread (Nb4P), for periodic, uniform boxes of the
+  // split layout without plane means, from the size where that is the faster
+  // mapping (quenched step, us, padded against one cell: 49^3 244 / 244, 65^3 412 /
+  // 484, 131^3 2051 / 2871, 301^3 19617 / 29798; the copies are 5% of it).
+  F.pad = (gr.nx % 4) != 0 && gr.nx >= 8 && !p.scalar_cells && !p.zwalls && !p.zc &&
+          !p.fuse_flux_div && !(p.t_chromo > 0) && !p.ediffav && !p.lnp_aver &&
+          F.geo.n >= 3 * (1LL << 16) && pad;
+  pad_geo(F);
   // One z-marching flux-divergence kernel per stage (on request; uniform z only).
   F.fdiv = p.fuse_flux_div && p.zc == nullptr;
   // z walls at the planes zghost and nz - 1 - zghost: 0 periodic, 1 closed
@@ -281,9 +324,8 @@ int fused_init(Fused& F, const stagger_grid& gr, const stagger_params& p) {
   F.dlmin = dlmin;
   F.dfac = fmax(1.0, fmax(p.nuE, p.nuB * dlmax / dlmin));
 
-  const size_t bytes = sizeof(float) * (size_t)F.geo.n;
   for (int i = 0; i < F_COUNT; ++i) F.fld[i] = nullptr;
-  for (int c = 0; c < 8; ++c) F.q[c] = F.ping[c] = F.pong[c] = nullptr;
+  for (int c = 0; c < 8; ++c) F.q[c] = F.ping[c] = F.pong[c] = F.padst[c] = nullptr;
   F.dt_dev = nullptr;
   F.bdt_dev = nullptr;
   F.red = nullptr;
@@ -417,17 +459,20 @@ int fused_init(Fused& F, const stagger_grid& gr, const stagger_params& p) {
   if (k.visc && k.do_quench)
     for (int f : {F_QXX, F_QYY, F_QZZ, F_QXY, F_QYZ, F_QZX}) need.push_back(f);
   for (int f : need)
-    if (cudaMalloc(&F.fld[f], bytes) != cudaSuccess) { F.fld[f] = nullptr; fused_release(F); return STAGGER_EOOM; }
+    if (!(F.fld[f] = new_array(F))) { fused_release(F); return STAGGER_EOOM; }
   for (int c = 0; c < 8; ++c) {
-    if (cudaMalloc(&F.q[c], bytes) != cudaSuccess || cudaMalloc(&F.ping[c], bytes) != cudaSuccess ||
-        cudaMalloc(&F.pong[c], bytes) != cudaSuccess) {
+    F.q[c] = new_array(F);
+    F.ping[c] = new_array(F);
+    F.pong[c] = new_array(F);
+    if (F.pad) F.padst[c] = new_array(F);
+    if (!F.q[c] || !F.ping[c] || !F.pong[c] || (F.pad && !F.padst[c])) {
       fused_release(F);
       return STAGGER_EOOM;
     }
   }
   dim3 gg = grid3(F.geo);
   F.red_blocks = (int)(gg.x * gg.y * gg.z);
-  if (k.d2div && cudaMalloc(&F.d2flag, (size_t)F.geo.n) != cudaSuccess) {
+  if (k.d2div && cudaMalloc(&F.d2flag, (size_t)F.kgeo.n) != cudaSuccess) {
     F.d2flag = nullptr;
     fused_release(F);
     return STAGGER_EOOM;
@@ -461,12 +506,9 @@ void fused_release(Fused& F) {
   F.pending.clear();
   for (auto e : F.pool) cudaEventDestroy(e);
   F.pool.clear();
-  for (int i = 0; i < F_COUNT; ++i) { if (F.fld[i]) cudaFree(F.fld[i]); F.fld[i] = nullptr; }
+  for (int i = 0; i < F_COUNT; ++i) free_array(F, F.fld[i]);
   for (int c = 0; c < 8; ++c) {
-    if (F.q[c]) cudaFree(F.q[c]);
-    if (F.ping[c]) cudaFree(F.ping[c]);
-    if (F.pong[c]) cudaFree(F.pong[c]);
-    F.q[c] = F.ping[c] = F.pong[c] = nullptr;
+    for (float** a : {&F.q[c], &F.ping[c], &F.pong[c], &F.padst[c]}) free_array(F, *a);
   }
   if (F.dt_dev) cudaFree(F.dt_dev);
   if (F.bdt_dev) cudaFree(F.bdt_dev);
@@ -533,7 +575,7 @@ static void merge(Fused& F, int i, cudaStream_t s) {
 // viscosity, stresses, edge fields and fluxes of state f.
 template <class N>
 static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
-  const Geo& g = F.geo;
+  const Geo& g = F.kgeo;
   const KPar& k = F.kp;
   float** d = F.fld;
   const dim3 bb = block_for(g, N::W, B_MIXED), bz8 = block_for(g, N::W, B_LONGZ),
@@ -575,11 +617,11 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
     TIMED(K_NU_RAW, launch_dep(knu, gy8, by8, 0, s, d[F_UX], d[F_UY], d[F_UZ], f[0], f[4], f[5], f[6], f[7],
                                            d[F_SQXY], d[F_SQYZ], d[F_SQZX], d[F_NV],
                                            cfl ? F.cmax : nullptr, k, g));
-    if (N::W == 4) {
+    if constexpr (N::W == 4) {
       // One z-marching pass for the 3x3x3 max and mean (four-cell layout).
       dim3 gm, bm;
       ms_launch(g, gm, bm);
-      auto kms = cfl ? k_nu_maxsmooth<true> : k_nu_maxsmooth<false>;
+      auto kms = cfl ? k_nu_maxsmooth<true, NB> : k_nu_maxsmooth<false, NB>;
       TIMED(K_NU_MS, launch_dep(kms, gm, bm, 0, s, d[F_NV], d[F_NU], d[F_LNU], F.cmax + 2, g));
     } else {
       TIMED(K_NU_MAX, launch_dep(k_nu_max<NB>, gg, bb, 0, s, d[F_NV], d[F_NM], g));
@@ -730,6 +772,7 @@ static void wall_launch(Fused& F, float* const f[8], bool zero, cudaStream_t s, 
 }
 
 static int pre_div(Fused& F, float* const f[8], cudaStream_t s, bool cfl = false) {
+  if (F.pad) return pre_div_t<Nb4P>(F, f, s, cfl);
   const bool v4 = F.cells4 && aligned16(f, 8);
   if (F.zs) return v4 ? pre_div_t<Nb4Z>(F, f, s, false) : pre_div_t<NbZ>(F, f, s, false);
   return v4 ? pre_div_t<Nb4>(F, f, s, cfl) : pre_div_t<Nb>(F, f, s, cfl);
@@ -815,15 +858,19 @@ static int launch_div(Fused& F, float* const f[8], float* q[8], float* o[8], flo
   DivIn di = div_in(F, f);
   float* oo[8];
   for (int c = 0; c < 8; ++c) oo[c] = o ? o[c] : q[c];
-  const bool v4 = F.cells4 && aligned16(f, 8) && aligned16(q, 8) && aligned16(oo, 8);
-  const dim3 bb = block_for(F.geo, v4 ? 4 : 1, B_LONGZ),
-             gg = v4 ? grid_for<Nb4>(F.geo, bb) : grid_for<Nb>(F.geo, bb);
+  const bool v4 = F.pad || (F.cells4 && aligned16(f, 8) && aligned16(q, 8) && aligned16(oo, 8));
+  const dim3 bb = block_for(F.kgeo, v4 ? 4 : 1, B_LONGZ),
+             gg = v4 ? grid_for<Nb4>(F.kgeo, bb) : grid_for<Nb>(F.kgeo, bb);
   // Momentum; mass and energy; induction (disjoint inputs, one kernel each).
   typedef void (*DivK)(DivIn, float*, float*, float*, float*, float*, float*, float*, float*,
                        float*, float*, float*, float*, float*, float*, float*, float*, float,
                        const float*, int, unsigned*, KPar, Geo);
   DivK kern[3];
-  if (F.zs) {
+  if (F.pad) {
+    kern[0] = k_div<Nb4P, 0x0E, false>;
+    kern[1] = cfl ? k_div<Nb4P, 0x11, true> : k_div<Nb4P, 0x11, false>;
+    kern[2] = k_div<Nb4P, 0xE0, false>;
+  } else if (F.zs) {
     kern[0] = v4 ? k_div<Nb4Z, 0x0E, false> : k_div<NbZ, 0x0E, false>;
     kern[1] = v4 ? k_div<Nb4Z, 0x11, false> : k_div<NbZ, 0x11, false>;
     kern[2] = v4 ? k_div<Nb4Z, 0xE0, false> : k_div<NbZ, 0xE0, false>;
@@ -850,12 +897,43 @@ static int launch_div(Fused& F, float* const f[8], float* q[8], float* o[8], flo
     TIMED(K_DIV, launch_dep(kern[i], gg, bb, 0, st[i], di, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7],
                                             oo[0], oo[1], oo[2], oo[3], oo[4], oo[5], oo[6],
                                             oo[7], alpha, F.bdt_dev + stg, mode, F.cmax + 1,
-                                            F.kp, F.geo));
+                                            F.kp, F.kgeo));
   STG_CUDA_OK(cudaGetLastError());
   return STAGGER_OK;
 }
 
+// The caller's state into F.padst, and padded arrays into the caller's.
+static void pad_in(Fused& F, float* const f[8], cudaStream_t s) {
+  Pad8 a;
+  for (int c = 0; c < 8; ++c) {
+    a.s[c] = f[c];
+    a.d[c] = F.padst[c];
+  }
+  const int rows = F.geo.ny * F.geo.nz;
+  TIMED(K_MISC, launch_dep(k_pad8, dim3((unsigned)((rows + 7) / 8), 8), dim3(32, 8), 0, s, a,
+                           F.geo.nx, (int)F.kgeo.sy, rows));
+}
+static void pad_out(Fused& F, float* const src[8], float* const dst[8], cudaStream_t s) {
+  Pad8 a;
+  for (int c = 0; c < 8; ++c) {
+    a.s[c] = src[c];
+    a.d[c] = dst[c];
+  }
+  const int rows = F.geo.ny * F.geo.nz;
+  TIMED(K_MISC, launch_dep(k_unpad8, dim3((unsigned)((rows + 7) / 8), 8), dim3(32, 8), 0, s, a,
+                           F.geo.nx, (int)F.kgeo.sy, rows));
+}
+
 int fused_rhs(Fused& F, float* const f[8], float* out[8], cudaStream_t s) {
+  if (F.pad) {
+    pad_in(F, f, s);
+    int st = pre_div(F, F.padst, s);
+    if (!st) st = launch_div(F, F.padst, F.q, nullptr, 0.f, 0, 0, s);
+    if (st) return st;
+    pad_out(F, F.q, out, s);
+    STG_CUDA_OK(cudaGetLastError());
+    return STAGGER_OK;
+  }
   if (F.wall) wall_launch(F, f, false, s);
   int st = pre_div(F, f, s);
   if (st) return st;
@@ -868,9 +946,9 @@ int fused_rhs(Fused& F, float* const f[8], float* out[8], cudaStream_t s) {
 
 template <class N>
 static void courant_part(Fused& F, float* const f[8], cudaStream_t s) {
-  const dim3 bb = block_for(F.geo, N::W, B_MIXED);
-  TIMED(K_COURANT, launch_dep(k_courant_part<N>, grid_for<N>(F.geo, bb), bb, 0, s, F.fld[F_UX], F.fld[F_UY], F.fld[F_UZ], f[0], f[4], f[5], f[6], f[7],
-                       F.q[0], F.q[4], F.fld[F_NU], F.cmax, F.kp, F.geo));
+  const dim3 bb = block_for(F.kgeo, N::W, B_MIXED);
+  TIMED(K_COURANT, launch_dep(k_courant_part<N>, grid_for<N>(F.kgeo, bb), bb, 0, s, F.fld[F_UX], F.fld[F_UY], F.fld[F_UZ], f[0], f[4], f[5], f[6], f[7],
+                       F.q[0], F.q[4], F.fld[F_NU], F.cmax, F.kp, F.kgeo));
 }
 
 static int courant_to_dev(Fused& F, float* const f[8], cudaStream_t s, bool fused) {
@@ -878,6 +956,8 @@ static int courant_to_dev(Fused& F, float* const f[8], cudaStream_t s, bool fuse
   // with fused, the stage kernels already took the three maxima.
   const bool v4 = F.cells4 && aligned16(f, 8);
   if (fused) {
+  } else if (F.pad) {
+    courant_part<Nb4P>(F, f, s);
   } else if (F.zs) {
     if (v4) courant_part<Nb4Z>(F, f, s); else courant_part<NbZ>(F, f, s);
   } else {
@@ -895,7 +975,12 @@ int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s) {
   float* A[8];
   float* B[8];
   float* C[8];
-  for (int c = 0; c < 8; ++c) { A[c] = f[c]; B[c] = F.ping[c]; C[c] = F.pong[c]; }
+  for (int c = 0; c < 8; ++c) {
+    A[c] = F.pad ? F.padst[c] : f[c];
+    B[c] = F.ping[c];
+    C[c] = F.pong[c];
+  }
+  if (F.pad) pad_in(F, f, s);
   float* const* st_in[3] = {A, B, C};
   float* const* st_out[3] = {B, C, A};
   for (int stg = 0; stg < 3; ++stg) {
@@ -921,7 +1006,7 @@ int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s) {
         if (rc) return rc;
       }
       Upd8 u;
-      int vec = (F.geo.n % 4) == 0, nu = 0;
+      int vec = (F.kgeo.n % 4) == 0, nu = 0;
       for (int c = 0; c < 8; ++c) {
         if (!F.fdiv && c != 0 && c != 4) continue;
         u.f[nu] = st_in[0][c];
@@ -930,10 +1015,10 @@ int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s) {
         vec &= (((uintptr_t)u.f[nu] | (uintptr_t)u.q[nu] | (uintptr_t)u.o[nu]) & 15) == 0;
         ++nu;
       }
-      const long long work = vec ? F.geo.n / 4 : F.geo.n;
+      const long long work = vec ? F.kgeo.n / 4 : F.kgeo.n;
       unsigned bx = (unsigned)((work + 255) / 256);
       if (bx > 2048) bx = 2048;
-      TIMED(K_UPDATE, launch_dep(k_update8, dim3(bx, (unsigned)nu), 256, 0, se, u, F.bdt_dev, F.geo.n, vec));
+      TIMED(K_UPDATE, launch_dep(k_update8, dim3(bx, (unsigned)nu), 256, 0, se, u, F.bdt_dev, F.kgeo.n, vec));
       merge(F, 0, s);
       merge(F, 1, s);
       STG_CUDA_OK(cudaGetLastError());
@@ -948,13 +1033,16 @@ int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s) {
     merge(F, 0, s);
     merge(F, 1, s);
   }
+  if (F.pad) pad_out(F, A, f, s);
   if (F.wall) wall_launch(F, f, false, s, false);
   STG_CUDA_OK(cudaGetLastError());
   return STAGGER_OK;
 }
 
-int fused_dt(Fused& F, float* const f[8], cudaStream_t s) {
+int fused_dt(Fused& F, float* const fu[8], cudaStream_t s) {
   const bool cfl = cfl_fused(F);
+  if (F.pad) pad_in(F, fu, s);
+  float* const* f = F.pad ? F.padst : fu;
   if (F.wall) wall_launch(F, f, false, s);
   int rc = pre_div(F, f, s, cfl);
   if (rc) return rc;

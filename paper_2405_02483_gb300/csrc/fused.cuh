@@ -94,7 +94,12 @@ enum KId { K_LR = 0, K_VEL, K_STRAIN2, K_NU_RAW, K_NU_MAX, K_NU_SMOOTH, K_NU_FAC
 extern const char* const KNAMES[K_COUNT];
 
 struct Fused {
-  Geo geo;
+  Geo geo;              // the caller's box
+  // The kernels' box: the same, or with pad (nx no multiple of four) rows of
+  // padded pitch, the stages running on a padded copy of the state (padst).
+  Geo kgeo;
+  int pad;
+  float* padst[8];
   KPar kp;
   float* fld[F_COUNT];
   float* q[8];          // dfdt (2N storage)

@@ -269,6 +269,16 @@ struct Nb4 {
   static __device__ __forceinline__ void stp(float* p, const F4& v) {
     *reinterpret_cast<float4*>(p) = make_float4(v.v[0], v.v[1], v.v[2], v.v[3]);
   }
+  // Columns of the chunk i, its left and its right neighbour in a row of nx
+  // cells, and the store of a chunk at column x0 of a row (the marching kernel).
+  static __device__ __forceinline__ void chunk(int i, int nx, int& x0, int& xl, int& xr) {
+    x0 = i;
+    xl = wrap(i - 4, nx);
+    xr = wrap(i + 4, nx);
+  }
+  static __device__ __forceinline__ void put(float* row, int i, int, float4 v) {
+    *reinterpret_cast<float4*>(row + i) = v;
+  }
   // Per-cell switch flags: the four cells' bytes as one word (byte l, cell i0+l).
   __device__ __forceinline__ unsigned ldflag(const unsigned char* __restrict__ p) const {
     return __ldg(reinterpret_cast<const unsigned*>(p + c));
@@ -283,6 +293,70 @@ struct Nb4 {
   static __device__ __forceinline__ F4 sel(unsigned fl, int a, const F4& x, const F4& y) {
     return F4(((fl >> a) & 1u) ? x.v[0] : y.v[0], ((fl >> (8 + a)) & 1u) ? x.v[1] : y.v[1],
               ((fl >> (16 + a)) & 1u) ? x.v[2] : y.v[2], ((fl >> (24 + a)) & 1u) ? x.v[3] : y.v[3]);
+  }
+};
+
+// Nb4 for rows of any length nx >= 8, in arrays whose rows hold 4 ghost columns,
+// the nx cells and ghost columns up to the chunk after the last one (row pitch
+// Geo's sy): x taps need no wrap, every chunk is aligned, and a store also writes
+// the periodic images of its cells.  The last chunk's lanes past the row are
+// images: they are computed and not stored (where a kernel updates an array in
+// place, those lanes may read an image before or after its owner rewrites it;
+// nothing uses what they then hold).
+struct Nb4P : Nb4 {
+  using Base = Nb4P;
+  int i0, nx;
+  // (whole 128-byte lines: a block of 8 lanes reads one line a row)
+  static __host__ __device__ __forceinline__ int pitch(int nx) {
+    return (4 + (nx + 3) / 4 * 4 + 4 + 31) / 32 * 32;
+  }
+  static __device__ __forceinline__ void chunk(int i, int, int& x0, int& xl, int& xr) {
+    xl = i;
+    x0 = i + 4;
+    xr = i + 8;
+  }
+  __device__ __forceinline__ bool init(const Geo& g) {
+    i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x + dep_wait());
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    const int k = blockIdx.z * blockDim.z + threadIdx.z;
+    if (i0 >= g.nx || j >= g.ny || k >= g.nz) return false;
+    nx = g.nx;
+    chunk(i0, nx, x0, xl, xr);
+#pragma unroll
+    for (int o = -3; o <= 3; ++o) {
+      y[o + 3] = wrap(j + o, g.ny) * (int)g.sy;
+      z[o + 3] = wrap(k + o, g.nz) * (int)g.sz;
+    }
+    c = z[3] + y[3] + x0;
+    kz = k;
+    return true;
+  }
+  __device__ __forceinline__ bool init(const Geo& g, const KPar&) { return init(g); }
+  // row: the first ghost column of the row.
+  static __device__ __forceinline__ void put(float* row, int i, int nx, float4 q) {
+    const float v[4] = {q.x, q.y, q.z, q.w};
+    float* p = row + 4 + i;
+    if (i + 4 <= nx) {
+      *reinterpret_cast<float4*>(p) = q;
+    } else {
+#pragma unroll
+      for (int l = 0; l < 4; ++l)
+        if (i + l < nx) p[l] = v[l];
+    }
+    if (i < 8) {   // images right of the row, up to column (nx + 3) / 4 * 4 + 3
+      const int end = (nx + 3) / 4 * 4 + 4;
+#pragma unroll
+      for (int l = 0; l < 4; ++l)
+        if (i + l + nx < end) p[l + nx] = v[l];
+    }
+    if (i + 8 > nx) {   // images left of it, columns -4 .. -1
+#pragma unroll
+      for (int l = 0; l < 4; ++l)
+        if (i + l < nx && i + l >= nx - 4) p[l - nx] = v[l];
+    }
+  }
+  __device__ __forceinline__ void st(float* p, const F4& v) const {
+    put(p + c - x0, i0, nx, make_float4(v.v[0], v.v[1], v.v[2], v.v[3]));
   }
 };
 
@@ -650,7 +724,7 @@ __global__ void STG_LB(N, STG_MINB_HI) k_nu_smooth(const float* __restrict__ a,
 #ifndef NUZ_ZC
 #define NUZ_ZC 32
 #endif
-template <bool CW>
+template <bool CW, class N = Nb4>
 __global__ void __launch_bounds__(32 * NUZ_TY) k_nu_maxsmooth(const float* __restrict__ nv,
                                                               float* __restrict__ nu,
                                                               float* __restrict__ lnu,
@@ -662,7 +736,8 @@ __global__ void __launch_bounds__(32 * NUZ_TY) k_nu_maxsmooth(const float* __res
   const int z1 = min(z0 + zc, g.nz);
   unsigned mb = 0u;
   if (i0 < g.nx && j < g.ny) {
-    const int xl = wrap(i0 - 4, g.nx), xr = wrap(i0 + 4, g.nx);
+    int x0, xl, xr;
+    N::chunk(i0, g.nx, x0, xl, xr);
     long long yo[5];
 #pragma unroll
     for (int r = 0; r < 5; ++r) yo[r] = (long long)wrap(j + r - 2, g.ny) * g.sy;
@@ -677,7 +752,7 @@ __global__ void __launch_bounds__(32 * NUZ_TY) k_nu_maxsmooth(const float* __res
       for (int r = 0; r < 5; ++r) {
         const float* row = nv + po + yo[r];
         const float4 a = *reinterpret_cast<const float4*>(row + xl);
-        const float4 b = *reinterpret_cast<const float4*>(row + i0);
+        const float4 b = *reinterpret_cast<const float4*>(row + x0);
         const float4 c = *reinterpret_cast<const float4*>(row + xr);
         // positions i0-2 .. i0+5
         const float v[8] = {a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y};
@@ -712,7 +787,7 @@ __global__ void __launch_bounds__(32 * NUZ_TY) k_nu_maxsmooth(const float* __res
       }
       if (p < z0 + 2) continue;
       // Output plane p-2.
-      const long long o = (long long)(p - 2) * g.sz + (long long)j * g.sy + i0;
+      const long long o = (long long)(p - 2) * g.sz + (long long)j * g.sy;
       float4 vv, lv;
       float* vp = &vv.x;
       float* lp = &lv.x;
@@ -724,8 +799,8 @@ __global__ void __launch_bounds__(32 * NUZ_TY) k_nu_maxsmooth(const float* __res
         lp[l] = logf(fmaxf(v, 1e-30f));
         if (CW) mb = max(mb, max_bits(v));
       }
-      *reinterpret_cast<float4*>(nu + o) = vv;
-      *reinterpret_cast<float4*>(lnu + o) = lv;
+      N::put(nu + o, i0, g.nx, vv);
+      N::put(lnu + o, i0, g.nx, lv);
     }
   }
   if constexpr (CW) block_max_to<32 * NUZ_TY>(mb, cnu);
@@ -1436,6 +1511,31 @@ __global__ void k_update8(Upd8 u, const float* bdtp, long long n, int vec) {
   }
 }
 
+
+#ifdef __CUDACC__   // (the host build knows no __grid_constant__)
+// ---------------------------------------------------------- padded rows ----
+// The eight state arrays to and from arrays of padded rows (Nb4P): blockIdx.y
+// the field, a warp a row.
+struct Pad8 {
+  const float* s[8];
+  float* d[8];
+};
+__global__ void k_pad8(const __grid_constant__ Pad8 a, int nx, int pitch, int rows) {
+  const int r = blockIdx.x * blockDim.y + threadIdx.y;
+  if (r >= rows) return;
+  const float* s = a.s[blockIdx.y] + (size_t)r * nx;
+  float* d = a.d[blockIdx.y] + (size_t)r * pitch;
+  const int end = 4 + (nx + 3) / 4 * 4 + 4;
+  for (int x = threadIdx.x + dep_wait(); x < end; x += 32) d[x] = s[wrap(x - 4, nx)];
+}
+__global__ void k_unpad8(const __grid_constant__ Pad8 a, int nx, int pitch, int rows) {
+  const int r = blockIdx.x * blockDim.y + threadIdx.y;
+  if (r >= rows) return;
+  const float* s = a.s[blockIdx.y] + (size_t)r * pitch + 4;
+  float* d = a.d[blockIdx.y] + (size_t)r * nx;
+  for (int x = threadIdx.x + dep_wait(); x < nx; x += 32) d[x] = s[x];
+}
+#endif
 
 // -------------------------------------------------------- plane means -----
 // Mean over each horizontal plane (constant z) of e - e0 = (E' + Ec - e0 r')/r, in
