@@ -789,7 +789,7 @@ static int stage_rhs(stagger_ctx* c, GraphExec<T>* G, T* const f[8], T* out[8], 
 template <>
 int stage_rhs<float>(stagger_ctx* c, GraphExec<float>*, float* const f[8], float* out[8],
                      cudaStream_t s) {
-  return fused_rhs(c->fused, f, out, s);
+  return fused_rhs_plain(c->fused, f, out, s);
 }
 template <>
 int stage_rhs<double>(stagger_ctx* c, GraphExec<double>* G, double* const f[8], double* out[8],

@@ -178,6 +178,7 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
   F.cap = nullptr;
   F.step_launches = 0;
   F.fork = 0;
+  F.plain = 0;
   for (int i = 0; i < 2; ++i) {
     F.br[i] = nullptr;
     F.brev[i] = nullptr;
@@ -534,10 +535,12 @@ void fused_release(Fused& F) {
 
 // Lanes along x of k_flux_e4's blocks (32, 16 or 8, the rest rows), those that
 // cover the plane with the fewest threads; 0 (k_flux_e) where they are a quarter
-// more than the cells need (planes of few rows), and on boxes of less than two
-// blocks an SM (64^3 step 213 us with k_flux_e4, 208 without; 80^3 389, 393).
-static int flux_e4_lanes(const Geo& g) {
-  if (g.n < 2LL * 152 * 4 * BX * BY * BZ) return 0;
+// more than the cells need (planes of few rows), and on boxes below 2^20 cells,
+// where it gains nothing (step, us, with k_flux_e4 / without: 64^3 213 / 208, 80^3
+// 389 / 393, 96^3 555 / 558, 128^3 1166 / 1189).
+static int flux_e4_lanes(const Fused& F) {
+  const Geo& g = F.kgeo;
+  if (F.plain || g.n < (1LL << 20)) return 0;
   const long long l4 = g.nx / 4;
   long long least = 0;
   int best = 0;
@@ -664,7 +667,7 @@ static int pre_div_t(Fused& F, float* const f[8], cudaStream_t s, bool cfl) {
                 d[F_LZ2], d[F_GX], d[F_GY], d[F_GZ], d[F_QT], d[F_EX], d[F_EY], d[F_EZ]};
   const cudaStream_t se = branch(F, 0, s);   // the energy fluxes, beside the others
   TIMED(K_FLUX, launch_dep(k_flux<N>, gz8, bz8, 0, s, fi, fo, k, g));
-  const int lx = std::is_same<N, Nb4>::value && k.visc ? flux_e4_lanes(g) : 0;
+  const int lx = std::is_same<N, Nb4>::value && k.visc ? flux_e4_lanes(F) : 0;
   if (lx) {
     const int ly = BX * BY * BZ / lx;
     const dim3 ge((unsigned)((g.nx / 4 + lx - 1) / lx), (unsigned)((g.ny + ly - 1) / ly),
@@ -969,6 +972,21 @@ static int courant_to_dev(Fused& F, float* const f[8], cudaStream_t s, bool fuse
                         (float)RK_BETA[2], F.cdt, F.cdtr, F.cdtd, F.zs ? 1.0 : F.dlmin, F.dfac,
                         F.zs ? 1 : F.kp.rm));
   return STAGGER_OK;
+}
+
+// The arrays of the padded layout are larger than the caller's: the plain one
+// runs on them too.
+int fused_rhs_plain(Fused& F, float* const f[8], float* out[8], cudaStream_t s) {
+  const int pad = F.pad;
+  const Geo kgeo = F.kgeo;
+  F.pad = 0;
+  F.kgeo = F.geo;
+  F.plain = 1;
+  const int rc = fused_rhs(F, f, out, s);
+  F.pad = pad;
+  F.kgeo = kgeo;
+  F.plain = 0;
+  return rc;
 }
 
 int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s) {

@@ -54,9 +54,9 @@ struct GNode {
   int c = -1, pop = 0;
   // Float copies of the constants, for the FP32 kernels, and whether the
   // epilogue is other than the identity (set when the graph is complete).
-  float f0 = 0, f1 = 0, f2 = 0, fps = 1, fpt = 0;
+  float f0 = 0, f1 = 0, f2 = 0, fh2 = 0, fps = 1, fpt = 0;
   int ep = 0;
-  // Inverse spacings of the stencils (1 / c0, 1 / h2) and their float copies.
+  // Reciprocal spacings of the stencils: 1 / c0, 1 / h2, and 1 / f0, 1 / fh2 in float.
   double ic0 = 1, ih2 = 1;
   float fi0 = 1, fih2 = 1;
 };

@@ -627,10 +627,11 @@ void build_rhs_graph(GraphDef& G, const stagger_grid& gr, const stagger_params& 
     nd.f0 = (float)nd.c0;
     nd.f1 = (float)nd.c1;
     nd.f2 = (float)nd.c2;
+    nd.fh2 = (float)nd.h2;
     nd.ic0 = nd.c0 != 0 ? 1.0 / nd.c0 : 0.0;
     nd.ih2 = nd.h2 != 0 ? 1.0 / nd.h2 : 0.0;
-    nd.fi0 = (float)nd.ic0;
-    nd.fih2 = (float)nd.ih2;
+    nd.fi0 = nd.f0 != 0 ? 1.0f / nd.f0 : 0.0f;
+    nd.fih2 = nd.fh2 != 0 ? 1.0f / nd.fh2 : 0.0f;
     nd.fps = (float)nd.ps;
     nd.fpt = (float)nd.pt;
     nd.ep = nd.ps != 1.0 || nd.pt != 0.0;

@@ -23,6 +23,28 @@ namespace stg {
 #endif
 #define GZU 1   // cells a thread takes along z
 
+// Roundings that do not depend on how the compiler contracts: the product a b
+// rounded, and a b + c rounded once (the host build rounds twice, like the graph of
+// one node per primitive it is compared with).  The reverse takes the branches of
+// max and |.| at these values, so a last bit can route a cell's gradient elsewhere.
+template <typename T>
+__device__ __forceinline__ T mul_rn(T a, T b) {
+#ifdef __CUDA_ARCH__
+  if constexpr (sizeof(T) == sizeof(float)) return __fmul_rn(a, b);
+  else return __dmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+template <typename T>
+__device__ __forceinline__ T mad(T a, T b, T c) {
+#ifdef __CUDA_ARCH__
+  return fma(a, b, c);
+#else
+  return a * b + c;
+#endif
+}
+
 // The cells of a thread: W consecutive x-cells i .. i + W - 1 of row (j, k), W 1
 // or 4 (4 needs nx a multiple of 4 and 16-byte aligned arrays: each tap is then
 // one 16-byte load and the index work is shared by four cells).  Every lane
@@ -168,40 +190,58 @@ __device__ __forceinline__ void taps6(const T* f, const GCell& c, int axis, int 
   }
 }
 
-// A stencil (kind, inverse spacing ih) from its six taps: up/dn are eq.
+// A node's first and second stencil's spacing and its reciprocal.
+template <typename T> struct Spc { T h, ih; };
+template <typename T> __device__ __forceinline__ Spc<T> sp1(const GNode& nd) {
+  return {kc<T>(nd.c0, nd.f0), kc<T>(nd.ic0, nd.fi0)};
+}
+template <typename T> __device__ __forceinline__ Spc<T> sp2(const GNode& nd) {
+  return {kc<T>(nd.h2, nd.fh2), kc<T>(nd.ih2, nd.fih2)};
+}
+
+// v / h from the rounded reciprocal ih of h, rounded as a division rounds it: the
+// product and one correction by its exact remainder (Markstein, IBM J. Res. Dev.
+// 34, 1990).  The product itself where it is exact (a zero keeps its sign) or
+// where it or the remainder is not finite.
+template <typename T>
+__device__ __forceinline__ T div_by(T v, T h, T ih) {
+  const T q = v * ih;
+  const T r = fma(-q, h, v);
+  const T most = sizeof(T) == 4 ? (T)3.4028235e38 : (T)1.7976931348623157e308;
+  return r != (T)0 && fabs(r) <= most ? fma(r, ih, q) : q;
+}
+
+// A stencil (kind, spacing h, its reciprocal ih) from its six taps: up/dn are eq.
 // (interp) to i+1/2 and i-1/2, ddup/dddn eq. (deriv) to i+1/2 and i-1/2.  One
 // form for the four kinds, sums for the interpolations and differences for the
 // derivatives by the factor s (the kind is known at run time only, and a
-// switch over four forms was a third of the sweeps' instructions).  Times the
-// inverse spacing: a division per cell was half the work of an FP64
-// derivative on the narrow FP64 pipe.
+// switch over four forms was a third of the sweeps' instructions).  The division
+// by the spacing was half the work of an FP64 derivative on the narrow FP64 pipe.
 template <int W, typename T>
-__device__ __forceinline__ void st_comb(int kind, T ih, const T (&t)[6][W], T (&v)[W]) {
+__device__ __forceinline__ void st_comb(int kind, const Spc<T>& sp, const T (&t)[6][W], T (&v)[W]) {
   const bool d = kind >= ST_DDUP;
   const T s = d ? (T)-1 : (T)1;
   const T a = d ? (T)STG_DA : (T)STG_IA, b = d ? (T)STG_DB : (T)STG_IB, e = d ? (T)STG_DC : (T)STG_IC;
 #pragma unroll
-  for (int l = 0; l < W; ++l)
-    v[l] = (a * (t[3][l] + s * t[2][l]) + b * (t[4][l] + s * t[1][l]) + e * (t[5][l] + s * t[0][l])) * ih;
+  for (int l = 0; l < W; ++l) {
+    const T x = a * (t[3][l] + s * t[2][l]) + b * (t[4][l] + s * t[1][l]) + e * (t[5][l] + s * t[0][l]);
+    v[l] = d ? div_by(x, sp.h, sp.ih) : x;
+  }
 }
 __device__ __forceinline__ int st_down(int kind) { return kind & 1; }   // ST_DN, ST_DDDN
-// A node's first and second stencil's inverse spacing.
-template <typename T> __device__ __forceinline__ T ih1(const GNode& nd) { return kc<T>(nd.ic0, nd.fi0); }
-template <typename T> __device__ __forceinline__ T ih2(const GNode& nd) { return kc<T>(nd.ih2, nd.fih2); }
-
-// The stencil (kind, axis, inverse spacing) of f at the thread's cells.
+// The stencil (kind, axis, spacing) of f at the thread's cells.
 template <int W, typename T>
-__device__ __forceinline__ void stencil(const T* f, const GCell& c, int axis, int kind, T ih,
-                                        const Geo& g, T (&v)[W]) {
+__device__ __forceinline__ void stencil(const T* f, const GCell& c, int axis, int kind,
+                                        const Spc<T>& sp, const Geo& g, T (&v)[W]) {
   T t[6][W];
   taps6<W>(f, c, axis, st_down(kind), g, t);
-  st_comb<W>(kind, ih, t, v);
+  st_comb<W>(kind, sp, t, v);
 }
 // The stencil of the product f (h - s): one tap array live, the product
 // formed as its second factor arrives.
 template <int W, typename T>
 __device__ __forceinline__ void stencil_mul(const T* f, const T* h, T s, const GCell& c, int axis,
-                                            int kind, T ih, const Geo& g, T (&v)[W]) {
+                                            int kind, const Spc<T>& sp, const Geo& g, T (&v)[W]) {
   T t[6][W];
   taps6<W>(f, c, axis, st_down(kind), g, t);
   {
@@ -210,9 +250,9 @@ __device__ __forceinline__ void stencil_mul(const T* f, const T* h, T s, const G
 #pragma unroll
     for (int q = 0; q < 6; ++q)
 #pragma unroll
-      for (int l = 0; l < W; ++l) t[q][l] = t[q][l] * (u[q][l] - s);
+      for (int l = 0; l < W; ++l) t[q][l] = mul_rn(t[q][l], u[q][l] - s);
   }
-  st_comb<W>(kind, ih, t, v);
+  st_comb<W>(kind, sp, t, v);
 }
 
 // Transposed kind and sign of a stencil: up^T = dn, dn^T = up, ddup^T =
@@ -460,25 +500,25 @@ __device__ __forceinline__ void node_value(int op, const GNode& nd, const T* A, 
     return;
   }
   switch (op) {
-    case G_STENCIL: stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, r); break;
+    case G_STENCIL: stencil<W>(A, c, nd.axis, nd.sk, sp1<T>(nd), g, r); break;
     case G_STEXP:
-      stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, r);
+      stencil<W>(A, c, nd.axis, nd.sk, sp1<T>(nd), g, r);
 #pragma unroll
       for (int l = 0; l < W; ++l) r[l] = exp(r[l]);
       break;
     case G_STBIN: {
       T b[W];
-      stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, r);
+      stencil<W>(A, c, nd.axis, nd.sk, sp1<T>(nd), g, r);
       ldw<T, W>(B, c.idx, b);
 #pragma unroll
       for (int l = 0; l < W; ++l) r[l] = stbin_val(nd, r[l], b[l]);
       break;
     }
-    case G_STMUL: stencil_mul<W>(A, B, (T)0, c, nd.axis, nd.sk, ih1<T>(nd), g, r); break;
+    case G_STMUL: stencil_mul<W>(A, B, (T)0, c, nd.axis, nd.sk, sp1<T>(nd), g, r); break;
     case G_ST2: {   // one after the other: one tap array live
       T s2[W];
-      stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, r);
-      stencil<W>(B, c, nd.axis2, nd.sk2, ih2<T>(nd), g, s2);
+      stencil<W>(A, c, nd.axis, nd.sk, sp1<T>(nd), g, r);
+      stencil<W>(B, c, nd.axis2, nd.sk2, sp2<T>(nd), g, s2);
 #pragma unroll
       for (int l = 0; l < W; ++l) r[l] = nd.iop == G_ADD ? r[l] + s2[l] : r[l] - s2[l];
       break;
@@ -526,10 +566,21 @@ __device__ __forceinline__ void node_forward(int op, const GNode& nd, const T* A
                                              const T* C, T* out, const T* mesh, const GCell& c,
                                              const Geo& g) {
   T r[W], cv[W] = {};
-  node_value<T, W>(op, nd, A, B, mesh, c, g, r);
   if (nd.pop) ldw<T, W>(C, c.idx, cv);
+  if (op == G_MUL && nd.pop) {   // a b and its folded sum, rounded once
+    T a[W], b[W];
+    ldw<T, W>(A, c.idx, a);
+    ldw<T, W>(B, c.idx, b);
 #pragma unroll
-  for (int l = 0; l < W; ++l) r[l] = finish(nd, r[l], cv[l]);
+    for (int l = 0; l < W; ++l) {
+      const T v = mad(nd.pop == 3 ? -a[l] : a[l], b[l], nd.pop == 2 ? -cv[l] : cv[l]);
+      r[l] = nd.ep ? kc<T>(nd.ps, nd.fps) * v + kc<T>(nd.pt, nd.fpt) : v;
+    }
+  } else {
+    node_value<T, W>(op, nd, A, B, mesh, c, g, r);
+#pragma unroll
+    for (int l = 0; l < W; ++l) r[l] = finish(nd, r[l], cv[l]);
+  }
   stw<T, W>(out, c.idx, r);
 }
 
@@ -604,10 +655,10 @@ __device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T*
     if (op == G_STBIN && nd.iop == G_MUL) {
       // y = st(a) b
       if (role == R_A) {
-        stencil_mul<W>(G, B, (T)0, c, nd.axis, tk, ih1<T>(nd), g, v);
+        stencil_mul<W>(G, B, (T)0, c, nd.axis, tk, sp1<T>(nd), g, v);
       } else {
         T gg[W];
-        stencil<W>(A, c, nd.axis, nd.sk, ih1<T>(nd), g, v);
+        stencil<W>(A, c, nd.axis, nd.sk, sp1<T>(nd), g, v);
         ldw<T, W>(G, c.idx, gg);
 #pragma unroll
         for (int l = 0; l < W; ++l) v[l] = gg[l] * v[l];
@@ -619,7 +670,7 @@ __device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T*
     } else if (op == G_STEXP) {
       // y = ps exp(st(a)) + pt: the stencil's transpose of g (y - pt), the
       // epilogue's factor included (it is in y).
-      stencil_mul<W>(G, Y, kc<T>(nd.pt, nd.fpt), c, nd.axis, tk, ih1<T>(nd), g, v);
+      stencil_mul<W>(G, Y, kc<T>(nd.pt, nd.fpt), c, nd.axis, tk, sp1<T>(nd), g, v);
     } else if (op == G_NB3) {
       // Gather over the three outputs y = x - o, x, x + o (o = sk) that read x
       // as their a(y + o), a(y), a(y - o); a max passes g by the primitive
@@ -659,12 +710,12 @@ __device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T*
       ng = false;
     } else if (op == G_ST2 && role == R_B) {
       // y = st1(a) +- st2(b)
-      stencil<W>(G, c, nd.axis2, st_transpose(nd.sk2), ih2<T>(nd), g, v);
+      stencil<W>(G, c, nd.axis2, st_transpose(nd.sk2), sp2<T>(nd), g, v);
       ng = st_negates(nd.sk2) != (nd.iop == G_SUB);
     } else {
       // The transposed stencil of G: STENCIL, ST2 and STBIN (a sum) to a; STMUL,
       // y = st(a b), times the other factor.
-      stencil<W>(G, c, nd.axis, tk, ih1<T>(nd), g, v);
+      stencil<W>(G, c, nd.axis, tk, sp1<T>(nd), g, v);
       if (op == G_STBIN && nd.iop == G_SUB && nd.side) ng = !ng;   // b - st
       if (op == G_STMUL) {
         T f[W];
@@ -692,8 +743,8 @@ __device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T*
 // one batch share operands); block-uniform switches pick the op.  A node alone
 // is a few microseconds of work (8 MB at 128^3), much of it the launch, its ramp
 // and its tail: one launch a node took 9.5 ms for an adjoint step at 128^3 and
-// 3.4 ms at 64^3 (on four streams), batches of 24 take 7.3 and 1.45 ms, batches
-// of 6 7.5 and 1.5.  The reverse gathers: the thread sums what every consumer
+// 3.4 ms at 64^3 (on four streams), batches of 24 take 7.4 and 1.5 ms, batches
+// of 6 7.6 and 1.6.  The reverse gathers: the thread sums what every consumer
 // passes to the node's cells and stores once, where a sweep by consumer reads
 // and rewrites the gradient for each of them.
 // ---------------------------------------------------------------------------

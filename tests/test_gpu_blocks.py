@@ -22,8 +22,8 @@ OPTS = dict(RM, csmag=0.1, c1=-0.3, do_2nddiv=1, d2lnr_lim=-1.0, g=(0.1, 0.0, -0
 
 
 @pytest.mark.parametrize("shape,kw", [
-    ((128, 53, 48), RM), ((64, 75, 66), RM), ((160, 60, 40), RM), ((1024, 308, 1), RM),
-    ((132, 51, 50), RM), ((128, 3, 850), RM),
+    ((128, 53, 156), RM), ((64, 75, 220), RM), ((160, 60, 110), RM), ((1024, 1028, 1), RM),
+    ((132, 51, 160), RM), ((128, 3, 2800), RM),
     ((131, 97, 75), RM), ((61, 60, 61), RM), ((62, 61, 59), {}), ((63, 1, 3300), OPTS),
     ((9, 150, 150), OPTS), ((1021, 200, 1), RM), ((127, 65, 29), dict(nu_const=1e-3)), ((66, 57, 60), OPTS)])
 def test_four_cell_blocks_match_one_cell(shape, kw):
