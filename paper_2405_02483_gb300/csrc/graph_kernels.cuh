@@ -798,10 +798,11 @@ struct QuenchBatch {
 
 // Both sweeps wait on their loads and on instruction issue (a stencil of four
 // cells is 6 loads, 28 operations and about as many for its indices), so warps
-// count: at 128^3 the FP32 adjoint takes 8.27 ms at 4 blocks an SM (64
-// registers), 7.57 at 5 and 7.34 at 6 (40); two planes a thread 7.54.  FP64 is
-// bound by its own pipe.
-#define STG_GRAPH_LB(T) __launch_bounds__(256, sizeof(T) == 4 ? 6 : 2)
+// count until the values no longer fit the registers.  FP32 adjoint step at
+// 128^3, blocks an SM for (forward, reverse): (4, 4) 8.27 ms, (5, 5) 7.52,
+// (6, 6) 7.60, (6, 5) 7.46-7.53, (6, 4) 7.62, (7, 6) 7.88, (6, 7) 8.03; two planes
+// a thread slower.  FP64 is bound by its own pipe.
+#define STG_GRAPH_LB(T, b32) __launch_bounds__(256, sizeof(T) == 4 ? b32 : 2)
 
 #ifdef __CUDACC__
 // f(integral constant) for the op of a task or term (uniform over the block).
@@ -820,7 +821,7 @@ __device__ __forceinline__ void for_op(int op, F f) {
 }
 
 template <typename T, int W>
-__global__ void STG_GRAPH_LB(T) g_level_fwd(const __grid_constant__ FwdBatch<T> b, const T* mesh,
+__global__ void STG_GRAPH_LB(T, 6) g_level_fwd(const __grid_constant__ FwdBatch<T> b, const T* mesh,
                                             Geo g) {
   const int kb = b.n == 1 ? (int)blockIdx.z : (int)__umulhi(blockIdx.z, b.rn);
   GCell c;
@@ -832,7 +833,7 @@ __global__ void STG_GRAPH_LB(T) g_level_fwd(const __grid_constant__ FwdBatch<T> 
 }
 
 template <typename T, int W>
-__global__ void STG_GRAPH_LB(T) g_level_rev(const __grid_constant__ RevBatch<T> b, Geo g) {
+__global__ void STG_GRAPH_LB(T, 5) g_level_rev(const __grid_constant__ RevBatch<T> b, Geo g) {
   const int kb = b.n == 1 ? (int)blockIdx.z : (int)__umulhi(blockIdx.z, b.rn);
   GCell c;
   if (!gcell_at<W>(c, kb, g)) return;
