@@ -24,6 +24,7 @@ struct stagger_ctx {
   double* w64 = nullptr;
   float* host_state = nullptr;  // device copy for stagger_step_host
   long long extra_launches = 0;
+  int work_arrays[2] = {0, 0};   // arrays of w32, w64
   // The adjoint step as a captured CUDA graph per precision (0 FP32, 1 FP64):
   // state 0 not tried, 1 captured, -1 capture unavailable (direct launches).
   int adj_state[2] = {0, 0};
@@ -685,13 +686,16 @@ template <typename T>
 static int ensure_work(stagger_ctx* c) {
   T*& w = work_of<T>(c);
   if (w) return STAGGER_OK;
-  // f1, f2, q, qbar, and the fixed state and cotangent buffers of the captured
-  // adjoint (8 arrays each).
-  if (cudaMalloc(&w, sizeof(T) * 48 * (size_t)c->geo.n) != cudaSuccess) {
-    w = nullptr;
-    return STAGGER_EOOM;
+  // f1, f2, q, qbar, the cotangent, and the fixed state buffers of the captured
+  // adjoint (8 arrays each); without room for the last the adjoint is launched
+  // directly.
+  int& na = c->work_arrays[sizeof(T) == sizeof(float) ? 0 : 1];
+  for (na = 48; na >= 40; na -= 8) {
+    if (cudaMalloc(&w, sizeof(T) * na * (size_t)c->geo.n) == cudaSuccess) return STAGGER_OK;
+    cudaGetLastError();
   }
-  return STAGGER_OK;
+  w = nullptr;
+  return STAGGER_EOOM;
 }
 
 template <typename T>
@@ -865,6 +869,10 @@ static int graph_step_adjoint(stagger_ctx* c, T* const f0[8], double dt, T* cons
   int rc = ensure_graph<T>(c, true);
   if (rc) return rc;
   rc = ensure_work<T>(c);
+  if (rc == STAGGER_EOOM && !graph_of<T>(c)->lean) {   // the graph gives up its spare sets
+    rc = graph_of<T>(c)->init(c->gdef, c->geo, true, true);
+    if (!rc) rc = ensure_work<T>(c);
+  }
   if (rc) return rc;
   if (!c->dtp && cudaMalloc(&c->dtp, sizeof(double) * 4) != cudaSuccess) {
     c->dtp = nullptr;
@@ -881,12 +889,14 @@ static int graph_step_adjoint(stagger_ctx* c, T* const f0[8], double dt, T* cons
   T* w = work_of<T>(c);
   T *f0c[8], *fb[8];
   for (int k = 0; k < 8; ++k) {
-    f0c[k] = w + (size_t)(32 + k) * n;
-    fb[k] = w + (size_t)(40 + k) * n;
+    fb[k] = w + (size_t)(32 + k) * n;
+    f0c[k] = w + (size_t)(40 + k) * n;
   }
   if (c->adj_state[pi] == 0) {
     c->adj_state[pi] = -1;
-    if (c->cap || cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) == cudaSuccess) {
+    if (c->work_arrays[pi] < 48) {
+      // (f0c is not there: launched directly, on the caller's state)
+    } else if (c->cap || cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) == cudaSuccess) {
       const int timing = c->fused.timing;
       c->fused.timing = 0;   // no event records inside the graph
       const long long before = stagger_launch_count(c);

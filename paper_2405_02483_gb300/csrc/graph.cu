@@ -148,8 +148,15 @@ static void plan_sweeps(const GraphDef& G, int cap, LevelPlan& P) {
 // Executor
 // ---------------------------------------------------------------------------
 template <typename T>
-int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads) {
+int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads, bool lean_only) {
   release();
+  lean = lean_only;
+  // Out of memory: what is held goes, and the lean layout is tried.
+  auto no_room = [&] {
+    cudaGetLastError();
+    release();
+    return lean || !with_grads ? (int)STAGGER_EOOM : init(d, g, with_grads, true);
+  };
   def = d;
   geo = g;
   size_t nn = def.nodes.size();
@@ -160,15 +167,11 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads) {
   // quenched physics to 128^3), so that the adjoint evaluates each stage once.
   // FP32 takes its stage states from the fused kernels, whose results differ from
   // the graph's by rounding, and keeps one set.
-  nsets = sizeof(T) == sizeof(double) && with_grads &&
+  nsets = sizeof(T) == sizeof(double) && with_grads && !lean &&
                   3.0 * sizeof(T) * nval * g.n <= 8.0 * (1ull << 30) ? 3 : 1;
   if (cudaMalloc(&vals, sizeof(T) * nsets * nval * g.n) != cudaSuccess) {
-    cudaGetLastError();
-    nsets = 1;
-    if (cudaMalloc(&vals, sizeof(T) * nval * g.n) != cudaSuccess) {
-      vals = nullptr;
-      return STAGGER_EOOM;
-    }
+    vals = nullptr;
+    return no_room();
   }
   bool has_pmean = false;
   int nquench = 0;
@@ -179,11 +182,14 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads) {
     if ((nd.op == G_SHIFT || nd.op == G_NB3) && nd.sk != 1 && nd.sk != -1) near = false;
   }
   if (nquench && with_grads) {
-    nscr = std::min(nquench, (int)QuenchBatch<T>::MAX);
-    if (cudaMalloc(&qscr, sizeof(T) * 15 * nscr * (size_t)g.n) != cudaSuccess) {
+    // Scratch for several quench nodes at a time, within 8 GiB (at 512^3 one
+    // node's launches fill the GPU by themselves).
+    const size_t one = sizeof(T) * 15 * (size_t)g.n;
+    const size_t fit = std::max<size_t>(1, ((size_t)8 << 30) / one);
+    nscr = lean ? 1 : (int)std::min({(size_t)nquench, (size_t)QuenchBatch<T>::MAX, fit});
+    if (cudaMalloc(&qscr, one * nscr) != cudaSuccess) {
       qscr = nullptr;
-      release();
-      return STAGGER_EOOM;
+      return no_room();
     }
   }
   if (has_pmean && cudaMalloc(&psum, sizeof(T) * g.nz) != cudaSuccess) {
@@ -207,8 +213,7 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads) {
   if (with_grads) {
     if (cudaMalloc(&grads, sizeof(T) * (size_t)std::max(1, lp.nslots) * g.n) != cudaSuccess) {
       grads = nullptr;
-      release();
-      return STAGGER_EOOM;
+      return no_room();
     }
   }
   nvals = nval;
@@ -332,7 +337,7 @@ static void quench_rev(GraphExec<T>& G, const std::vector<int>& q, const LevelGr
   const int most = lg.most(G.nscr);
   for (size_t q0 = 0; q0 < q.size(); q0 += most) {
     QuenchBatch<T> b;
-      b.n = (int)std::min<size_t>(most, q.size() - q0);
+    b.n = (int)std::min<size_t>(most, q.size() - q0);
     b.rn = recip32(b.n);
     for (int j = 0; j < b.n; ++j) {
       const int i = q[q0 + j];

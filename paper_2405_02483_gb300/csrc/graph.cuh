@@ -121,14 +121,15 @@ struct GraphDef {
 void build_rhs_graph(GraphDef& G, const stagger_grid& grid, const stagger_params& p,
                      bool fuse = true);
 
-// The reverse sweep's plan, from the graph alone: which nodes receive a
+// A serial reverse sweep's plan, one transpose at a time in node order, from the
+// graph alone (the sweeps on the GPU run by LevelPlan below): which nodes receive a
 // gradient (hasg), which operand slot of a node gives an input its first
 // contribution and so writes rather than adds (wa, wb, wc), and the gradient
 // array of each node.  A gradient is live from its first contribution (by its
 // highest-numbered consumer) to its own transpose; arrays are reused once the
 // transpose that read them has run: gslot[i] is node i's array (-1: none),
 // gprev[i] the node whose transpose last read that array before (-1: a fresh
-// array), which the first writer must wait for.  Returns the number of arrays.
+// array); nslots the number of arrays.
 struct ReversePlan {
   std::vector<char> hasg, wa, wb, wc;
   std::vector<int> gslot, gprev;
@@ -170,12 +171,15 @@ struct GraphExec {
   T* qscr = nullptr;     // scratch of the G_QUENCH transposes, nscr sets of 15 arrays, or null
   T* grads = nullptr;    // cotangent arrays (lp.nslots)
   int nscr = 0;
+  bool lean = false;     // one set of values and of scratch, where memory is short
   bool near = true;      // every shift is one cell
   std::vector<T*> ptr;   // value pointer per node
   LevelPlan lp;
   long long launches = 0;
 
-  int init(const GraphDef& d, const Geo& g, bool with_grads);
+  // Allocates; where the device has no room for the full layout, or with
+  // lean_only, the lean one.
+  int init(const GraphDef& d, const Geo& g, bool with_grads, bool lean_only = false);
   void release();
   // The values of a set, evaluated on the inputs in.
   void use(int set, T* const in[8]);
