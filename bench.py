@@ -51,25 +51,23 @@ REF_N = 96                      # per-step sample grid of the reference (oracle)
 # Distinct FP32 arrays each kernel reads + writes per launch (every array
 # touched once), for the viscous, quenched workload: the traffic of the
 # arrays the design materialises, not the method's algorithmic minimum.
-# k_div: per stage, over its three launches (momentum; mass and energy;
-# induction; their arrays are disjoint): stage 1 (Courant) reads 25 and
-# writes 8; stages 2 and 3 read 38 (fluxes, state, previous dfdt) and write
-# 16; k_update is the stage-1 update of all 8 fields (f, dfdt in; f out).
+# k_div: per stage, the sum over its three launches (momentum; mass and energy;
+# induction): 15 + 7 + 3 fluxes and sources, then the state read and written and
+# the accumulated dfdt.  Stage 1 (Courant) has no dfdt to read, and its mass and
+# energy wait for dt: 24 + 11 + 12; stage 2: 27 + 15 + 15; stage 3 writes no
+# dfdt: 24 + 13 + 12.  k_update is the stage-1 update of density and energy.
 KERNEL_ARRAYS = {"k_lr_ed": 4, "k_vel": 10, "k_nu_raw": 9, "k_nu_max": 2, "k_nu_smooth": 3,
                  "k_nu_maxsmooth": 3,
-                 "k_nu_faces": 4, "k_tau": 26, "k_edge": 28, "k_flux": 40, "k_flux_e": 17,
-                 "k_div": (33 + 54 + 54) / 3.0, "k_update": 24}
-# DRAM bytes (read + write) per cell per launch from one ncu capture of each
-# kernel on the same workload at 192^3 (traffic grows with the cells).  Only
-# kernels unchanged since their capture.
-NCU_TRAFFIC_PER_CELL = {"k_flux": 1112.1e6 / 192 ** 3, "k_flux_e": 500.6e6 / 192 ** 3,
-                        "k_edge": 762.6e6 / 192 ** 3, "k_tau": 710.2e6 / 192 ** 3,
+                 "k_nu_faces": 4, "k_tau": 26, "k_edge": 28, "k_flux": 37, "k_flux_e": 17,
+                 "k_div": (47 + 57 + 49) / 3.0, "k_update": 6}
+# DRAM bytes (read + write) per cell per launch from one ncu launch list of the
+# same workload at 192^3 (traffic grows with the cells).
+NCU_TRAFFIC_PER_CELL = {"k_flux": 1012.3e6 / 192 ** 3, "k_flux_e": 496.3e6 / 192 ** 3,
+                        "k_edge": 758.3e6 / 192 ** 3, "k_tau": 711.6e6 / 192 ** 3,
                         # per unit of three launches, the mean over the three stages
-                        "k_div": (940.6e6 + 2 * 1539.8e6) / 3 / 192 ** 3}
-# DRAM bytes per zone of one whole step (read + write summed over its 38
-# launches), from an ncu launch list with DRAM counters of the same step at
-# 192^3 (traffic grows with the cells): 10.537 GB + 5.189 GB over 192^3 zones.
-STEP_TRAFFIC_PER_ZONE = (10537.0e6 + 5189.3e6) / 192 ** 3
+                        "k_div": (1259.7e6 + 1533.9e6 + 1353.8e6) / 3 / 192 ** 3}
+# DRAM bytes per zone of one whole step: the sum over the 38 launches of that list.
+STEP_TRAFFIC_PER_ZONE = 15136.2e6 / 192 ** 3
 # Launches that together form one unit of KERNEL_ARRAYS.
 LAUNCHES_PER_UNIT = {"k_div": 3}
 FP32_LANES_PER_SM = 128         # FP32 multiply-add lanes per SM (4 partitions x 32)

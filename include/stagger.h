@@ -86,8 +86,11 @@ typedef struct {
   /* Thread mapping of the fused FP32 kernels (no effect on the results beyond
    * rounding order).  0 (default): four consecutive x-cells per thread with
    * 16-byte loads and stores wherever nx % 4 == 0 and every array of the call
-   * is 16-byte aligned, one cell per thread otherwise; 1: one cell per thread
-   * everywhere.  Other values: STAGGER_EINVAL. */
+   * is 16-byte aligned, or, with other nx, on padded copies of the state for
+   * periodic boxes of uniform z from 196608 cells (without plane means and
+   * fuse_flux_div, and where there is room for the copies); one cell per thread
+   * otherwise; 1: one cell per thread everywhere.  Other values:
+   * STAGGER_EINVAL. */
   int scalar_cells;
   /* Second-order switch of the viscous stress (Sect. Equations, do_2nddiv):
    * where |D2_a ln rho| or |D2_a ln e| of a cell exceeds d2lnr_lim (D2_a f =
@@ -249,8 +252,9 @@ typedef struct {
 int stagger_params_default(stagger_params* p);
 
 /* Create a context for one grid and parameter set on the current CUDA device.
- * Allocates all device scratch once (about 30 fields of nx*ny*nz floats for
- * the fused step; more on the first adjoint call).  *out receives the handle.
+ * Allocates all device scratch once (up to 86 fields of nx*ny*nz floats for
+ * the fused step, 8 more where it runs on padded rows; more on the first adjoint
+ * call).  *out receives the handle.
  * Errors: EINVAL (bad grid/params/NULL), EOOM, ECUDA. */
 int stagger_create(const stagger_grid* grid, const stagger_params* params,
                    stagger_ctx** out);
@@ -275,8 +279,8 @@ int stagger_step(stagger_ctx* ctx, float* state[8], double dt, double* dt_used, 
 /* Run nsteps steps as stagger_step does, with dt <= 0 meaning Courant.
  * A Courant-mode step (dt <= 0) with per-kernel timing off is replayed from a
  * CUDA graph of its launches, captured on the first such call for the given
- * state arrays (on a private stream; launched on `stream`) and captured again
- * when the arrays change; stagger_step and stagger_step_host do the same. */
+ * state arrays (on a private stream and two branches of it; launched on
+ * `stream`) and captured again when the arrays change; stagger_step and stagger_step_host do the same. */
 int stagger_run(stagger_ctx* ctx, float* state[8], int nsteps, double dt, void* stream);
 
 /* The Courant step of eq. (courantcond) for this state (FP64 reduction on the
@@ -309,14 +313,16 @@ int stagger_diagnostics(stagger_ctx* ctx, float* const state[8], double out[10],
  * cotangent lam_np1 of the output state, write the cotangent of the input
  * state to lam_n (8 device arrays, may alias lam_np1).  Recomputes the stage
  * states, then reverses the RK3 recurrence and the right-hand side.  The
- * first call allocates the reverse-sweep workspace (about 3 x the number of
- * graph nodes x nx*ny*nz floats).  Async. */
+ * first call allocates the node values, the gradient and quench arrays and the
+ * workspace (for viscous, quenched physics 330 arrays of nx*ny*nz values, 292
+ * where memory is short; in FP64 twice the node values more while three sets of
+ * them take at most 8 GiB).  Async. */
 int stagger_step_adjoint(stagger_ctx* ctx, float* const state_n[8], double dt,
                          float* const lam_np1[8], float* lam_n[8], void* stream);
 
 /* Unfused evaluation of the same right-hand side: the equations as a graph
  * of primitive staggered operations (eqs. (deriv), (interp) and pointwise
- * arithmetic), one launch per operation.  It is the forward of the adjoint's
+ * arithmetic), each launch a batch of operations that are ready.  It is the forward of the adjoint's
  * reverse sweep and a cross-check of the fused path.  The first call
  * allocates one array of nx*ny*nz values per graph node (a few hundred).
  * _f64 variants take FP64 device arrays (deviations, as above) and compute

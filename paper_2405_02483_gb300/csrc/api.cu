@@ -860,7 +860,7 @@ static int adjoint_body(stagger_ctx* c, T* const f0[8], T* fb[8], cudaStream_t s
 
 // Adjoint of one fixed-dt step (see stagger_step_adjoint).  The first call
 // captures adjoint_body on fixed workspace buffers into a CUDA graph (about
-// 220 launches); every call copies the state and cotangent in, replays the
+// 260 launches); every call copies the state and cotangent in, replays the
 // graph on the caller's stream, and copies the result out.  If capture is not
 // available the body is launched directly (the same kernels).
 template <typename T>

@@ -1,13 +1,14 @@
-// Fused FP32 forward path: one RK stage is eight launches, each a star
-// stencil of reach <= 3 cells per axis over one or a few fields, with the
-// intermediate fluxes kept in HBM between launches:
+// Fused FP32 forward path: one RK stage is up to twelve launches (seven without
+// viscosity), each a star stencil of reach <= 3 cells per axis over one or a few
+// fields, with the intermediate fluxes kept in HBM between launches:
 //   lr      ln(rho/r0)                                   (pointwise)
 //   vel     u = p / rho_face                              (Sect. "Centering")
 //   nu_raw  Richtmyer-Morton nu, eq. (RMnu)               (viscous runs)
 //   nu_max  3x3x3 max;  nu_smooth  3x3x3 mean, ln<nu>      (Sect. "Richtmyer & Morton")
-//   tau     stresses eq. (itv), eta J, J                  (edges, centres)
-//   edge    quench eq. (quench), E = -u x B + eta J eq. (ohm), heating densities
-//   flux    momentum, Lorentz and energy fluxes, -P div u + Q
+//   tau     stresses eq. (itv), eta J, J                  (viscous runs)
+//   edge    quench eq. (quench), eta J, heating densities  (viscous runs)
+//   flux    momentum and Lorentz fluxes, E = -u x B + eta J eq. (ohm)
+//   flux_e  energy fluxes, -P div u + Q
 //   div     divergences -> F(f), eqs. (mass) (mom) (ien) (indu), then the
 //           low-storage update eqs. (ddt), (tupdate)
 #include <math.h>
