@@ -801,7 +801,7 @@ struct QuenchBatch {
 // count until the values no longer fit the registers.  FP32 adjoint step at
 // 128^3, blocks an SM for (forward, reverse): (4, 4) 8.27 ms, (5, 5) 7.52,
 // (6, 6) 7.60, (6, 5) 7.46-7.53, (6, 4) 7.62, (7, 6) 7.88, (6, 7) 8.03; two planes
-// a thread slower.  FP64 is bound by its own pipe.
+// a thread slower.  FP64 is bound by its own pipe (1 to 4 blocks: the same).
 #define STG_GRAPH_LB(T, b32) __launch_bounds__(256, sizeof(T) == 4 ? b32 : 2)
 
 #ifdef __CUDACC__
@@ -859,10 +859,12 @@ __global__ void STG_GRAPH_LB(T, 5) g_level_rev(const __grid_constant__ RevBatch<
 }
 
 // The quench's transpose: PASS 0 q and its derivatives, 1 the cotangents the q
-// receive, 2 the operand's contribution over the node's own cotangent.
+// receive, 2 the operand's contribution over the node's own cotangent.  The passes
+// stream 4 to 15 arrays a node and wait on them: blocks an SM for FP32 (quenched
+// adjoint step at 128^3): uncapped 9.99 ms, 3 9.71, 4 9.57, 5 9.46, 6 9.51.
 template <typename T, int W, int PASS>
-__global__ void __launch_bounds__(256) g_level_quench(const __grid_constant__ QuenchBatch<T> b,
-                                                      Geo g) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1)
+    g_level_quench(const __grid_constant__ QuenchBatch<T> b, Geo g) {
   const int kb = b.n == 1 ? (int)blockIdx.z : (int)__umulhi(blockIdx.z, b.rn);
   const int ti = (int)blockIdx.z - kb * b.n;
   GCell c;
