@@ -179,7 +179,6 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
   F.cap = nullptr;
   F.step_launches = 0;
   F.fork = 0;
-  F.plain = 0;
   for (int i = 0; i < 2; ++i) {
     F.br[i] = nullptr;
     F.brev[i] = nullptr;
@@ -535,13 +534,15 @@ void fused_release(Fused& F) {
 }
 
 // Lanes along x of k_flux_e4's blocks (32, 16 or 8, the rest rows), those that
-// cover the plane with the fewest threads; 0 (k_flux_e) where they are a quarter
-// more than the cells need (planes of few rows), and on boxes below 2^20 cells,
-// where it gains nothing (step, us, with k_flux_e4 / without: 64^3 213 / 208, 80^3
-// 389 / 393, 96^3 555 / 558, 128^3 1166 / 1189).
+// cover the plane with the fewest threads; 0 (k_flux_e, the same bits) where they
+// are a quarter more than the cells need (planes of few rows), and on boxes below
+// 2^20 cells: the barrier and the halo cost small boxes 6% and pay from about 10^6
+// cells (quenched step, us, with k_flux_e4 / without: 64^3 224 / 212, 80^3 389 / 388,
+// 96^3 553 / 555, 112^3 921 / 925, 128^3 1170 / 1177, 512^3 69340 / 69990; one plane
+// 512^2 215 / 211, 1024^2 683 / 684).
 static int flux_e4_lanes(const Fused& F) {
   const Geo& g = F.kgeo;
-  if (F.plain || g.n < (1LL << 20)) return 0;
+  if (g.n < (1LL << 20)) return 0;
   const long long l4 = g.nx / 4;
   long long least = 0;
   int best = 0;
@@ -982,11 +983,9 @@ int fused_rhs_plain(Fused& F, float* const f[8], float* out[8], cudaStream_t s) 
   const Geo kgeo = F.kgeo;
   F.pad = 0;
   F.kgeo = F.geo;
-  F.plain = 1;
   const int rc = fused_rhs(F, f, out, s);
   F.pad = pad;
   F.kgeo = kgeo;
-  F.plain = 0;
   return rc;
 }
 

@@ -99,7 +99,6 @@ struct Fused {
   // padded pitch, the stages running on a padded copy of the state (padst).
   Geo kgeo;
   int pad;
-  int plain;            // fused_rhs_plain is running
   float* padst[8];
   KPar kp;
   float* fld[F_COUNT];
@@ -150,10 +149,9 @@ int fused_init(Fused& F, const stagger_grid& g, const stagger_params& p);
 void fused_release(Fused& F);
 // F(f) into out[8] (plain derivatives).
 int fused_rhs(Fused& F, float* const f[8], float* out[8], cudaStream_t s);
-// The same without padded rows and the two-pass centring of the heating, whose
-// rounding differs in the last bits: the adjoint's stage states.  The reverse takes
-// the branches of max and |.| at these states, so a gradient does not depend on
-// which layout the size of the box selects.
+// The same without padded rows, on which the centred heating differs in the last
+// bits: the adjoint's stage states.  The reverse takes the branches of max and |.|
+// at these states, so a gradient does not depend on the layout of the step.
 int fused_rhs_plain(Fused& F, float* const f[8], float* out[8], cudaStream_t s);
 // One RK3 step in place on f.  dt > 0 fixed, else Courant (device-side).
 int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s);

@@ -1208,14 +1208,19 @@ __global__ void STG_LB_HI(N, STG_MINB) k_flux_e(FluxIn in, FluxOut out, KPar k, 
 // k_flux_e for four-cell threads on a uniform mesh, the edge heating densities
 // centred in two passes.  Their 3 x 36 taps a cell are 72 of k_flux_e's 131 loads
 // a thread; here a block of LX x LY threads (one plane) forms the first of the two
-// interpolations once per row and column (up_x w_z and up_z w_x with three rows
-// above and two below, up_z w_y with a chunk of four columns at each side), passes
-// it through shared memory and takes the second from there: 21 loads and 15 shared
-// ones (512^3: 3.27 -> 2.97 ms; 128^3 step 1189 -> 1166 us).
+// interpolations once per row and column (up_y w_z with a chunk of four columns at
+// each side, up_z w_x with three rows above and two below), passes it through
+// shared memory and takes the second from there.  w_y is interpolated along x and
+// then z, out of the block's plane: its 18 loads stay with the thread and run ahead of
+// the barrier (after it: 69.86 ms a 512^3 step against 69.34; neighbour chunks by
+// warp shuffles: 70.5).  30 loads and 9 shared ones for the 72: 3.10 ms at 512^3 where
+// k_flux_e takes 3.31.  The order of the interpolations is that of k_flux_e, and so
+// are the bits: a last bit of the heating, through the quench of small stresses,
+// reaches 1e-4 to 2e-3 of the rms of B in a cell within ten steps of a plane.
 template <int LX>
 __global__ void STG_LB_N(Nb4, 3, 3) k_flux_e4(FluxIn in, FluxOut out, KPar k, Geo g) {
   constexpr int LY = BX * BY * BZ / LX;
-  __shared__ float4 swz[LY + 5][LX], swx[LY + 5][LX], swy[LY][LX + 2];
+  __shared__ float4 swz[LY][LX + 2], swx[LY + 5][LX];
   const int lx = threadIdx.x + dep_wait(), ly = threadIdx.y;
   const int kz = blockIdx.z, i0 = 4 * blockIdx.x * LX, j0 = blockIdx.y * LY;
   // Threads past the box stand for the periodic cells there.
@@ -1232,39 +1237,31 @@ __global__ void STG_LB_N(Nb4, 3, 3) k_flux_e4(FluxIn in, FluxOut out, KPar k, Ge
   }
   n.c = n.z[3] + n.y[3] + n.x0;
   auto put = [](float4& d, const F4& v) { d = make_float4(v.v[0], v.v[1], v.v[2], v.v[3]); };
-  auto up_z = [&](const float* f, int off) {
-    return s_up([&](int o) { return Nb4::row(f, n.z[o + 3] + off); });
-  };
-  auto up_x = [&](const float* f, int row, int xl, int x0, int xr) {
-    const F4 a = Nb4::row(f, row + xl), b = Nb4::row(f, row + x0), c = Nb4::row(f, row + xr);
-    return s_up([&](int o) { return o == 0 ? b : o < 0 ? Nb4::shift(a, b, 4 + o) : Nb4::shift(b, c, o); });
-  };
-  put(swz[ly + 2][lx], up_x(in.wz, n.z[3] + n.y[3], n.xl, n.x0, n.xr));
-  put(swx[ly + 2][lx], up_z(in.wx, n.y[3] + n.x0));
-  put(swy[ly][lx + 1], up_z(in.wy, n.y[3] + n.x0));
-  // Halo: rows -2, -1, LY .. LY + 2 of the two row arrays, then the chunks left and
-  // right of the rows.
-  for (int t = ly * LX + lx; t < 10 * LX + 2 * LY; t += BX * BY * BZ) {
-    if (t < 10 * LX) {
-      const int r = t / LX, c = t - r * LX, h = r % 5, row = h < 2 ? h : LY + h;   // of LY + 5
-      const int y = wrap(j0 + row - 2, g.ny) * (int)g.sy, x = wrap(i0 + 4 * c, g.nx);
-      if (r < 5) put(swz[row][c], up_x(in.wz, n.z[3] + y, wrap(x - 4, g.nx), x, wrap(x + 4, g.nx)));
-      else put(swx[row][c], up_z(in.wx, y + x));
+  put(swz[ly][lx + 1], s_up([&](int o) { return Nb4::row(in.wz, n.z[3] + n.y[o + 3] + n.x0); }));
+  put(swx[ly + 2][lx], s_up([&](int o) { return Nb4::row(in.wx, n.z[o + 3] + n.y[3] + n.x0); }));
+  // Halo: the chunks left and right of the rows of w_z, rows -2, -1, LY .. LY + 2 of w_x.
+  for (int t = ly * LX + lx; t < 5 * LX + 2 * LY; t += BX * BY * BZ) {
+    if (t < 5 * LX) {
+      const int h = t / LX, c = t - h * LX, row = h < 2 ? h : LY + h;   // of LY + 5
+      const int off = wrap(j0 + row - 2, g.ny) * (int)g.sy + wrap(i0 + 4 * c, g.nx);
+      put(swx[row][c], s_up([&](int o) { return Nb4::row(in.wx, n.z[o + 3] + off); }));
     } else {
-      const int r = (t - 10 * LX) / 2, side = (t - 10 * LX) & 1;
-      const int y = wrap(j0 + r, g.ny) * (int)g.sy;
-      put(swy[r][side * (LX + 1)], up_z(in.wy, y + wrap(i0 + (side ? 4 * LX : -4), g.nx)));
+      const int r = (t - 5 * LX) / 2, side = (t - 5 * LX) & 1;
+      const int off = n.z[3] + wrap(i0 + (side ? 4 * LX : -4), g.nx);
+      put(swz[r][side * (LX + 1)], s_up([&](int o) {
+            return Nb4::row(in.wz, wrap(j0 + r + o, g.ny) * (int)g.sy + off);
+          }));
     }
   }
+  const F4 y = up2(in.wy, n, 2, 0);
   __syncthreads();
   if (i0 + 4 * lx >= g.nx || j0 + ly >= g.ny) return;
   flux_energy_cell(n, in, out, k, [&] {
-    const F4 z = s_up([&](int o) { return Nb4::v4(swz[ly + 2 + o][lx]); });
-    const F4 x = s_up([&](int o) { return Nb4::v4(swx[ly + 2 + o][lx]); });
-    const F4 a = Nb4::v4(swy[ly][lx]), b = Nb4::v4(swy[ly][lx + 1]), c = Nb4::v4(swy[ly][lx + 2]);
-    const F4 y = s_up([&](int o) {
+    const F4 a = Nb4::v4(swz[ly][lx]), b = Nb4::v4(swz[ly][lx + 1]), c = Nb4::v4(swz[ly][lx + 2]);
+    const F4 z = s_up([&](int o) {
       return o == 0 ? b : o < 0 ? Nb4::shift(a, b, 4 + o) : Nb4::shift(b, c, o);
     });
+    const F4 x = s_up([&](int o) { return Nb4::v4(swx[ly + 2 + o][lx]); });
     return (z + x) + y;
   });
 }
