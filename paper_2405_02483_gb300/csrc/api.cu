@@ -639,7 +639,7 @@ static int open_fill_g(stagger_ctx* c, T* const f[8], cudaStream_t s) {
   if (!c->omean_g &&
       cudaMalloc(&c->omean_g, sizeof(double) * (size_t)rows * (1 + nb)) != cudaSuccess) {
     c->omean_g = nullptr;
-    return STAGGER_EOOM;
+    return no_memory();
   }
   OpenG<T> a = open_args<T>(c, f);
   const unsigned bx = (unsigned)((g.sz + 255) / 256);
@@ -674,7 +674,7 @@ template <> double*& work_of<double>(stagger_ctx* c) { return c->w64; }
 template <typename T>
 static int ensure_graph(stagger_ctx* c, bool grads) {
   GraphExec<T>*& G = graph_of<T>(c);
-  if (G && (!grads || G->grads)) return STAGGER_OK;
+  if (G && G->ready(grads)) return STAGGER_OK;
   if (!G) {
     G = new (std::nothrow) GraphExec<T>();
     if (!G) return STAGGER_EOOM;
@@ -876,11 +876,11 @@ static int graph_step_adjoint(stagger_ctx* c, T* const f0[8], double dt, T* cons
   if (rc) return rc;
   if (!c->dtp && cudaMalloc(&c->dtp, sizeof(double) * 4) != cudaSuccess) {
     c->dtp = nullptr;
-    return STAGGER_EOOM;
+    return no_memory();
   }
   if (!c->bdtf && cudaMalloc(&c->bdtf, sizeof(float) * 4) != cudaSuccess) {
     c->bdtf = nullptr;
-    return STAGGER_EOOM;
+    return no_memory();
   }
   k_set_dt3<<<1, 1, 0, s>>>(c->dtp, c->bdtf, dt, RK_BETA[0], RK_BETA[1], RK_BETA[2]);
   ++c->extra_launches;
@@ -984,7 +984,7 @@ int stagger_step_host(stagger_ctx* c, float* state_host[8], int nsteps, double d
   if (!c->host_state) {
     if (cudaMalloc(&c->host_state, sizeof(float) * 8 * n) != cudaSuccess) {
       c->host_state = nullptr;
-      return STAGGER_EOOM;
+      return no_memory();
     }
   }
   float* d[8];

@@ -91,6 +91,13 @@ inline void launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, c
 }
 #endif
 
+// The status of a failed device allocation, whose error the next check of the
+// launches must not report.
+inline int no_memory() {
+  cudaGetLastError();
+  return STAGGER_EOOM;
+}
+
 // Grid and parameter checks of stagger_create (STAGGER_OK or STAGGER_EINVAL).
 int validate_inputs(const stagger_grid* g, const stagger_params* p);
 

@@ -169,7 +169,6 @@ int fused_init(Fused& F, const stagger_grid& gr, const stagger_params& p) {
   // Without room for the padded copies the one-cell kernels run on the caller's rows.
   const int rc = fused_init_t(F, gr, p, 1);
   if (rc != STAGGER_EOOM || !F.pad) return rc;
-  cudaGetLastError();
   return fused_init_t(F, gr, p, 0);
 }
 static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& p, int pad) {
@@ -346,7 +345,7 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
         cudaSuccess) {
       F.pplane = nullptr;
       fused_release(F);
-      return STAGGER_EOOM;
+      return no_memory();
     }
     k.Emean = F.pplane;
     k.pa = reinterpret_cast<const float*>(F.pplane + nd);
@@ -361,7 +360,7 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
     if (cudaMalloc(&F.oplane, sizeof(double) * rows * (1 + F.plane_nb)) != cudaSuccess) {
       F.oplane = nullptr;
       fused_release(F);
-      return STAGGER_EOOM;
+      return no_memory();
     }
     k.omean = F.oplane;
   }
@@ -373,7 +372,7 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
     if (cudaMalloc(&F.pot, sizeof(float) * nfl) != cudaSuccess) {
       F.pot = nullptr;
       fused_release(F);
-      return STAGGER_EOOM;
+      return no_memory();
     }
     std::vector<float> w(2 * ((size_t)gr.nx + gr.ny));
     for (int r = 0; r < gr.nx; ++r) {
@@ -409,7 +408,7 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
     if (cudaMalloc(&F.plane, sizeof(double) * (size_t)gr.nz * (1 + F.plane_nb)) != cudaSuccess) {
       F.plane = nullptr;
       fused_release(F);
-      return STAGGER_EOOM;
+      return no_memory();
     }
     k.emean = F.plane;
   }
@@ -425,7 +424,7 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
     if (cudaMalloc(&F.mesh, sizeof(float) * m.size()) != cudaSuccess) {
       F.mesh = nullptr;
       fused_release(F);
-      return STAGGER_EOOM;
+      return no_memory();
     }
     if (cudaMemcpy(F.mesh, m.data(), sizeof(float) * m.size(), cudaMemcpyHostToDevice) !=
         cudaSuccess) {
@@ -460,7 +459,7 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
   if (k.visc && k.do_quench)
     for (int f : {F_QXX, F_QYY, F_QZZ, F_QXY, F_QYZ, F_QZX}) need.push_back(f);
   for (int f : need)
-    if (!(F.fld[f] = new_array(F))) { fused_release(F); return STAGGER_EOOM; }
+    if (!(F.fld[f] = new_array(F))) { fused_release(F); return no_memory(); }
   for (int c = 0; c < 8; ++c) {
     F.q[c] = new_array(F);
     F.ping[c] = new_array(F);
@@ -468,7 +467,7 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
     if (F.pad) F.padst[c] = new_array(F);
     if (!F.q[c] || !F.ping[c] || !F.pong[c] || (F.pad && !F.padst[c])) {
       fused_release(F);
-      return STAGGER_EOOM;
+      return no_memory();
     }
   }
   dim3 gg = grid3(F.geo);
@@ -476,18 +475,18 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
   if (k.d2div && cudaMalloc(&F.d2flag, (size_t)F.kgeo.n) != cudaSuccess) {
     F.d2flag = nullptr;
     fused_release(F);
-    return STAGGER_EOOM;
+    return no_memory();
   }
   if (cudaMalloc(&F.cmax, sizeof(unsigned) * 4) != cudaSuccess ||
       cudaMemset(F.cmax, 0, sizeof(unsigned) * 4) != cudaSuccess) {
     fused_release(F);
-    return STAGGER_EOOM;
+    return no_memory();
   }
   if (cudaMalloc(&F.dt_dev, sizeof(double) * 8) != cudaSuccess ||
       cudaMalloc(&F.bdt_dev, sizeof(float) * 4) != cudaSuccess ||
       cudaMalloc(&F.red, sizeof(double) * 10 * (size_t)F.red_blocks) != cudaSuccess) {
     fused_release(F);
-    return STAGGER_EOOM;
+    return no_memory();
   }
   return STAGGER_OK;
 }

@@ -153,9 +153,9 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads, bool le
   lean = lean_only;
   // Out of memory: what is held goes, and the lean layout is tried.
   auto no_room = [&] {
-    cudaGetLastError();
     release();
-    return lean || !with_grads ? (int)STAGGER_EOOM : init(d, g, with_grads, true);
+    const int rc = no_memory();
+    return lean || !with_grads ? rc : init(d, g, with_grads, true);
   };
   def = d;
   geo = g;
@@ -194,15 +194,13 @@ int GraphExec<T>::init(const GraphDef& d, const Geo& g, bool with_grads, bool le
   }
   if (has_pmean && cudaMalloc(&psum, sizeof(T) * g.nz) != cudaSuccess) {
     psum = nullptr;
-    release();
-    return STAGGER_EOOM;
+    return no_room();
   }
   if (!def.mesh.empty()) {
     std::vector<T> m(def.mesh.begin(), def.mesh.end());
     if (cudaMalloc(&mesh, sizeof(T) * m.size()) != cudaSuccess) {
       mesh = nullptr;
-      release();
-      return STAGGER_EOOM;
+      return no_room();
     }
     if (cudaMemcpy(mesh, m.data(), sizeof(T) * m.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
       release();

@@ -181,6 +181,9 @@ struct GraphExec {
   // lean_only, the lean one.
   int init(const GraphDef& d, const Geo& g, bool with_grads, bool lean_only = false);
   void release();
+  // Whether it holds its arrays (an init without room leaves it released), with
+  // grads those of the reverse sweep too.
+  bool ready(bool with_grads) const { return !ptr.empty() && (!with_grads || grads); }
   // The values of a set, evaluated on the inputs in.
   void use(int set, T* const in[8]);
   // Evaluate every node into a set; inputs are the 8 stored deviation arrays.
