@@ -71,7 +71,11 @@ __device__ __forceinline__ int dep_wait() {
 #endif
   return zero;
 }
-#ifdef __CUDACC__
+#ifdef __CUDACC__   // (a host build brings launch and launch_dep of its own)
+template <class... P, class... A>
+inline void launch(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t s, A&&... args) {
+  kern<<<grid, block, 0, s>>>(static_cast<P>(args)...);
+}
 template <class... P, class... A>
 inline void launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                        A&&... args) {

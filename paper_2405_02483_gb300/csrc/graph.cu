@@ -303,8 +303,8 @@ static int forward_w(GraphExec<T>& G, cudaStream_t s) {
       const T* A = nd.a >= 0 ? G.ptr[nd.a] : nullptr;
       if (nd.op == G_PMEAN) {
         const LevelGrid l1(g, 1);
-        g_plane_sum<T><<<g.nz, 256, 0, s>>>(A, G.psum, g);
-        g_plane_bcast<T><<<l1.grid(1), l1.b, 0, s>>>(G.psum, G.ptr[i], 0, g);
+        launch(g_plane_sum<T>, dim3(g.nz), dim3(256), s, A, G.psum, g);
+        launch(g_plane_bcast<T>, l1.grid(1), l1.b, s, G.psum, G.ptr[i], 0, g);
         G.launches += 2;
         continue;
       }
@@ -415,8 +415,8 @@ static int backward_w(GraphExec<T>& G, T* const seed[8], T* gin[8], cudaStream_t
     quench_rev<T, W>(G, quench, lg, s);
     for (int i : pmean) {
       const LevelGrid l1(g, 1);
-      g_plane_sum<T><<<g.nz, 256, 0, s>>>(garr(i), G.psum, g);
-      g_plane_bcast<T><<<l1.grid(1), l1.b, 0, s>>>(G.psum, garr(i), 0, g);
+      launch(g_plane_sum<T>, dim3(g.nz), dim3(256), s, garr(i), G.psum, g);
+      launch(g_plane_bcast<T>, l1.grid(1), l1.b, s, G.psum, garr(i), 0, g);
       G.launches += 2;
     }
   }

@@ -750,6 +750,20 @@ __device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T*
 // ---------------------------------------------------------------------------
 // x / n as the high word of x times recip32(n), exact for x < 65536, n <= 64.
 inline unsigned recip32(int n) { return n == 1 ? 0u : 0xffffffffu / (unsigned)n + 1u; }
+__device__ __forceinline__ int div_small(unsigned x, int n, unsigned rn) {
+#ifdef __CUDA_ARCH__
+  return n == 1 ? (int)x : (int)__umulhi(x, rn);
+#else
+  return n == 1 ? (int)x : (int)(((unsigned long long)x * rn) >> 32);
+#endif
+}
+// Nodes and terms a batch holds.
+#ifndef STG_FWD_MAX
+#define STG_FWD_MAX 24
+#endif
+#ifndef STG_REV_MAX
+#define STG_REV_MAX 32
+#endif
 template <typename T>
 struct FwdTask {
   GNode nd;
@@ -758,7 +772,7 @@ struct FwdTask {
 };
 template <typename T>
 struct FwdBatch {
-  static constexpr int MAX = 24;
+  static constexpr int MAX = STG_FWD_MAX;
   int n;         // tasks
   unsigned rn;   // recip32(n)
   FwdTask<T> t[MAX];
@@ -779,7 +793,7 @@ struct RevTask {
 };
 template <typename T>
 struct RevBatch {
-  static constexpr int MAX = 32;
+  static constexpr int MAX = STG_REV_MAX;
   int n, nterm;
   unsigned rn;
   RevTask<T> t[MAX];
@@ -804,7 +818,6 @@ struct QuenchBatch {
 // a thread slower.  FP64 is bound by its own pipe (1 to 4 blocks: the same).
 #define STG_GRAPH_LB(T, b32) __launch_bounds__(256, sizeof(T) == 4 ? b32 : 2)
 
-#ifdef __CUDACC__
 // f(integral constant) for the op of a task or term (uniform over the block).
 template <int OP> struct OpC { static constexpr int value = OP; };
 template <class F>
@@ -823,7 +836,7 @@ __device__ __forceinline__ void for_op(int op, F f) {
 template <typename T, int W>
 __global__ void STG_GRAPH_LB(T, 6) g_level_fwd(const __grid_constant__ FwdBatch<T> b, const T* mesh,
                                             Geo g) {
-  const int kb = b.n == 1 ? (int)blockIdx.z : (int)__umulhi(blockIdx.z, b.rn);
+  const int kb = div_small(blockIdx.z, b.n, b.rn);
   GCell c;
   if (!gcell_at<W>(c, kb, g)) return;
   const FwdTask<T>& t = b.t[(int)blockIdx.z - kb * b.n];
@@ -834,7 +847,7 @@ __global__ void STG_GRAPH_LB(T, 6) g_level_fwd(const __grid_constant__ FwdBatch<
 
 template <typename T, int W>
 __global__ void STG_GRAPH_LB(T, 5) g_level_rev(const __grid_constant__ RevBatch<T> b, Geo g) {
-  const int kb = b.n == 1 ? (int)blockIdx.z : (int)__umulhi(blockIdx.z, b.rn);
+  const int kb = div_small(blockIdx.z, b.n, b.rn);
   GCell c;
   if (!gcell_at<W>(c, kb, g)) return;
   const RevTask<T>& t = b.t[(int)blockIdx.z - kb * b.n];
@@ -865,7 +878,7 @@ __global__ void STG_GRAPH_LB(T, 5) g_level_rev(const __grid_constant__ RevBatch<
 template <typename T, int W, int PASS>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1)
     g_level_quench(const __grid_constant__ QuenchBatch<T> b, Geo g) {
-  const int kb = b.n == 1 ? (int)blockIdx.z : (int)__umulhi(blockIdx.z, b.rn);
+  const int kb = div_small(blockIdx.z, b.n, b.rn);
   const int ti = (int)blockIdx.z - kb * b.n;
   GCell c;
   if (!gcell_at<W>(c, kb, g)) return;
@@ -880,7 +893,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1)
     stw<T, W>(b.G[ti], c.idx, acc);
   }
 }
-#endif  // __CUDACC__
 
 // ---------------------------------------------------------------------------
 // One node per launch (op a template constant), the reverse by consumer: the
