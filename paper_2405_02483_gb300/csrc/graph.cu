@@ -241,17 +241,17 @@ void GraphExec<T>::release() {
 
 static inline bool al16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
-// Block shape of a sweep with w cells a thread: the widest along x among those
-// that cover the box with the fewest threads (256 threads; at nx = 64 half the
-// lanes of a 32-lane row of four-cell threads have no cell).
-static dim3 level_block(const Geo& g, int w) {
+// Block shape of a sweep with w cells a thread along x and wz along z: the widest
+// along x among those that cover the box with the fewest threads (256 threads; at nx
+// = 64 half the lanes of a 32-lane row of four-cell threads have no cell).
+static dim3 level_block(const Geo& g, int w, int wz) {
   static const int sh[6][3] = {{32, 2, 4}, {16, 4, 4}, {8, 8, 4}, {32, 8, 1}, {16, 16, 1}, {8, 32, 1}};
   const long long lanes = (g.nx + w - 1) / w;
   const int* best = sh[0];
   long long least = -1;
   for (const auto& s : sh) {
     const long long t = (lanes + s[0] - 1) / s[0] * s[0] * ((g.ny + s[1] - 1) / s[1] * s[1]) *
-                        ((g.nz + s[2] - 1) / s[2] * s[2]);
+                        ((g.nz + wz * s[2] - 1) / (wz * s[2]) * s[2]);
     if (least < 0 || t < least) {
       least = t;
       best = s;
@@ -263,10 +263,12 @@ struct LevelGrid {
   dim3 b;
   unsigned gx, gy;
   int nzb;
-  LevelGrid(const Geo& g, int w) : b(level_block(g, w)) {
+  LevelGrid(const Geo& g, int W) {   // W as in GCell
+    const int w = W == 4 ? 4 : 1, wz = W / w;
+    b = level_block(g, w, wz);
     gx = (unsigned)((g.nx + b.x * w - 1) / (b.x * w));
     gy = (unsigned)((g.ny + b.y - 1) / b.y);
-    nzb = (int)((g.nz + b.z - 1) / b.z);
+    nzb = (int)((g.nz + b.z * wz - 1) / (b.z * wz));
   }
   int most(int cap) const { return std::max(1, std::min(cap, 65535 / nzb)); }   // gridDim.z
   dim3 grid(int n) const { return dim3(gx, gy, (unsigned)(nzb * n)); }
@@ -279,6 +281,14 @@ static bool cells4(const GraphExec<T>& G, T* const* a, int n) {
   bool ok = G.geo.nx % 4 == 0 && G.near;
   for (int i = 0; i < n; ++i) ok = ok && al16(a[i]);
   return ok;
+}
+
+// FP32 rows of other lengths: three planes a thread (GCell), from the size where
+// fewer threads still fill the GPU (viscous adjoint step, us, one plane / three: 30^3
+// 848 / 980, 43^3 1371 / 1449, 53^3 2029 / 1858, 65^3 3612 / 2993).
+template <typename T>
+static bool planes3(const GraphExec<T>& G) {
+  return G.geo.nz >= 3 && G.geo.n >= G.planes3_from;
 }
 
 template <typename T, int W>
@@ -324,7 +334,9 @@ int GraphExec<T>::forward(T* const in[8], cudaStream_t s, int set) {
   // FP64 takes one cell a thread: its pipe, not the loads, is the bound (32^3
   // adjoint step 2.8 ms against 3.8 with four).
   if constexpr (sizeof(T) == sizeof(float))
-    if (cells4(*this, in, 8)) return forward_w<T, 4>(*this, s);
+    return cells4(*this, in, 8) ? forward_w<T, 4>(*this, s)
+           : planes3(*this)      ? forward_w<T, 3>(*this, s)
+                                 : forward_w<T, 1>(*this, s);
   return forward_w<T, 1>(*this, s);
 }
 
@@ -432,8 +444,10 @@ int GraphExec<T>::backward(T* const seed[8], T* gin[8], cudaStream_t s) {
   for (size_t i = 0; i < def.nodes.size() && ni < 8; ++i)
     if (def.nodes[i].op == G_INPUT) in[ni++] = ptr[i];
   if constexpr (sizeof(T) == sizeof(float))
-    if (cells4(*this, seed, 8) && cells4(*this, gin, 8) && cells4(*this, in, ni))
-      return backward_w<T, 4>(*this, seed, gin, s);
+    return cells4(*this, seed, 8) && cells4(*this, gin, 8) && cells4(*this, in, ni)
+               ? backward_w<T, 4>(*this, seed, gin, s)
+           : planes3(*this) ? backward_w<T, 3>(*this, seed, gin, s)
+                            : backward_w<T, 1>(*this, seed, gin, s);
   return backward_w<T, 1>(*this, seed, gin, s);
 }
 

@@ -173,6 +173,7 @@ struct GraphExec {
   int nscr = 0;
   bool lean = false;     // one set of values and of scratch, where memory is short
   bool near = true;      // every shift is one cell
+  long long planes3_from = 1 << 17;   // cells from which FP32 threads may take three planes
   std::vector<T*> ptr;   // value pointer per node
   LevelPlan lp;
   long long launches = 0;

@@ -45,22 +45,40 @@ __device__ __forceinline__ T mad(T a, T b, T c) {
 #endif
 }
 
-// The cells of a thread: W consecutive x-cells i .. i + W - 1 of row (j, k), W 1
-// or 4 (4 needs nx a multiple of 4 and 16-byte aligned arrays: each tap is then
-// one 16-byte load and the index work is shared by four cells).  Every lane
-// takes the one-cell arithmetic, so the values do not depend on W.
+// The cells of a thread.  W 4: the consecutive x-cells i .. i + 3 of row (j, k) (needs
+// nx a multiple of 4 and 16-byte aligned arrays: each tap is then one 16-byte load and
+// the index work is shared by four cells).  W 1: one cell.  W 3, for rows of other
+// lengths: the cells (i, j) of planes k, k + blockDim.z and k + 2 blockDim.z, which share
+// the offsets of the taps along x and y and the reads of the node's constants (indexed
+// reads of the launch's parameters: with one cell a thread the unit that serves them is
+// 69% busy and the rest of the SM waits on it); a cell past the last plane is the
+// first one again.  FP32 adjoint step, viscous, one plane / three: 90^3 7.64 / 5.02
+// ms, 199 x 150 x 150 41.4 / 25.2, 251 x 250 x 250 140 / 75.8 (one launch a node on
+// four streams: 6.0, 27.8 and 87.8; two planes 5.59, 27.2, 89.6).  Every cell takes the
+// same arithmetic, so the values do not depend on W.
 struct GCell {
   int i, j, k;
-  int idx;   // (a box has less than 2^31 cells)
+  int idx;       // (a box has less than 2^31 cells)
+  int dk[4];     // planes from k to each cell (0 for W 4), the most of them,
+  int dmax;
+  int off[4];    // and cells from idx
 };
 
 template <int W>
 __device__ __forceinline__ bool gcell_at(GCell& c, int kb, const Geo& g) {
-  c.i = W * (int)(blockIdx.x * blockDim.x + threadIdx.x + dep_wait());
+  constexpr int WX = W == 4 ? 4 : 1, WZ = W / WX;
+  c.i = WX * (int)(blockIdx.x * blockDim.x + threadIdx.x + dep_wait());
   c.j = blockIdx.y * blockDim.y + threadIdx.y;
-  c.k = kb * (int)blockDim.z + (int)threadIdx.z;
+  c.k = kb * (WZ * (int)blockDim.z) + (int)threadIdx.z;
   if (c.i >= g.nx || c.j >= g.ny || c.k >= g.nz) return false;
   c.idx = c.k * (int)g.sz + c.j * (int)g.sy + c.i;
+  c.dmax = 0;
+#pragma unroll
+  for (int l = 0; l < W; ++l) {
+    c.dk[l] = WZ > 1 && c.k + l * (int)blockDim.z < g.nz ? l * (int)blockDim.z : 0;
+    c.off[l] = c.dk[l] * (int)g.sz;
+    c.dmax = c.dk[l] > c.dmax ? c.dk[l] : c.dmax;
+  }
   return true;
 }
 template <int W>
@@ -98,15 +116,48 @@ __device__ __forceinline__ void st4(T* p, long long i, const T (&v)[4]) {
     *reinterpret_cast<double2*>(p + i + 2) = make_double2(v[2], v[3]);
   }
 }
+// The thread's cells, o elements further on.
 template <typename T, int W>
-__device__ __forceinline__ void ldw(const T* p, int i, T (&v)[W]) {
-  if constexpr (W == 4) ld4(p, i, v);
-  else v[0] = p[i];
+__device__ __forceinline__ void ldw(const T* p, const GCell& c, int o, T (&v)[W]) {
+  if constexpr (W == 4) ld4(p, c.idx + o, v);
+  else
+#pragma unroll
+    for (int l = 0; l < W; ++l) v[l] = p[c.idx + o + c.off[l]];
 }
 template <typename T, int W>
-__device__ __forceinline__ void stw(T* p, int i, const T (&v)[W]) {
-  if constexpr (W == 4) st4(p, i, v);
-  else p[i] = v[0];
+__device__ __forceinline__ void stw(T* p, const GCell& c, const T (&v)[W]) {
+  if constexpr (W == 4) st4(p, c.idx, v);
+  else
+#pragma unroll
+    for (int l = 0; l < W; ++l) p[c.idx + c.off[l]] = v[l];
+}
+
+// Stride, position and length of an axis.
+struct GAxis {
+  int st, pos, n;
+};
+__device__ __forceinline__ GAxis gaxis(const GCell& c, int axis, const Geo& g) {
+  return {axis == 0 ? 1 : axis == 1 ? (int)g.sy : (int)g.sz, axis == 0 ? c.i : axis == 1 ? c.j : c.k,
+          axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz};
+}
+// f at offset o along the axis from each of the thread's cells, with the wrapped index.
+template <int W, typename T>
+__device__ __forceinline__ void tap_wrap(const T* f, const GCell& c, int axis, const GAxis& a, int o,
+                                         T (&v)[W]) {
+  if (W > 1 && W < 4 && axis == 2) {   // the cells wrap on their own
+#pragma unroll
+    for (int l = 0; l < W; ++l) {
+      const int q = a.pos + c.dk[l];
+      v[l] = f[c.idx + c.off[l] + (wrap(q + o, a.n) - q) * a.st];
+    }
+  } else {
+    ldw<T, W>(f, c, (wrap(a.pos + o, a.n) - a.pos) * a.st, v);
+  }
+}
+// Whether the offsets lo .. hi from each of the thread's cells stay in the box.
+template <int W>
+__device__ __forceinline__ bool inner(const GCell& c, int axis, const GAxis& a, int lo, int hi) {
+  return a.pos + lo >= 0 && a.pos + (W > 1 && W < 4 && axis == 2 ? c.dmax : 0) + hi < a.n;
 }
 
 // t[o + K][l]: f at cell (i + l, j, k) + o e_axis, o = -K .. K (K <= 3):
@@ -115,11 +166,10 @@ template <int K, int W, typename T>
 __device__ __forceinline__ void taps(const T* f, const GCell& c, int axis, const Geo& g,
                                      T (&t)[2 * K + 1][W]) {
   if (W == 4 && axis == 0) {
-    const int row = c.idx - c.i;
     T L[W], M[W], R[W];
-    ldw<T, W>(f, row + wrap(c.i - 4, g.nx), L);
-    ldw<T, W>(f, c.idx, M);
-    ldw<T, W>(f, row + wrap(c.i + 4, g.nx), R);
+    ldw<T, W>(f, c, wrap(c.i - 4, g.nx) - c.i, L);
+    ldw<T, W>(f, c, 0, M);
+    ldw<T, W>(f, c, wrap(c.i + 4, g.nx) - c.i, R);
 #pragma unroll
     for (int o = -K; o <= K; ++o)
 #pragma unroll
@@ -128,13 +178,19 @@ __device__ __forceinline__ void taps(const T* f, const GCell& c, int axis, const
         t[o + K][l] = q < 4 ? L[q & (W - 1)] : q < 8 ? M[(q - 4) & (W - 1)] : R[(q - 8) & (W - 1)];
       }
   } else {
-    const int st = axis == 0 ? 1 : axis == 1 ? (int)g.sy : (int)g.sz;
-    const int pos = axis == 0 ? c.i : axis == 1 ? c.j : c.k;
-    const int n = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
-    const bool inner = pos >= K && pos + K < n;
+    const GAxis a = gaxis(c, axis, g);
+    if (W == 1 || W == 4) {
+      const bool in = inner<W>(c, axis, a, -K, K);
 #pragma unroll
-    for (int o = -K; o <= K; ++o)
-      ldw<T, W>(f, c.idx + (inner ? o : wrap(pos + o, n) - pos) * st, t[o + K]);
+      for (int o = -K; o <= K; ++o)
+        ldw<T, W>(f, c, (in ? o : wrap(a.pos + o, a.n) - a.pos) * a.st, t[o + K]);
+    } else if (inner<W>(c, axis, a, -K, K)) {
+#pragma unroll
+      for (int o = -K; o <= K; ++o) ldw<T, W>(f, c, o * a.st, t[o + K]);
+    } else {
+#pragma unroll
+      for (int o = -K; o <= K; ++o) tap_wrap<W>(f, c, axis, a, o, t[o + K]);
+    }
   }
 }
 
@@ -150,10 +206,7 @@ __device__ __forceinline__ void tap(const T* f, const GCell& c, int axis, int o,
       v[l] = o == -1 ? t[2][l] : o == 1 ? t[4][l] : o == 0 ? t[3][l] : o == -2 ? t[1][l]
            : o == 2 ? t[5][l] : o == -3 ? t[0][l] : t[6][l];
   } else {
-    const int st = axis == 0 ? 1 : axis == 1 ? (int)g.sy : (int)g.sz;
-    const int pos = axis == 0 ? c.i : axis == 1 ? c.j : c.k;
-    const int n = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
-    ldw<T, W>(f, c.idx + (wrap(pos + o, n) - pos) * st, v);
+    tap_wrap<W>(f, c, axis, gaxis(c, axis, g), o, v);
   }
 }
 
@@ -163,11 +216,10 @@ template <int W, typename T>
 __device__ __forceinline__ void taps6(const T* f, const GCell& c, int axis, int dn, const Geo& g,
                                       T (&t)[6][W]) {
   if (W == 4 && axis == 0) {
-    const int row = c.idx - c.i;
     T w[3][W];   // the 12-cell window i - 4 .. i + 7
-    ldw<T, W>(f, row + wrap(c.i - 4, g.nx), w[0]);
-    ldw<T, W>(f, c.idx, w[1]);
-    ldw<T, W>(f, row + wrap(c.i + 4, g.nx), w[2]);
+    ldw<T, W>(f, c, wrap(c.i - 4, g.nx) - c.i, w[0]);
+    ldw<T, W>(f, c, 0, w[1]);
+    ldw<T, W>(f, c, wrap(c.i + 4, g.nx) - c.i, w[2]);
 #pragma unroll
     for (int q = 0; q < 6; ++q)
 #pragma unroll
@@ -176,16 +228,14 @@ __device__ __forceinline__ void taps6(const T* f, const GCell& c, int axis, int 
         t[q][l] = dn ? w[d / 4][d & (W - 1)] : w[u / 4][u & (W - 1)];
       }
   } else {
-    const int st = axis == 0 ? 1 : axis == 1 ? (int)g.sy : (int)g.sz;
-    const int pos = (axis == 0 ? c.i : axis == 1 ? c.j : c.k) - 2 - dn;
-    const int n = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
-    const int base = c.idx - (2 + dn) * st;
-    if (pos >= 0 && pos + 5 < n) {
+    const GAxis a = gaxis(c, axis, g);
+    const int lo = -2 - dn;
+    if (inner<W>(c, axis, a, lo, lo + 5)) {
 #pragma unroll
-      for (int q = 0; q < 6; ++q) ldw<T, W>(f, base + q * st, t[q]);
+      for (int q = 0; q < 6; ++q) ldw<T, W>(f, c, (lo + q) * a.st, t[q]);
     } else {
 #pragma unroll
-      for (int q = 0; q < 6; ++q) ldw<T, W>(f, base + (wrap(pos + q, n) - pos) * st, t[q]);
+      for (int q = 0; q < 6; ++q) tap_wrap<W>(f, c, axis, a, lo + q, t[q]);
     }
   }
 }
@@ -372,10 +422,10 @@ __device__ __forceinline__ void quench_q(const GNode& nd, const T* A, T* Q, cons
       d1[l] = dq[1];
       d2[l] = dq[2];
     }
-    stw<T, W>(Q + (long long)(4 * t) * g.n, c.idx, q);
-    stw<T, W>(Q + (long long)(4 * t + 1) * g.n, c.idx, d0);
-    stw<T, W>(Q + (long long)(4 * t + 2) * g.n, c.idx, d1);
-    stw<T, W>(Q + (long long)(4 * t + 3) * g.n, c.idx, d2);
+    stw<T, W>(Q + (long long)(4 * t) * g.n, c, q);
+    stw<T, W>(Q + (long long)(4 * t + 1) * g.n, c, d0);
+    stw<T, W>(Q + (long long)(4 * t + 2) * g.n, c, d1);
+    stw<T, W>(Q + (long long)(4 * t + 3) * g.n, c, d2);
   }
 }
 
@@ -390,8 +440,8 @@ __device__ __forceinline__ void quench_b1(const GNode& nd, const T* A, const T* 
   taps<1, W>(Q, c, nd.axis, g, tq[0]);
   if (nd.sk >= 0) taps<1, W>(Q + 4 * g.n, c, nd.sk, g, tq[1]);
   T a[W], gg[W], s0[W], sw[6][W];
-  ldw<T, W>(A, c.idx, a);
-  ldw<T, W>(gout, c.idx, gg);
+  ldw<T, W>(A, c, 0, a);
+  ldw<T, W>(gout, c, 0, gg);
 #pragma unroll
   for (int l = 0; l < W; ++l) {
     T wq[6];
@@ -404,10 +454,10 @@ __device__ __forceinline__ void quench_b1(const GNode& nd, const T* A, const T* 
 #pragma unroll
     for (int j = 0; j < 6; ++j) sw[j][l] = base * wq[j];
   }
-  stw<T, W>(S, c.idx, s0);
+  stw<T, W>(S, c, s0);
 #pragma unroll
   for (int j = 0; j < 6; ++j)
-    if (j < 3 || nd.sk >= 0) stw<T, W>(S + (long long)(1 + j) * g.n, c.idx, sw[j]);
+    if (j < 3 || nd.sk >= 0) stw<T, W>(S + (long long)(1 + j) * g.n, c, sw[j]);
 }
 
 // Transpose, second pass (per input cell x): Tbar(x) = S0(x) + the sum over
@@ -416,7 +466,7 @@ __device__ __forceinline__ void quench_b1(const GNode& nd, const T* A, const T* 
 template <typename T, int W>
 __device__ __forceinline__ void quench_b3(const GNode& nd, const T* Q, const T* S, const GCell& c,
                                           const Geo& g, T (&acc)[W]) {
-  ldw<T, W>(S, c.idx, acc);
+  ldw<T, W>(S, c, 0, acc);
   for (int t = 0; t < 2; ++t) {
     const int ax = t == 0 ? nd.axis : nd.sk;
     if (ax < 0) continue;
@@ -493,8 +543,8 @@ __device__ __forceinline__ void node_value(int op, const GNode& nd, const T* A, 
                                            T (&r)[W]) {
   if (pointwise_op(op)) {
     T a[W] = {}, b[W] = {};
-    if (A) ldw<T, W>(A, c.idx, a);
-    if (B) ldw<T, W>(B, c.idx, b);
+    if (A) ldw<T, W>(A, c, 0, a);
+    if (B) ldw<T, W>(B, c, 0, b);
 #pragma unroll
     for (int l = 0; l < W; ++l) r[l] = pw_value(op, nd, a[l], b[l]);
     return;
@@ -509,7 +559,7 @@ __device__ __forceinline__ void node_value(int op, const GNode& nd, const T* A, 
     case G_STBIN: {
       T b[W];
       stencil<W>(A, c, nd.axis, nd.sk, sp1<T>(nd), g, r);
-      ldw<T, W>(B, c.idx, b);
+      ldw<T, W>(B, c, 0, b);
 #pragma unroll
       for (int l = 0; l < W; ++l) r[l] = stbin_val(nd, r[l], b[l]);
       break;
@@ -526,7 +576,7 @@ __device__ __forceinline__ void node_value(int op, const GNode& nd, const T* A, 
     case G_NB3: {
       T m[W], z[W], p[W];
       tap<W>(A, c, nd.axis, nd.sk, g, m);
-      ldw<T, W>(A, c.idx, z);
+      ldw<T, W>(A, c, 0, z);
       tap<W>(A, c, nd.axis, -nd.sk, g, p);
 #pragma unroll
       for (int l = 0; l < W; ++l) {
@@ -554,9 +604,8 @@ __device__ __forceinline__ void node_value(int op, const GNode& nd, const T* A, 
       break;
     }
     default: {   // G_ZFIELD
-      const T z = mesh[(long long)nd.sk * g.nz + c.k];
 #pragma unroll
-      for (int l = 0; l < W; ++l) r[l] = z;
+      for (int l = 0; l < W; ++l) r[l] = mesh[(long long)nd.sk * g.nz + c.k + c.dk[l]];
     }
   }
 }
@@ -566,11 +615,11 @@ __device__ __forceinline__ void node_forward(int op, const GNode& nd, const T* A
                                              const T* C, T* out, const T* mesh, const GCell& c,
                                              const Geo& g) {
   T r[W], cv[W] = {};
-  if (nd.pop) ldw<T, W>(C, c.idx, cv);
+  if (nd.pop) ldw<T, W>(C, c, 0, cv);
   if (op == G_MUL && nd.pop) {   // a b and its folded sum, rounded once
     T a[W], b[W];
-    ldw<T, W>(A, c.idx, a);
-    ldw<T, W>(B, c.idx, b);
+    ldw<T, W>(A, c, 0, a);
+    ldw<T, W>(B, c, 0, b);
 #pragma unroll
     for (int l = 0; l < W; ++l) {
       const T v = mad(nd.pop == 3 ? -a[l] : a[l], b[l], nd.pop == 2 ? -cv[l] : cv[l]);
@@ -581,7 +630,7 @@ __device__ __forceinline__ void node_forward(int op, const GNode& nd, const T* A
 #pragma unroll
     for (int l = 0; l < W; ++l) r[l] = finish(nd, r[l], cv[l]);
   }
-  stw<T, W>(out, c.idx, r);
+  stw<T, W>(out, c, r);
 }
 
 // A pointwise op's cotangents of a and b from y = its value and gg = y's
@@ -632,17 +681,17 @@ __device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T*
   const T sv = kc<T>(nd.ps, nd.fps) * (nd.pop == 3 ? (T)-1 : (T)1);
   if (role >= R_C) {
     const T sc = role == R_C ? kc<T>(nd.ps, nd.fps) * (nd.pop == 2 ? (T)-1 : (T)1) : (T)1;
-    ldw<T, W>(G, c.idx, v);
+    ldw<T, W>(G, c, 0, v);
 #pragma unroll
     for (int l = 0; l < W; ++l) v[l] = sc * v[l];
     return;
   }
   if (pointwise_op(op)) {
     T a[W] = {}, b[W] = {}, y[W], gg[W];
-    if (A) ldw<T, W>(A, c.idx, a);
-    if (B) ldw<T, W>(B, c.idx, b);
-    ldw<T, W>(Y, c.idx, y);
-    ldw<T, W>(G, c.idx, gg);
+    if (A) ldw<T, W>(A, c, 0, a);
+    if (B) ldw<T, W>(B, c, 0, b);
+    ldw<T, W>(Y, c, 0, y);
+    ldw<T, W>(G, c, 0, gg);
 #pragma unroll
     for (int l = 0; l < W; ++l) {
       T ca, cb;
@@ -659,13 +708,13 @@ __device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T*
       } else {
         T gg[W];
         stencil<W>(A, c, nd.axis, nd.sk, sp1<T>(nd), g, v);
-        ldw<T, W>(G, c.idx, gg);
+        ldw<T, W>(G, c, 0, gg);
 #pragma unroll
         for (int l = 0; l < W; ++l) v[l] = gg[l] * v[l];
         ng = false;
       }
     } else if (op == G_STBIN && role == R_B) {
-      ldw<T, W>(G, c.idx, v);
+      ldw<T, W>(G, c, 0, v);
       ng = nd.iop == G_SUB && !nd.side;                    // st - b
     } else if (op == G_STEXP) {
       // y = ps exp(st(a)) + pt: the stencil's transpose of g (y - pt), the
@@ -678,14 +727,14 @@ __device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T*
       const int ax = nd.axis, o = nd.sk;
       T gm[W], g0[W], gp[W];
       tap<W>(G, c, ax, -o, g, gm);
-      ldw<T, W>(G, c.idx, g0);
+      ldw<T, W>(G, c, 0, g0);
       tap<W>(G, c, ax, o, g, gp);
       if (nd.iop == G_ADD) {
 #pragma unroll
         for (int l = 0; l < W; ++l) v[l] = (gm[l] + g0[l]) + gp[l];
       } else {
         T a0[W], am[W], am2[W], ap[W], ap2[W];
-        ldw<T, W>(A, c.idx, a0);
+        ldw<T, W>(A, c, 0, a0);
         tap<W>(A, c, ax, -o, g, am);
         tap<W>(A, c, ax, -2 * o, g, am2);
         tap<W>(A, c, ax, o, g, ap);
@@ -719,7 +768,7 @@ __device__ __forceinline__ void pull(int op, int role, const GNode& nd, const T*
       if (op == G_STBIN && nd.iop == G_SUB && nd.side) ng = !ng;   // b - st
       if (op == G_STMUL) {
         T f[W];
-        ldw<T, W>(role == R_A ? B : A, c.idx, f);
+        ldw<T, W>(role == R_A ? B : A, c, 0, f);
 #pragma unroll
         for (int l = 0; l < W; ++l) v[l] = (ng ? -v[l] : v[l]) * f[l];
         ng = false;
@@ -852,7 +901,7 @@ __global__ void STG_GRAPH_LB(T, 5) g_level_rev(const __grid_constant__ RevBatch<
   if (!gcell_at<W>(c, kb, g)) return;
   const RevTask<T>& t = b.t[(int)blockIdx.z - kb * b.n];
   T acc[W];
-  if (t.add == ADD_FIRST) ldw<T, W>((const T*)t.dst, c.idx, acc);
+  if (t.add == ADD_FIRST) ldw<T, W>((const T*)t.dst, c, 0, acc);
   for (int q = 0; q < t.n; ++q) {
     const RevTerm<T>& r = b.c[t.first + q];
     T v[W];
@@ -864,11 +913,11 @@ __global__ void STG_GRAPH_LB(T, 5) g_level_rev(const __grid_constant__ RevBatch<
   }
   if (t.add == ADD_LAST) {
     T o[W];
-    ldw<T, W>((const T*)t.dst, c.idx, o);
+    ldw<T, W>((const T*)t.dst, c, 0, o);
 #pragma unroll
     for (int l = 0; l < W; ++l) acc[l] = o[l] + acc[l];
   }
-  stw<T, W>(t.dst, c.idx, acc);
+  stw<T, W>(t.dst, c, acc);
 }
 
 // The quench's transpose: PASS 0 q and its derivatives, 1 the cotangents the q
@@ -890,7 +939,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1)
   if (PASS == 2) {
     T acc[W];
     quench_b3<T, W>(nd, Q, S, c, g, acc);
-    stw<T, W>(b.G[ti], c.idx, acc);
+    stw<T, W>(b.G[ti], c, acc);
   }
 }
 
@@ -937,10 +986,10 @@ __device__ __forceinline__ void push_cell(int op, const GNode& nd, const T* A, c
     T v[W], o[W];
     pull<T, W>(op, r, nd, A, B, out, gout, c, g, v);
     if (!w[r]) {
-      ldw<T, W>((const T*)dst[r], c.idx, o);
+      ldw<T, W>((const T*)dst[r], c, 0, o);
       for (int l = 0; l < W; ++l) v[l] = o[l] + v[l];
     }
-    stw<T, W>(dst[r], c.idx, v);
+    stw<T, W>(dst[r], c, v);
   }
 }
 template <typename T, int OP>
@@ -1004,10 +1053,10 @@ __device__ __forceinline__ void quench_put(const GNode& nd, const T* Q, const T*
   T acc[W], o[W];
   quench_b3<T, W>(nd, Q, S, c, g, acc);
   if (!wA) {
-    ldw<T, W>((const T*)gA, c.idx, o);
+    ldw<T, W>((const T*)gA, c, 0, o);
     for (int l = 0; l < W; ++l) acc[l] = o[l] + acc[l];
   }
-  stw<T, W>(gA, c.idx, acc);
+  stw<T, W>(gA, c, acc);
 }
 template <typename T>
 __global__ void g_quench_b3(GNode nd, const T* Q, const T* S, T* gA, int wA, Geo g) {

@@ -234,9 +234,11 @@ static int compare(const char* name, const stagger_grid& gg, const stagger_param
   reference(d1, g, in, seed, ro, rg);
   int fails = 0;
   size_t took = 0;
-  for (int set = 0; set < (sizeof(T) == 8 ? 2 : 1); ++set) {
+  // FP64 with a second set of values, FP32 with one and with three planes a thread.
+  for (int set = 0; set < 2; ++set) {
     GraphExec<T> G;
-    fails += sweeps(G, d, g, in, seed, gin0, out, gin, set, shift) != 0;
+    G.planes3_from = set ? 0 : 1LL << 40;
+    fails += sweeps(G, d, g, in, seed, gin0, out, gin, sizeof(T) == 8 ? set : 0, shift) != 0;
     took = g_used;
     int deep = 0;
     for (const auto& t : G.lp.terms) deep = std::max(deep, (int)t.size());
@@ -251,7 +253,7 @@ static int compare(const char* name, const stagger_grid& gg, const stagger_param
       worst = e / std::max(s, 1.0) <= worst ? worst : e / std::max(s, 1.0);
     }
     const bool ok = same(ro, out) && worst <= tol && G.ready(true);
-    printf("%s %s %dx%dx%d set %d: %d levels, longest sum %d of %d a batch, forward %s, reverse max rel err "
+    printf("%s %s %dx%dx%d run %d: %d levels, longest sum %d of %d a batch, forward %s, reverse max rel err "
            "%.2e%s\n", name, sizeof(T) == 8 ? "FP64" : "FP32", g.nx, g.ny, g.nz, set, G.lp.nrlev, deep,
            RevBatch<T>::MAX, same(ro, out) ? "equal" : "DIFFERS", worst, ok ? "" : "  FAIL");
     fails += !ok;
@@ -332,6 +334,7 @@ int main() {
     fails += compare<double>("viscosity+quench", g, visc);
     fails += compare<float>("viscosity+quench", g, visc);
   }
+  for (int nz : {3, 4, 5, 13, 26}) fails += compare<float>("planes", grid(9, 6, nz), visc);
   fails += compare<float>("unaligned caller", grid(16, 6, 5), visc, 1);
   fails += compare<float>("one plane", grid(12, 9, 1), visc);
   fails += compare<double>("cooling", grid(13, 11, 9), cool);
