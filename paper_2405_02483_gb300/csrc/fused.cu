@@ -906,6 +906,21 @@ static int launch_div(Fused& F, float* const f[8], float* q[8], float* o[8], flo
   return STAGGER_OK;
 }
 
+// Launch of the copies: a warp a row, or, where that leaves the GPU without work (few
+// long rows: a shock tube is one), 256 threads on each of several parts of a row
+// (inviscid right-hand side, us, a warp a row / so: 1021 x 14 x 14 68 / 50, 4001 x 8 x 8
+// 139 / 52, 200001 cells 2499 / 49).
+static void pad_launch(int nx, int rows, dim3& gd, dim3& bd) {
+  const int fill = 40000;   // threads a field
+  bd = dim3(32, 8);
+  int parts = 1;
+  if ((long long)rows * 32 < fill && nx > 128) {
+    bd = dim3(256, 1);
+    parts = std::max(1, std::min((nx + 255) / 256, fill / 256 / rows));
+  }
+  gd = dim3((unsigned)((rows + bd.y - 1) / bd.y), 8, (unsigned)parts);
+}
+
 // The caller's state into F.padst, and padded arrays into the caller's.
 static void pad_in(Fused& F, float* const f[8], cudaStream_t s) {
   Pad8 a;
@@ -914,8 +929,9 @@ static void pad_in(Fused& F, float* const f[8], cudaStream_t s) {
     a.d[c] = F.padst[c];
   }
   const int rows = F.geo.ny * F.geo.nz;
-  TIMED(K_MISC, launch_dep(k_pad8, dim3((unsigned)((rows + 7) / 8), 8), dim3(32, 8), 0, s, a,
-                           F.geo.nx, (int)F.kgeo.sy, rows));
+  dim3 gd, bd;
+  pad_launch(F.geo.nx, rows, gd, bd);
+  TIMED(K_MISC, launch_dep(k_pad8, gd, bd, 0, s, a, F.geo.nx, (int)F.kgeo.sy, rows));
 }
 static void pad_out(Fused& F, float* const src[8], float* const dst[8], cudaStream_t s) {
   Pad8 a;
@@ -924,8 +940,9 @@ static void pad_out(Fused& F, float* const src[8], float* const dst[8], cudaStre
     a.d[c] = dst[c];
   }
   const int rows = F.geo.ny * F.geo.nz;
-  TIMED(K_MISC, launch_dep(k_unpad8, dim3((unsigned)((rows + 7) / 8), 8), dim3(32, 8), 0, s, a,
-                           F.geo.nx, (int)F.kgeo.sy, rows));
+  dim3 gd, bd;
+  pad_launch(F.geo.nx, rows, gd, bd);
+  TIMED(K_MISC, launch_dep(k_unpad8, gd, bd, 0, s, a, F.geo.nx, (int)F.kgeo.sy, rows));
 }
 
 int fused_rhs(Fused& F, float* const f[8], float* out[8], cudaStream_t s) {

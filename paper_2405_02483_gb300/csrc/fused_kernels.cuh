@@ -1512,7 +1512,7 @@ __global__ void k_update8(Upd8 u, const float* bdtp, long long n, int vec) {
 #ifdef __CUDACC__   // (the host build knows no __grid_constant__)
 // ---------------------------------------------------------- padded rows ----
 // The eight state arrays to and from arrays of padded rows (Nb4P): blockIdx.y
-// the field, a warp a row.
+// the field, blockIdx.z the part of the row.
 struct Pad8 {
   const float* s[8];
   float* d[8];
@@ -1523,14 +1523,17 @@ __global__ void k_pad8(const __grid_constant__ Pad8 a, int nx, int pitch, int ro
   const float* s = a.s[blockIdx.y] + (size_t)r * nx;
   float* d = a.d[blockIdx.y] + (size_t)r * pitch;
   const int end = 4 + (nx + 3) / 4 * 4 + 4;
-  for (int x = threadIdx.x + dep_wait(); x < end; x += 32) d[x] = s[wrap(x - 4, nx)];
+  const int step = blockDim.x * gridDim.z;
+  for (int x = blockIdx.z * blockDim.x + threadIdx.x + dep_wait(); x < end; x += step)
+    d[x] = s[wrap(x - 4, nx)];
 }
 __global__ void k_unpad8(const __grid_constant__ Pad8 a, int nx, int pitch, int rows) {
   const int r = blockIdx.x * blockDim.y + threadIdx.y;
   if (r >= rows) return;
   const float* s = a.s[blockIdx.y] + (size_t)r * pitch + 4;
   float* d = a.d[blockIdx.y] + (size_t)r * nx;
-  for (int x = threadIdx.x + dep_wait(); x < nx; x += 32) d[x] = s[x];
+  const int step = blockDim.x * gridDim.z;
+  for (int x = blockIdx.z * blockDim.x + threadIdx.x + dep_wait(); x < nx; x += step) d[x] = s[x];
 }
 #endif
 
