@@ -87,10 +87,12 @@ typedef struct {
    * rounding order).  0 (default): four consecutive x-cells per thread with
    * 16-byte loads and stores wherever nx % 4 == 0 and every array of the call
    * is 16-byte aligned, or, with other nx, on padded copies of the state for
-   * periodic boxes of uniform z from 196608 cells (without plane means and
-   * fuse_flux_div, and where there is room for the copies); one cell per thread
-   * otherwise; 1: one cell per thread everywhere.  Other values:
-   * STAGGER_EINVAL. */
+   * periodic boxes of uniform z from 196608 cells, where a row (nx + 8 rounded up
+   * to whole 128-byte lines) is at most 1.5 nx (without plane means and
+   * fuse_flux_div, and where there is room for the copies: a later call of the
+   * context that finds no room takes theirs, unless it has been captured into a
+   * caller's CUDA graph); one cell per thread otherwise; 1: one cell per thread
+   * everywhere.  Other values: STAGGER_EINVAL. */
   int scalar_cells;
   /* Second-order switch of the viscous stress (Sect. Equations, do_2nddiv):
    * where |D2_a ln rho| or |D2_a ln e| of a cell exceeds d2lnr_lim (D2_a f =
@@ -252,9 +254,9 @@ typedef struct {
 int stagger_params_default(stagger_params* p);
 
 /* Create a context for one grid and parameter set on the current CUDA device.
- * Allocates all device scratch once (up to 86 fields of nx*ny*nz floats for
- * the fused step, 8 more where it runs on padded rows; more on the first adjoint
- * call).  *out receives the handle.
+ * Allocates all device scratch once (up to 88 fields of nx*ny*nz floats for
+ * the fused step, on padded rows 8 more and each up to 1.5 times that; more on the
+ * first adjoint call).  *out receives the handle.
  * Errors: EINVAL (bad grid/params/NULL), EOOM, ECUDA. */
 int stagger_create(const stagger_grid* grid, const stagger_params* params,
                    stagger_ctx** out);

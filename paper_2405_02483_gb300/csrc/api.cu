@@ -671,6 +671,18 @@ template <typename T> T*& work_of(stagger_ctx* c);
 template <> float*& work_of<float>(stagger_ctx* c) { return c->w32; }
 template <> double*& work_of<double>(stagger_ctx* c) { return c->w64; }
 
+// Where an allocation finds no room, the padding of the fused path's rows gives up
+// its own (a captured FP32 adjoint, which runs fused stages, is captured again).
+template <class F>
+static int or_unpad(stagger_ctx* c, F alloc) {
+  const int rc = alloc();
+  if (rc != STAGGER_EOOM || !fused_unpad(c->fused)) return rc;
+  if (c->adj_exec[0]) cudaGraphExecDestroy(c->adj_exec[0]);
+  c->adj_exec[0] = nullptr;
+  if (c->adj_state[0] == 1) c->adj_state[0] = 0;
+  return alloc();
+}
+
 template <typename T>
 static int ensure_graph(stagger_ctx* c, bool grads) {
   GraphExec<T>*& G = graph_of<T>(c);
@@ -679,13 +691,12 @@ static int ensure_graph(stagger_ctx* c, bool grads) {
     G = new (std::nothrow) GraphExec<T>();
     if (!G) return STAGGER_EOOM;
   }
-  return G->init(c->gdef, c->geo, grads);
+  return or_unpad(c, [&] { return G->init(c->gdef, c->geo, grads); });
 }
 
 template <typename T>
-static int ensure_work(stagger_ctx* c) {
+static int alloc_work(stagger_ctx* c) {
   T*& w = work_of<T>(c);
-  if (w) return STAGGER_OK;
   // f1, f2, q, qbar, the cotangent, and the fixed state buffers of the captured
   // adjoint (8 arrays each); without room for the last the adjoint is launched
   // directly.
@@ -696,6 +707,11 @@ static int ensure_work(stagger_ctx* c) {
   }
   w = nullptr;
   return STAGGER_EOOM;
+}
+template <typename T>
+static int ensure_work(stagger_ctx* c) {
+  if (work_of<T>(c)) return STAGGER_OK;
+  return or_unpad(c, [&] { return alloc_work<T>(c); });
 }
 
 template <typename T>
@@ -732,6 +748,7 @@ static void lin2x8(stagger_ctx* c, T* const o[8], T* const x[8], double a, T* co
 
 template <typename T>
 static int graph_rhs(stagger_ctx* c, T* const f[8], T* out[8], cudaStream_t s) {
+  fused_note_capture(c->fused, s);
   int rc = ensure_graph<T>(c, false);
   if (rc) return rc;
   GraphExec<T>* G = graph_of<T>(c);
@@ -754,6 +771,7 @@ static int graph_rhs(stagger_ctx* c, T* const f[8], T* out[8], cudaStream_t s) {
 // One fixed-dt RK3 step through the graph, in place on f.
 template <typename T>
 static int graph_step(stagger_ctx* c, T* f[8], double dt, cudaStream_t s) {
+  fused_note_capture(c->fused, s);
   int rc = ensure_graph<T>(c, false);
   if (rc) return rc;
   rc = ensure_work<T>(c);
@@ -866,6 +884,7 @@ static int adjoint_body(stagger_ctx* c, T* const f0[8], T* fb[8], cudaStream_t s
 template <typename T>
 static int graph_step_adjoint(stagger_ctx* c, T* const f0[8], double dt, T* const lam_in[8],
                               T* lam_out[8], cudaStream_t s) {
+  fused_note_capture(c->fused, s);
   int rc = ensure_graph<T>(c, true);
   if (rc) return rc;
   rc = ensure_work<T>(c);
@@ -982,10 +1001,13 @@ int stagger_step_host(stagger_ctx* c, float* state_host[8], int nsteps, double d
   cudaStream_t s = (cudaStream_t)stream;
   const size_t n = (size_t)c->geo.n;
   if (!c->host_state) {
-    if (cudaMalloc(&c->host_state, sizeof(float) * 8 * n) != cudaSuccess) {
+    fused_note_capture(c->fused, s);
+    const int rc = or_unpad(c, [&] {
+      if (cudaMalloc(&c->host_state, sizeof(float) * 8 * n) == cudaSuccess) return (int)STAGGER_OK;
       c->host_state = nullptr;
       return no_memory();
-    }
+    });
+    if (rc) return rc;
   }
   float* d[8];
   for (int k = 0; k < 8; ++k) {

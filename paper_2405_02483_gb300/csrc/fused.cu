@@ -155,13 +155,40 @@ static void pad_geo(Fused& F) {
 static const int PAD_OFF = 28;
 static float* new_array(const Fused& F) {
   float* a = nullptr;
-  const int off = F.pad ? PAD_OFF : 0;
-  if (cudaMalloc(&a, sizeof(float) * ((size_t)F.kgeo.n + off)) != cudaSuccess) return nullptr;
-  return a + off;
+  if (cudaMalloc(&a, sizeof(float) * ((size_t)F.kgeo.n + F.off)) != cudaSuccess) return nullptr;
+  return a + F.off;
 }
 static void free_array(const Fused& F, float*& a) {
-  if (a) cudaFree(a - (F.pad ? PAD_OFF : 0));
+  if (a) cudaFree(a - F.off);
   a = nullptr;
+}
+
+int fused_unpad(Fused& F) {
+  if (!F.pad || F.pinned) return 0;
+  cudaDeviceSynchronize();
+  if (F.step_exec) cudaGraphExecDestroy(F.step_exec);
+  F.step_exec = nullptr;
+  if (F.step_state == 1) F.step_state = 0;
+  for (int c = 0; c < 8; ++c) {
+    F.step_key[c] = nullptr;
+    free_array(F, F.padst[c]);
+  }
+  F.pad = 0;
+  F.kgeo = F.geo;
+  auto shrink = [&](float*& a) {   // (one that finds no room keeps its size)
+    if (!a) return;
+    float* b = new_array(F);
+    if (!b) {
+      no_memory();
+      return;
+    }
+    free_array(F, a);
+    a = b;
+  };
+  for (int i = 0; i < F_COUNT; ++i) shrink(F.fld[i]);
+  for (int c = 0; c < 8; ++c)
+    for (float** a : {&F.q[c], &F.ping[c], &F.pong[c]}) shrink(*a);
+  return 1;
 }
 
 static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& p, int pad);
@@ -187,12 +214,18 @@ static int fused_init_t(Fused& F, const stagger_grid& gr, const stagger_params& 
   // Rows of no multiple of four cells: the stages run on padded copies of the
   // state with four cells a thread (Nb4P), for periodic, uniform boxes of the
   // split layout without plane means, from the size where that is the faster
-  // mapping (quenched step, us, padded against one cell: 49^3 244 / 244, 65^3 412 /
-  // 484, 131^3 2051 / 2871, 301^3 19617 / 29798; the copies are 5% of it).
+  // mapping (quenched step, us, padded against one cell: 49^3 244 / 244, 65^3 406 /
+  // 482, 131^3 2051 / 2871, 301^3 19617 / 29798; the copies are 5% of it), where
+  // the padding is at most half a row: shorter rows take up to 3.6 times the memory
+  // and the copies cost more than is gained (right-hand side, inviscid: 9 x 150 x
+  // 150 149 / 101, 33 x 100 x 100 109 / 92, 57 x 200 x 200 391 / 392; the longest
+  // rows left out gain in steps, 57 x 200 x 200 quenched 2149 / 2697).
   F.pad = (gr.nx % 4) != 0 && gr.nx >= 8 && !p.scalar_cells && !p.zwalls && !p.zc &&
           !p.fuse_flux_div && !(p.t_chromo > 0) && !p.ediffav && !p.lnp_aver &&
-          F.geo.n >= 3 * (1LL << 16) && pad;
+          F.geo.n >= 3 * (1LL << 16) && 2 * Nb4P::pitch(gr.nx) <= 3 * gr.nx && pad;
   pad_geo(F);
+  F.off = F.pad ? PAD_OFF : 0;
+  F.pinned = 0;
   // One z-marching flux-divergence kernel per stage (on request; uniform z only).
   F.fdiv = p.fuse_flux_div && p.zc == nullptr;
   // z walls at the planes zghost and nz - 1 - zghost: 0 periodic, 1 closed
@@ -921,8 +954,16 @@ static void pad_launch(int nx, int rows, dim3& gd, dim3& bd) {
   gd = dim3((unsigned)((rows + bd.y - 1) / bd.y), 8, (unsigned)parts);
 }
 
+void fused_note_capture(Fused& F, cudaStream_t s) {
+  if (!F.pad) return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(s, &cap);
+  if (cap != cudaStreamCaptureStatusNone) F.pinned = 1;
+}
+
 // The caller's state into F.padst, and padded arrays into the caller's.
 static void pad_in(Fused& F, float* const f[8], cudaStream_t s) {
+  if (s != F.cap) fused_note_capture(F, s);
   Pad8 a;
   for (int c = 0; c < 8; ++c) {
     a.s[c] = f[c];

@@ -99,6 +99,8 @@ struct Fused {
   // padded pitch, the stages running on a padded copy of the state (padst).
   Geo kgeo;
   int pad;
+  int off;              // floats before the first cell of each array
+  int pinned;           // a caller's own CUDA graph may hold the arrays' addresses
   float* padst[8];
   KPar kp;
   float* fld[F_COUNT];
@@ -147,6 +149,11 @@ struct Fused {
 
 int fused_init(Fused& F, const stagger_grid& g, const stagger_params& p);
 void fused_release(Fused& F);
+// Back to the caller's rows, the padding's memory freed (the arrays move: not
+// where a caller may have captured them).  Returns whether there was any.
+int fused_unpad(Fused& F);
+// Notes that a call is being captured on a caller's stream.
+void fused_note_capture(Fused& F, cudaStream_t s);
 // F(f) into out[8] (plain derivatives).
 int fused_rhs(Fused& F, float* const f[8], float* out[8], cudaStream_t s);
 // The same without padded rows, on which the centred heating differs in the last
