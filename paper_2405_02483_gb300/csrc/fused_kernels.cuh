@@ -416,7 +416,10 @@ __device__ __forceinline__ auto s_dn_dd(V v, float ih, decltype(v(0))& d) -> dec
 // Ask for the cell's line of an array the kernel reads later, without a
 // register to receive it: the DRAM read of the first arrays' taps then runs
 // beside those of the later ones (512^3: k_tau 3.71 -> 3.54 ms, the three k_div
-// 5.27 -> 4.82 ms; no gain in k_flux, k_flux_e and k_edge).
+// 5.27 -> 4.82 ms; no gain in k_flux, k_flux_e and k_edge).  The one-cell k_div, which
+// has four times the threads, asks only where it updates the state (Courant step with
+// one cell a thread, ms, always / so / never: 301 x 200 x 150 9.77 / 9.51 / 10.06, 33 x
+// 300 x 300 5.58 / 5.43 / 5.70, 9 x 150 x 150 0.734 / 0.723 / 0.717).
 template <class N> __device__ __forceinline__ void pf(const N& n, const float* p) {
 #ifdef __CUDA_ARCH__
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p + n.c));
@@ -1445,7 +1448,7 @@ __global__ void STG_LB_4(N, STG_MINB) k_div(DivIn in, float* q0, float* q1, floa
   const bool inside = n.init(g, k);
   float* qs[8] = {q0, q1, q2, q3, q4, q5, q6, q7};
   float* os[8] = {o0, o1, o2, o3, o4, o5, o6, o7};
-  if (inside) {
+  if (inside && (N::W == 4 || mode)) {
     if (M & 14)
       for (const float* p : {in.mxx, in.mxy, in.mxz, in.lx1, in.lx2, in.myx, in.myy, in.myz,
                              in.ly1, in.ly2, in.mzx, in.mzy, in.mzz, in.lz1, in.lz2})
