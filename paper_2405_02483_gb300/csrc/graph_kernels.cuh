@@ -357,10 +357,10 @@ __device__ __forceinline__ T q_val(T vm, T v0, T vp, T iq, T eps, T* dq) {
     T wim, wi0, woi, wop;
     max_w(am, a0, wim, wi0);
     max_w(inner, ap, woi, wop);
-    // a2 / den^2 as q times 1 / den: den^2 underflows in FP32 where T and D2 T are
-    // both zero (den = 1e-30), and 0 / 0 would poison the cotangent.
-    const T rd = qdiv((T)1, den), qd = q * rd;
-    const T dq_da2 = rd - iq * qd;
+    // a2 / den^2 as q / den, one rounding: den^2 underflows in FP32 where T and
+    // D2 T are both zero (den = 1e-30), and 0 / 0 would poison the cotangent.
+    const T qd = qdiv(q, den);
+    const T dq_da2 = qdiv((T)1, den) - iq * qd;
     const T dq_dM = -qd;
     const T sd = sgn(d2);
     dq[0] = dq_da2 * sd + dq_dM * (cM * (woi * wim)) * sgn(vm);
