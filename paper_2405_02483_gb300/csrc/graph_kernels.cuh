@@ -249,10 +249,11 @@ template <typename T> __device__ __forceinline__ Spc<T> sp2(const GNode& nd) {
   return {kc<T>(nd.h2, nd.fh2), kc<T>(nd.ih2, nd.fih2)};
 }
 
-// v / h from the rounded reciprocal ih of h, rounded as a division rounds it: the
-// product and one correction by its exact remainder (Markstein, IBM J. Res. Dev.
-// 34, 1990).  The product itself where it is exact (a zero keeps its sign) or
-// where it or the remainder is not finite.
+// v / h from the rounded reciprocal ih of h, rounded as a division rounds it while the
+// remainder of the product can be represented (|v| above 2e-31 in FP32, 2e-291 in FP64;
+// within two units in the last place below): the product and one correction by its
+// exact remainder (Markstein, IBM J. Res. Dev. 34, 1990).  The product itself where
+// it is exact (a zero keeps its sign) or where it or the remainder is not finite.
 template <typename T>
 __device__ __forceinline__ T div_by(T v, T h, T ih) {
   const T q = v * ih;
