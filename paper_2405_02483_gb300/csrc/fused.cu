@@ -1,6 +1,9 @@
-// Fused FP32 forward path: one RK stage is up to twelve launches (seven without
-// viscosity), each a star stencil of reach <= 3 cells per axis over one or a few
-// fields, with the intermediate fluxes kept in HBM between launches:
+// Fused FP32 forward path: one RK stage is twelve launches with Richtmyer-Morton
+// viscosity on four-cell threads (thirteen on one-cell threads, whose max and mean of
+// nu are two), nine with a constant nu, seven without viscosity; the Smagorinsky
+// strain, the second-order switch, chromospheric and coronal cooling, plane means and
+// walls add theirs.  Each is a star stencil of reach <= 3 cells per axis over one or a
+// few fields, with the intermediate fluxes kept in HBM between launches:
 //   lr      ln(rho/r0)                                   (pointwise)
 //   vel     u = p / rho_face                              (Sect. "Centering")
 //   nu_raw  Richtmyer-Morton nu, eq. (RMnu)               (viscous runs)
@@ -1128,8 +1131,8 @@ int fused_dt(Fused& F, float* const fu[8], cudaStream_t s) {
   return STAGGER_OK;
 }
 
-// A Courant-mode step is 38 to 50 launches whose arguments depend only on the
-// state arrays and the context (the step dt lives on the device), so it is
+// A Courant-mode step is 24 launches without viscosity and 38 to 50 with, whose
+// arguments depend only on the state arrays and the context (the step dt lives on the device), so it is
 // captured once, on a private stream, into a CUDA graph and replayed on the
 // caller's stream: on small grids the launches, not the kernels, set the time.
 // The capture is redone when the state arrays change, and not used while

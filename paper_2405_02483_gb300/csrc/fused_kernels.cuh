@@ -1041,7 +1041,7 @@ __global__ void STG_LB(N, STG_MINB_HI) k_edge(
 }
 
 // ---------------------------------------------------------------- flux -----
-struct FluxIn {
+struct FluxIn {   // (Jx, Jy, Jz are k_tau's; the flux kernels form J from the taps of B)
   const float *px, *py, *pz, *rd, *Ed, *bx, *by, *bz, *ls, *ux, *uy, *uz;
   const float *qxx, *qyy, *qzz, *qxy, *qyz, *qzx, *Jx, *Jy, *Jz, *nu, *wc, *wx, *wy, *wz;
   const float* ed;   // e - e0 at centres

@@ -314,7 +314,7 @@ static int forward_w(GraphExec<T>& G, cudaStream_t s) {
       if (nd.op == G_PMEAN) {
         const LevelGrid l1(g, 1);
         launch(g_plane_sum<T>, dim3(g.nz), dim3(256), s, A, G.psum, g);
-        launch(g_plane_bcast<T>, l1.grid(1), l1.b, s, G.psum, G.ptr[i], 0, g);
+        launch(g_plane_bcast<T>, l1.grid(1), l1.b, s, G.psum, G.ptr[i], g);
         G.launches += 2;
         continue;
       }
@@ -428,7 +428,7 @@ static int backward_w(GraphExec<T>& G, T* const seed[8], T* gin[8], cudaStream_t
     for (int i : pmean) {
       const LevelGrid l1(g, 1);
       launch(g_plane_sum<T>, dim3(g.nz), dim3(256), s, garr(i), G.psum, g);
-      launch(g_plane_bcast<T>, l1.grid(1), l1.b, s, G.psum, garr(i), 0, g);
+      launch(g_plane_bcast<T>, l1.grid(1), l1.b, s, G.psum, garr(i), g);
       G.launches += 2;
     }
   }

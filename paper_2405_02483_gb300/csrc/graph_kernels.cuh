@@ -11,7 +11,7 @@
 
 namespace stg {
 
-// The launch shape of the one-cell kernels (threads along x, y, z).
+// The launch shape of the one-node kernels (threads along x, y, z).
 #ifndef GBX
 #define GBX 32
 #endif
@@ -21,7 +21,7 @@ namespace stg {
 #ifndef GBZ
 #define GBZ 4
 #endif
-#define GZU 1   // cells a thread takes along z
+#define GZU 1   // planes a thread of the one-node kernels takes
 
 // Roundings that do not depend on how the compiler contracts: the product a b
 // rounded, and a b + c rounded once (the host build rounds twice, like the graph of
@@ -498,8 +498,7 @@ __device__ __forceinline__ T stbin_val(const GNode& nd, T st, T b) {
   return nd.side ? b - st : st - b;     // G_SUB
 }
 
-// The ops whose value at a cell reads only that cell of their operands: they
-// run as flat kernels over the arrays (g_forward_pw, g_backward_pw).
+// The ops whose value at a cell reads only that cell of their operands.
 __host__ __device__ __forceinline__ bool pointwise_op(int op) {
   constexpr unsigned mask = 1u << G_ADD | 1u << G_SUB | 1u << G_MUL | 1u << G_DIV | 1u << G_MAX |
                             1u << G_EXP | 1u << G_LOG | 1u << G_LOG1P | 1u << G_SQRT |
@@ -865,7 +864,7 @@ struct QuenchBatch {
 // count until the values no longer fit the registers.  FP32 adjoint step at
 // 128^3, blocks an SM for (forward, reverse): (4, 4) 8.27 ms, (5, 5) 7.52,
 // (6, 6) 7.60, (6, 5) 7.46-7.53, (6, 4) 7.62, (7, 6) 7.88, (6, 7) 8.03; two planes
-// a thread slower.  FP64 is bound by its own pipe (1 to 4 blocks: the same).
+// of four cells a thread slower.  FP64 is bound by its own pipe (1 to 4 blocks: the same).
 #define STG_GRAPH_LB(T, b32) __launch_bounds__(256, sizeof(T) == 4 ? b32 : 2)
 
 // f(integral constant) for the op of a task or term (uniform over the block).
@@ -945,8 +944,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1)
 }
 
 // ---------------------------------------------------------------------------
-// One node per launch (op a template constant), the reverse by consumer: the
-// form the host build runs against the graph of one node per primitive.
+// One node per launch (op a template constant), the reverse by consumer: not run by
+// the library, whose host tests sweep the merged graph and the graph of one node per
+// primitive with it.
 // ---------------------------------------------------------------------------
 template <typename T, int OP>
 __global__ void g_forward(GNode nd, const T* A, const T* B, const T* C, T* out, const T* mesh,
@@ -1071,8 +1071,8 @@ __global__ void g_quench_b3_4(GNode nd, const T* Q, const T* S, T* gA, int wA, G
 }
 
 // Horizontal-plane mean (G_PMEAN): one block per z sums its plane in a fixed
-// order; the broadcast writes (or, for the transpose, adds) sum / (nx ny).
-// The mean is linear and symmetric, so its transpose is the same mean.
+// order; the broadcast writes sum / (nx ny).  The mean is linear and symmetric, so
+// its transpose is the same mean, of the node's cotangent in place.
 template <typename T>
 __global__ void g_plane_sum(const T* A, T* psum, Geo g) {
   __shared__ T sm[256];
@@ -1090,11 +1090,10 @@ __global__ void g_plane_sum(const T* A, T* psum, Geo g) {
 }
 
 template <typename T>
-__global__ void g_plane_bcast(const T* psum, T* out, int add, Geo g) {
+__global__ void g_plane_bcast(const T* psum, T* out, Geo g) {
   GCell c;
   if (!gcell<1>(c, g)) return;
-  const T v = psum[c.k] / (T)((double)g.nx * g.ny);
-  out[c.idx] = add ? out[c.idx] + v : v;
+  out[c.idx] = psum[c.k] / (T)((double)g.nx * g.ny);
 }
 
 }  // namespace stg
