@@ -156,9 +156,8 @@ int fused_unpad(Fused& F);
 void fused_note_capture(Fused& F, cudaStream_t s);
 // F(f) into out[8] (plain derivatives).
 int fused_rhs(Fused& F, float* const f[8], float* out[8], cudaStream_t s);
-// The same without padded rows, on which the centred heating differs in the last
-// bits: the adjoint's stage states.  The reverse takes the branches of max and |.|
-// at these states, so a gradient does not depend on the layout of the step.
+// The same on the caller's rows also where the context pads them (the same bits): the
+// stage states of the captured adjoint, which holds no copies.
 int fused_rhs_plain(Fused& F, float* const f[8], float* out[8], cudaStream_t s);
 // One RK3 step in place on f.  dt > 0 fixed, else Courant (device-side).
 int fused_step(Fused& F, float* f[8], double dt, cudaStream_t s);

@@ -121,11 +121,25 @@ __device__ __forceinline__ F4 fdiv(const F4& a, const F4& b) {
             fdiv(a.v[3], b.v[3]));
 }
 
+// a b + c rounded once (the host build, which contracts nothing, rounds twice).
+__device__ __forceinline__ float fma_rn(float a, float b, float c) {
+#ifdef __CUDA_ARCH__
+  return __fmaf_rn(a, b, c);
+#else
+  return a * b + c;
+#endif
+}
+__device__ __forceinline__ F4 fma_rn(const F4& a, const F4& b, const F4& c) {
+  return F4(fma_rn(a.v[0], b.v[0], c.v[0]), fma_rn(a.v[1], b.v[1], c.v[1]),
+            fma_rn(a.v[2], b.v[2], c.v[2]), fma_rn(a.v[3], b.v[3], c.v[3]));
+}
+
 // Periodic neighbour offsets of one cell, offsets -3..3 per axis.
 struct Nb {
   using T = float;
   using Base = Nb;
   static constexpr int W = 1;
+  static constexpr bool PADDED = false;
   int c;
   int kz;       // z index of the cell
   int x[7];
@@ -206,6 +220,7 @@ struct Nb4 {
   using T = F4;
   using Base = Nb4;
   static constexpr int W = 4;
+  static constexpr bool PADDED = false;
   int c;        // offset of cell i0
   int kz;       // z index of the cells
   int x0, xl, xr;   // x of the chunk at, left of and right of i0 (periodic)
@@ -305,6 +320,7 @@ struct Nb4 {
 // nothing uses what they then hold).
 struct Nb4P : Nb4 {
   using Base = Nb4P;
+  static constexpr bool PADDED = true;
   int i0, nx;
   // (whole 128-byte lines: a block of 8 lanes reads one line a row)
   static __host__ __device__ __forceinline__ int pitch(int nx) {
@@ -1036,7 +1052,12 @@ __global__ void STG_LB(N, STG_MINB_HI) k_edge(
   const T sxx = Sd.a, syy = Sd.b, szz = Sd.c, sxy = So.a, syz = So.b, szx = So.c;
   n.st(wc, (txx_ * sxx + tyy_ * syy) + tzz_ * szz);
   n.st(wx, 2.f * (tyz_ * syz) + rx_ * n.ld(Jx));
-  n.st(wy, 2.f * (tzx_ * szx) + ry_ * n.ld(Jy));
+  // Without the second-order switch the compiler fuses this sum's other product on
+  // one-cell threads than on four-cell ones.  Padded rows take over from one-cell
+  // threads and keep their rounding: the results of a box do not depend on whether
+  // its size lets it be padded.
+  if constexpr (N::PADDED && !D2) n.st(wy, fma_rn(ry_, n.ld(Jy), 2.f * (tzx_ * szx)));
+  else n.st(wy, 2.f * (tzx_ * szx) + ry_ * n.ld(Jy));
   n.st(wz, 2.f * (txy_ * sxy) + rz_ * n.ld(Jz));
 }
 

@@ -48,6 +48,17 @@ def test_rhs_of_a_repeated_field(shape, times, kw):
         assert torch.equal(a, e)
 
 
+@pytest.mark.parametrize("kw", [dict(), RM, dict(RM, do_quench=1), dict(RM, do_quench=1, quench_max3=1),
+                                dict(RM, csmag=0.1, c1=-0.3, do_quench=1, do_2nddiv=1, d2lnr_lim=0.05),
+                                dict(nu_const=1e-3), dict(RM, g=(0.1, 0.0, -0.2), t_cool=0.3, e_cool=0.8,
+                                                          cor_L0=0.5, cor_Tunit=8e3)])
+@pytest.mark.parametrize("shape,times", [((65, 40, 36), (1, 2, 2)), ((131, 38, 30), (1, 2, 3)),
+                                         ((43, 52, 36), (3, 2, 2)), ((350, 250, 1), (3, 1, 1))])
+def test_rhs_of_a_repeated_field_on_padded_rows(shape, times, kw):
+    """One-cell threads on the small box's rows, padded rows on the large one's."""
+    test_rhs_of_a_repeated_field(shape, times, kw)
+
+
 def test_steps_of_a_repeated_plane():
     import paper_2405_02483_gb300 as S
     shape, times = (512, 512, 1), (2, 2, 1)
