@@ -62,12 +62,12 @@ KERNEL_ARRAYS = {"k_lr_ed": 4, "k_vel": 10, "k_nu_raw": 9, "k_nu_max": 2, "k_nu_
                  "k_div": (47 + 57 + 49) / 3.0, "k_update": 6}
 # DRAM bytes (read + write) per cell per launch from one ncu launch list of the
 # same workload at 192^3 (traffic grows with the cells).
-NCU_TRAFFIC_PER_CELL = {"k_flux": 1012.3e6 / 192 ** 3, "k_flux_e": 496.3e6 / 192 ** 3,
-                        "k_edge": 758.3e6 / 192 ** 3, "k_tau": 711.6e6 / 192 ** 3,
+NCU_TRAFFIC_PER_CELL = {"k_flux": 1013.2e6 / 192 ** 3, "k_flux_e": 495.8e6 / 192 ** 3,
+                        "k_edge": 757.9e6 / 192 ** 3, "k_tau": 711.2e6 / 192 ** 3,
                         # per unit of three launches, the mean over the three stages
                         "k_div": (1259.7e6 + 1533.9e6 + 1353.8e6) / 3 / 192 ** 3}
 # DRAM bytes per zone of one whole step: the sum over the 38 launches of that list.
-STEP_TRAFFIC_PER_ZONE = 15136.2e6 / 192 ** 3
+STEP_TRAFFIC_PER_ZONE = 15131.6e6 / 192 ** 3
 # Launches that together form one unit of KERNEL_ARRAYS.
 LAUNCHES_PER_UNIT = {"k_div": 3}
 FP32_LANES_PER_SM = 128         # FP32 multiply-add lanes per SM (4 partitions x 32)
