@@ -1138,6 +1138,7 @@ int fused_dt(Fused& F, float* const fu[8], cudaStream_t s) {
 // The capture is redone when the state arrays change, and not used while
 // per-kernel timing is on; a failed capture falls back to direct launches.
 int fused_step_graphed(Fused& F, float* f[8], double dt, cudaStream_t s) {
+  fused_note_capture(F, s);
   if (dt > 0 || F.timing || F.step_state < 0) return fused_step(F, f, dt, s);
   bool same = F.step_state == 1;
   for (int c = 0; c < 8 && same; ++c) same = F.step_key[c] == f[c];
